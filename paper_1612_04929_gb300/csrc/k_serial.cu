@@ -529,7 +529,7 @@ cudaError_t launch_chain(const ChainArgs<R>& a, cudaStream_t st) {
 // backward costate sweep: G_{j-1} = U_j^dag G_j + src_{j-1}, one CTA per (panel, member, segment)
 // ------------------------------------------------------------------------------------------
 // Segment z covers local slices a = z * seg .. b = min(wlen, a + seg) - 1.  With in-carry Y
-// (zero when a.cin is null) the CTA sets G_b = Y + src_b, runs G_{jl-1} = U_jl^dag G_jl + src_{jl-1}
+// (zero when a.cin is null) the CTA sets G_b = Y + src_b (src = 0 when neither source is given), runs G_{jl-1} = U_jl^dag G_jl + src_{jl-1}
 // down to jl = a + 1, and leaves out = U_a^dag G_a, the in-carry of the segment below; `out`
 // goes to a.cout.  A whole wave is one segment (seg = wlen) with the carry as in- and out-carry.
 template <typename R, int RING, typename S, typename Mt, int NCB>
@@ -545,7 +545,8 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 1024) k_costate(Costate
     const int n = b0 - a0 + 1;
     const size_t slice = A.sv.slice(), panel = (size_t)d * cb, poff = (size_t)kb * A.sv.pstride;
     const size_t ub = ring_bytes((size_t)d * d, sizeof(Mt));
-    const size_t pb = (size_t)A.sv.pstride * sizeof(S);
+    const bool has_src = A.src || A.srck;
+    const size_t pb = has_src ? (size_t)A.sv.pstride * sizeof(S) : 0;
     const size_t slot = ub + pb;
     unsigned char* ring = smraw;
     K* xa = reinterpret_cast<K*>(smraw + RING * slot);   // RING 0: no ring
@@ -561,11 +562,12 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 1024) k_costate(Costate
     K* Gk = A.Gk ? A.Gk + e * A.g_es + poff : nullptr;
     {   // G_b = Y + src_b
         const K* ci = A.cin ? A.cin + e * A.cin_es + (size_t)z * slice + poff : nullptr;
-        const S* s_last = Se + (size_t)b0 * slice;
         for (int i = tid; i < (int)panel; i += blockDim.x) {
             K v = ci ? ci[i] : kzero<K>();
-            kadd(v, kfrom(s_last[i]));
-            knorm(v);
+            if (has_src) {
+                kadd(v, kfrom(Se[(size_t)b0 * slice + i]));
+                knorm(v);
+            }
             xa[i] = v;
             if constexpr (sizeof(R) == 4) atomicMax(&smax[0], pair_maxbits(v));
             if (Ge) Ge[(size_t)b0 * slice + i] = kround(v);
@@ -605,7 +607,8 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 1024) k_costate(Costate
         for (int t = 0; t < n; ++t) {
             const int jl = b0 - t;
             __syncthreads();
-            step(UHe + (size_t)jl * A.ustride, (jl > a0) ? Se + (size_t)(jl - 1) * slice : nullptr, t, emit_for(jl));
+            step(UHe + (size_t)jl * A.ustride, (has_src && jl > a0) ? Se + (size_t)(jl - 1) * slice : nullptr, t,
+                 emit_for(jl));
         }
     } else if constexpr (RING == 1) {
 #pragma unroll 1
@@ -613,11 +616,11 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 1024) k_costate(Costate
             const int jl = b0 - t;
             __syncthreads();
             ring_issue(ring, UHe + (size_t)jl * A.ustride, ub);
-            if (jl > a0) ring_issue(ring + ub, Se + (size_t)(jl - 1) * slice, pb);
+            if (has_src && jl > a0) ring_issue(ring + ub, Se + (size_t)(jl - 1) * slice, pb);
             cp_async_commit();
             cp_async_wait<0>();
             __syncthreads();
-            step(reinterpret_cast<const Mt*>(ring), (jl > a0) ? reinterpret_cast<const S*>(ring + ub) : nullptr, t,
+            step(reinterpret_cast<const Mt*>(ring), (has_src && jl > a0) ? reinterpret_cast<const S*>(ring + ub) : nullptr, t,
                  emit_for(jl));
         }
     } else {
@@ -625,7 +628,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 1024) k_costate(Costate
             const int jl = b0 - t;
             unsigned char* sl = ring + (t % RING) * slot;
             ring_issue(sl, UHe + (size_t)jl * A.ustride, ub);
-            if (jl > a0) ring_issue(sl + ub, Se + (size_t)(jl - 1) * slice, pb);
+            if (has_src && jl > a0) ring_issue(sl + ub, Se + (size_t)(jl - 1) * slice, pb);
         };
 #pragma unroll 1
         for (int t = 0; t < RING - 1; ++t) {
@@ -641,7 +644,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 1024) k_costate(Costate
             if (tn < n) issue(tn);
             cp_async_commit();
             const unsigned char* sl = ring + (t % RING) * slot;
-            step(reinterpret_cast<const Mt*>(sl), (jl > a0) ? reinterpret_cast<const S*>(sl + ub) : nullptr, t,
+            step(reinterpret_cast<const Mt*>(sl), (has_src && jl > a0) ? reinterpret_cast<const S*>(sl + ub) : nullptr, t,
                  emit_for(jl));
         }
     }
@@ -678,7 +681,7 @@ template <typename R, typename S, typename Mt>
 static cudaError_t costate_dispatch(const CostateArgs<R>& a, cudaStream_t st) {
     const size_t panel = (size_t)a.d * a.sv.cb;
     const size_t ub = ring_bytes((size_t)a.d * a.d, sizeof(Mt));
-    const size_t pb = (size_t)a.sv.pstride * sizeof(S);
+    const size_t pb = (a.src || a.srck) ? (size_t)a.sv.pstride * sizeof(S) : 0;
     const size_t fixed = 2 * sizeof(K_t<R>) * panel + grid_block_bytes<R>(a.d, a.sv.cb);
     if (fixed > kMaxDynSmem) return cudaErrorInvalidValue;
     for (int ring : {8, 4, 2, 1}) {
@@ -694,12 +697,12 @@ static cudaError_t costate_dispatch(const CostateArgs<R>& a, cudaStream_t st) {
 
 template <typename R>
 cudaError_t launch_costate(const CostateArgs<R>& a, cudaStream_t st) {
-    if (a.wlen <= 0 || a.seg <= 0 || (a.zero_next && !a.cout) || (a.src != nullptr) == (a.srck != nullptr))
+    if (a.wlen <= 0 || a.seg <= 0 || (a.zero_next && !a.cout) || (a.src && a.srck))
         return cudaErrorInvalidValue;
     if ((a.U != nullptr) == (a.Uk != nullptr)) return cudaErrorInvalidValue;
     // carried sources go with carried matrices (the scan over segments), plain with plain
-    if (a.srck && a.Uk) return costate_dispatch<R, K_t<R>, K_t<R>>(a, st);
-    if (a.src && a.U) return costate_dispatch<R, C_t<R>, C_t<R>>(a, st);
+    if (!a.src && a.Uk) return costate_dispatch<R, K_t<R>, K_t<R>>(a, st);
+    if (!a.srck && a.U) return costate_dispatch<R, C_t<R>, C_t<R>>(a, st);
     return cudaErrorInvalidValue;
 }
 

@@ -301,9 +301,11 @@ void plan_impl(qoc_ctx* c) {
     if (c->scan && c->opt.ckpt_stride <= 0 && N >= 16) {
         // Checkpoint stride and panel width of the segmented form from a cost model of one wave's
         // sweeps: three passes of `seg` dependent steps over all segments at once (replay, the
-        // costate's two segment passes), each running in whole rounds of resident CTAs, and two
+        // costate's two segment passes; two for a terminal cost, which has no zero-carry pass), each running in whole rounds of resident CTAs, and two
         // scans of `nseg` steps (one CTA per panel); a CTA step costs col_cost(panel width).
         const long wave = ((long)N + 1) / 2;
+        const bool terminal = (c->nF == 0 || c->alpha[3] == 0.0) && c->alpha[4] == 0.0;
+        const double passes = terminal ? 2.0 : 3.0;
         double best = -1.0;
         int best_seg = seg;
         const int lo = std::max(4, (int)std::sqrt((double)N) / 2), hi = std::min(N, 2 * (int)std::ceil(std::sqrt((double)N)));
@@ -313,7 +315,7 @@ void plan_impl(qoc_ctx* c) {
                 if (w < 1) continue;
                 const long ctas = (long)((S + w - 1) / w) * E * nseg;
                 const long rounds = (ctas + want_ctas - 1) / want_ctas;
-                const double cost = col_cost(w) * (3.0 * sg * rounds + 2.0 * nseg);
+                const double cost = col_cost(w) * (passes * sg * rounds + 2.0 * nseg);
                 if (best < 0.0 || cost < best) {
                     best = cost;
                     best_seg = sg;
@@ -550,6 +552,10 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
                    c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]}};
     DevParams* prm = c->prm.as<DevParams>();
     const int seg = c->seg;
+    // A cost on the final state alone (gates, state transfer without C5 / C67) has one source, the
+    // terminal block: no source kernel, and in the segmented form no zero-carry pass over the
+    // segments (their h_z is zero), a fourth of the backward sweeps' work at S = d.
+    const bool terminal = cost_is_terminal(cv);
     // two sets of wave buffers: wave w uses set w % 2, so the serial sweep of one wave overlaps
     // the parallel kernels of its neighbour
     const size_t u_set = (size_t)E * W * c->ustride, s_set = (size_t)E * (W + 1) * slice, g_set = (size_t)E * W * slice;
@@ -748,7 +754,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
         a.U = Ub(w);
         a.ustride = c->ustride;
         a.u_es = (size_t)W * c->ustride;
-        a.src = Rb(w);
+        a.src = terminal ? nullptr : Rb(w);
         a.src_es = (size_t)W * slice;
         a.g_es = (size_t)W * slice;
         a.prm = prm;
@@ -771,17 +777,24 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
               "slice_costs", sx);
             rec(ev_fwd[w], sx);
         }
-        check_cuda(c, cudaMemsetAsync(c->carry.p, 0, c->carry.bytes, sx), "memset carry");
+        if (terminal) {
+            B(sx);
+            L(launch_terminal<R>(d, sv, E, cv, c->Ofin.as<double2>(), c->carry.as<K>(), sx), "sources", sx);
+        } else {
+            check_cuda(c, cudaMemsetAsync(c->carry.p, 0, c->carry.bytes, sx), "memset carry");
+        }
         rec(ev_fwd_done, sx);
         wait(st, ev_fwd_done);
         // ---- backward: recompute + replay of wave w - 1 on st overlap the costate of wave w on sx ----
         for (int w = nw - 1; w >= 0; --w) {
             const int j0 = w * W, wlen = std::min(W, N - j0);
             if (w != nw - 1) wait(sx, ev_rep[w]);           // the last wave is resident from the forward sweep
-            B(sx);
-            L(launch_sources<R>(d, sv, j0, wlen, N, E, Sb(w), W, cv, c->Oj.as<double2>(), c->Ofin.as<double2>(), Rb(w),
-                                sx),
-              "sources", sx);
+            if (!terminal) {
+                B(sx);
+                L(launch_sources<R>(d, sv, j0, wlen, N, E, Sb(w), W, cv, c->Oj.as<double2>(), c->Ofin.as<double2>(),
+                                    Rb(w), sx),
+                  "sources", sx);
+            }
             B(sx);
             CostateArgs<R> ca = costate_args(w);
             ca.seg = ca.wlen;                                // the whole wave as one segment
@@ -849,6 +862,10 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
         replay_costs(nw - 1);
         rec(ev_fwd_done, st);
         wait(sx, ev_fwd_done);
+        if (terminal) {
+            B(sx);
+            L(launch_terminal<R>(d, sv, E, cv, c->Ofin.as<double2>(), c->carry.as<K>(), sx), "sources", sx);
+        }
         // ---- backward: per wave, the costate of every segment from a zero in-carry, the scan
         //      Y_{z-1} = P_z^dag Y_z + h_z over segments, then every segment from its carry (sx);
         //      recompute + replay of wave w - 1 and the adjoint of wave w on st ----
@@ -856,16 +873,18 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             const int j0 = w * W, wlen = std::min(W, N - j0);
             const int nz = (wlen + seg - 1) / seg;
             if (w != nw - 1) wait(sx, ev_rep[w]);
-            B(sx);
-            L(launch_sources<R>(d, sv, j0, wlen, N, E, Sb(w), W, cv, c->Oj.as<double2>(), c->Ofin.as<double2>(), Rb(w),
-                                sx),
-              "sources", sx);
-            CostateArgs<R> loc = costate_args(w);
-            loc.cout = c->hbuf.as<K>();
-            loc.cout_es = (size_t)(nzmax + 1) * slice;
-            loc.zero_next = 1;
-            B(sx);
-            L(launch_costate<R>(loc, sx), "costate (segments)", sx);
+            if (!terminal) {
+                B(sx);
+                L(launch_sources<R>(d, sv, j0, wlen, N, E, Sb(w), W, cv, c->Oj.as<double2>(), c->Ofin.as<double2>(),
+                                    Rb(w), sx),
+                  "sources", sx);
+                CostateArgs<R> loc = costate_args(w);
+                loc.cout = c->hbuf.as<K>();
+                loc.cout_es = (size_t)(nzmax + 1) * slice;
+                loc.zero_next = 1;
+                B(sx);
+                L(launch_costate<R>(loc, sx), "costate (segments)", sx);
+            }
             CostateArgs<R> sc{};
             sc.prm = prm;
             sc.d = d;
@@ -876,12 +895,13 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             sc.Uk = Pb(w);
             sc.ustride = c->ustride;
             sc.u_es = (size_t)nzmax * c->ustride;
-            sc.srck = c->hbuf.as<K>() + slice;   // h_{z} is the source added after step z (slot nz is zero)
+            // h_{z} is the source added after step z (slot nz is zero); none for a terminal cost
+            sc.srck = terminal ? nullptr : c->hbuf.as<K>() + slice;
             sc.src_es = (size_t)(nzmax + 1) * slice;
             sc.Gk = Yb(w);
             sc.g_es = (size_t)nzmax * slice;
-            sc.cin = (w == nw - 1) ? nullptr : Yb(w + 1);
-            sc.cin_es = (size_t)nzmax * slice;
+            sc.cin = (w == nw - 1) ? (terminal ? c->carry.as<K>() : nullptr) : Yb(w + 1);
+            sc.cin_es = (w == nw - 1) ? slice : (size_t)nzmax * slice;
             B(sx);
             L(launch_costate<R>(sc, sx), "costate (scan)", sx);
             CostateArgs<R> fin = costate_args(w);

@@ -47,7 +47,7 @@ struct StateView {
 // Cost inputs (Table I).
 template <typename R>
 struct CostView {
-    int nF;
+    int nF;                 // forbidden basis states (0: fmask is all zero; an upper bound will do)
     const int* fmask;       // d: 1 for forbidden basis states
     const double* w;        // Spad column weights (0 on padding)
     double Wsum;            // sum of weights
@@ -358,7 +358,7 @@ struct CostateArgs {
     long long ustride;
     size_t u_es;
     const C_t<R>* src;      // src_j at src + e * src_es + j * slice ...
-    const K_t<R>* srck;     // ... or carried sources (exactly one of the two is set)
+    const K_t<R>* srck;     // ... or carried sources (at most one of the two is set; neither: none)
     size_t src_es;
     C_t<R>* G;              // G_j (rounded) at G + e * g_es + j * slice, or nullptr
     K_t<R>* Gk;             // G_j (carried), same layout, or nullptr
@@ -453,6 +453,15 @@ template <typename R>
 cudaError_t launch_sources(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* states,
                            int wmax, const CostView<R>& cv, const double2* Oj, const double2* Ofin,
                            C_t<R>* src, cudaStream_t st);
+// No cost term acts on the states of slices 1 .. N - 1 (no weight on C5 and C67): every source but
+// the last slice's is zero, so the costate is G_{j-1} = U_j^dag G_j from the terminal block alone
+template <typename R>
+inline bool cost_is_terminal(const CostView<R>& cv) {
+    return (cv.nF == 0 || cv.alpha[3] == 0.0) && cv.alpha[4] == 0.0;
+}
+template <typename R>
+cudaError_t launch_terminal(int d, StateView<R> sv, int E, const CostView<R>& cv, const double2* Ofin, K_t<R>* out,
+                            cudaStream_t st);
 // the paper's first-order gradient (Eq. 11) from Psi_j and G_j, in place of the exact adjoint
 template <typename R>
 cudaError_t launch_grad_first_order(const SysView<R>& sys, const StateView<R>& sv, int j0, int wlen, int E,

@@ -149,7 +149,7 @@ extern "C" qoc_status qoc_evaluate_static(int d, int M, int N, int S, double dt,
         return QOC_ERR_CUDA;
 
     SysView<R> sys{d, M, N, H0, Hk, nullptr, nullptr, u_dev};
-    CostView<R> cost{0, fmask_dev ? fmask_dev : fmask_zero, colw, (double)S, psiT, nullptr,
+    CostView<R> cost{fmask_dev ? d : 0, fmask_dev ? fmask_dev : fmask_zero, colw, (double)S, psiT, nullptr,
                      {alpha[0], alpha[1], alpha[2], alpha[3], alpha[4]}};
     ChainArgs<R> ch{d, sv, N, N, 0, 1, ckpt, slice, 0, 1, Ubuf, ustride, N, states, nullptr, prm};
     if (!ok(launch_theta(u_dev, M, N, norms, nullptr, 1, dt, 0.25, 1e-15, 0, -1, prm, st))) return QOC_ERR_CUDA;
