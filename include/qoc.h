@@ -195,7 +195,8 @@ typedef struct qoc_info {
                              2: state mode (matrix-vector Horner chains) */
     long long device_bytes; /* device memory held by the context */
     int adjoint_form;     /* gradient of the last evaluation: 0 reverse mode over the stored products
-                             (2 products per forward product), 1 block recursion (3), 2 first-order
+                             (2 products per forward product; on the batched path with few columns
+                             its cotangents may be kept as low-rank factors), 1 block recursion (3), 2 first-order
                              (Eq. 11, no adjoint exponential), 3 low-rank reverse mode (the cotangent
                              kept as d x r factors, r = 2^n S; small S, per-slice kernels), 4 the
                              state mode's reverse pass over its matrix-vector chain */

@@ -687,6 +687,10 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
         if (c->opt.gradient == QOC_GRAD_FIRST_ORDER)
             return launch_grad_first_order<R>(sys, sv, j0, wlen, E, Sb(w), Gb(w), W, c->dt, c->gpart.as<double>(), st);
         if constexpr (sizeof(R) == 4) {
+            // few columns: the same derivative with low-rank cotangents (BF16_SPLIT keeps its dense
+            // products on the tensor cores)
+            if (big && big_rev && c->ps && c->opt.precision == QOC_PREC_FP32 && big_lr_applies(d, sv.S, hp.p, hp.n))
+                return launch_big_adj_lr(big_args(w), sys, sv, Sb(w), Gb(w), c->gpart.as<double>(), hp, zbig(w), st);
             if (big && big_rev && c->ps) {       // Paterson-Stockmeyer reverse mode (tensor cores: BF16_SPLIT)
                 int n_l = 0;
                 OzRev oz{c->opt.fault_inject, prm, d, E * wlen, E * W, c->tc_planes.as<unsigned char>(), c->tc_maps,

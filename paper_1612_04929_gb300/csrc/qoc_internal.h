@@ -216,6 +216,11 @@ template <typename R>
 cudaError_t launch_big_adj_rev_ps(const BigArgs<R>& a, const SysView<R>& sys, const StateView<R>& sv,
                                   const C_t<R>* states, const C_t<R>* Gbuf, double* gpart, const DevParams& hp,
                                   const C_t<R>* zst, cudaStream_t st, int* launches, const OzRev* oz = nullptr);
+// its low-rank form (k_big_lr.cu, FP32 form, few columns): the cotangents kept as d x r factors
+bool big_lr_applies(int d, int S, int p, int n);
+cudaError_t launch_big_adj_lr(const BigArgs<float>& a, const SysView<float>& sys, const StateView<float>& sv,
+                              const float2* states, const float2* Gbuf, double* gpart, const DevParams& hp,
+                              const float2* zst, cudaStream_t st);
 template <typename R>
 cudaError_t launch_big_adj(const BigArgs<R>& a, const SysView<R>& sys, const StateView<R>& sv, const C_t<R>* states,
                            const C_t<R>* Gbuf, double* gpart, int p, int n, cudaStream_t st, int* launches);
