@@ -144,6 +144,7 @@ struct qoc_ctx {
     double theta_max = 0.0;              // in effect (the option, or the path's default)
     bool ps = false;                     // Paterson-Stockmeyer form of the per-slice FP32 exponential
     int nzmax = 0;                       // checkpoint segments per wave
+    int state_cs = 0;                    // state mode: CTAs per cluster of the recursions (0: one CTA)
     std::vector<int> cols;               // propagated columns (positive weight)
     size_t mstride = 0;                  // elements per matrix slot of the batched path
     long long ustride = 0;
@@ -401,6 +402,7 @@ void plan_impl(qoc_ctx* c) {
     const int nseg_total = c->nseg_total;
 
     StateView<R> sv{c->Spad, c->cb, c->ncb, c->pstride, c->S_eff};
+    c->state_cs = state_mode ? state_cluster_size<R>(d, sv, E) : 0;
     cudaStream_t st = c->stream;
     auto A = [&](DevBuf& b, size_t bytes, const char* what) { check_cuda(c, b.alloc(bytes), what); };
 
@@ -1080,7 +1082,7 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
         const int j0 = w * W, wlen = std::min(W, N - j0);
         StateChainArgs<R> a{d, E, wlen, 0, sv, X, xs, ck + (size_t)w * slice, ck_es,
                             (store_next && w + 1 < nw) ? ck + (size_t)(w + 1) * slice : nullptr, ck_es,
-                            states, (size_t)(W + 1) * slice, nullptr, 0, prm, chebd};
+                            states, (size_t)(W + 1) * slice, nullptr, 0, prm, chebd, c->state_cs};
         B();
         L(launch_state_chain<R>(a, st), "state_chain (forward)");
     };
@@ -1104,7 +1106,7 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
         L(launch_sources<R>(d, sv, j0, wlen, N, E, states, W, cv, c->Oj.as<double2>(), c->Ofin.as<double2>(), src, st),
           "sources");
         StateChainArgs<R> b{d, E, wlen, 1, sv, X, xs, c->carry.as<K>(), slice, c->carry.as<K>(), slice,
-                            G, (size_t)W * slice, src, (size_t)W * slice, prm, chebd};
+                            G, (size_t)W * slice, src, (size_t)W * slice, prm, chebd, c->state_cs};
         B();
         L(launch_state_chain<R>(b, st), "state_chain (costate)");
         if (c->opt.gradient == QOC_GRAD_FIRST_ORDER) {

@@ -423,7 +423,12 @@ struct StateChainArgs {
     size_t src_es;
     const DevParams* prm;
     const ChebCoef* cheb = nullptr;   // device coefficients: Chebyshev in place of Taylor
+    int cs = 0;                       // CTAs per cluster (state_cluster_size), 0: one CTA per panel
 };
+// the same recursion of single-column panels by a cluster of CTAs per (panel, member)
+// (k_state_cluster.cu); state_cluster_size: its size for a plan, 0 when k_state_chain takes it
+template <typename R> int state_cluster_size(int d, const StateView<R>& sv, int E);
+template <typename R> cudaError_t launch_state_cluster(const StateChainArgs<R>& a, cudaStream_t st);
 template <typename R>
 struct StateGradArgs {
     int d, E, M, N, j0, wlen, wmax;
