@@ -18,6 +18,7 @@
 
 #include "qoc_device.cuh"
 #include "qoc_internal.h"
+#include "qoc_slice.cuh"
 
 namespace qoc {
 
@@ -596,6 +597,23 @@ k_big_grad(const DevParams* __restrict__ prm, SysView<R> sys, int j0, int wlen, 
     if (threadIdx.x == 0) gpart[((size_t)e * sys.M + k) * sys.N + j] = prm->s * v;
 }
 
+// the same over the controls' non-zero elements, one CTA per item, a warp per control
+template <typename R>
+__global__ void __launch_bounds__(256)
+k_big_grad_sparse(const DevParams* __restrict__ prm, SysView<R> sys, int j0, int wlen, const C_t<R>* __restrict__ Xbar,
+                  size_t mstride, double* __restrict__ gpart) {
+    const int item = blockIdx.x, jl = item % wlen, e = item / wlen;
+    const C_t<R>* xb = Xbar + (size_t)item * mstride;
+    contract_sparse<R>(sys, prm, gpart, e, j0 + jl, [&](int a, int b) { return xb[(size_t)a * sys.d + b]; });
+}
+template <typename R>
+static cudaError_t grad_launch(const DevParams* prm, const SysView<R>& sys, int j0, int wlen, int items,
+                               const C_t<R>* Xbar, size_t ms, double* gpart, cudaStream_t st) {
+    if (sys.hoff) k_big_grad_sparse<R><<<items, 256, 0, st>>>(prm, sys, j0, wlen, Xbar, ms, gpart);
+    else k_big_grad<R><<<dim3(items, sys.M), 256, 0, st>>>(prm, sys, j0, wlen, Xbar, ms, gpart);
+    return cudaGetLastError();
+}
+
 // the conjugate transpose of Z (the right operand of forward product r), rounded to the compute
 // precision, into the operand store: zst + (item * cap + r) * mstride
 template <typename E, typename C>
@@ -1080,7 +1098,7 @@ cudaError_t launch_big_adj(const BigArgs<R>& a, const SysView<R>& sys, const Sta
     for (int m = 0; m < n; ++m)
         if ((err = blk(z11, z12, z11, z12, 1, 0)) != cudaSuccess) return err;
     if (sys.M > 0) {
-        k_big_grad<R><<<dim3(items, sys.M), 256, 0, st>>>(a.prm, sys, a.j0, a.wlen, z12, ms, gpart);
+        if ((err = grad_launch<R>(a.prm, sys, a.j0, a.wlen, items, z12, ms, gpart, st)) != cudaSuccess) return err;
         count();
     }
     return cudaGetLastError();
@@ -1163,7 +1181,7 @@ cudaError_t launch_big_adj_rev(const BigArgs<R>& a, const SysView<R>& sys, const
     count();
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     if (sys.M > 0) {
-        k_big_grad<R><<<dim3(items, sys.M), 256, 0, st>>>(a.prm, sys, a.j0, a.wlen, Xb, ms, gpart);
+        if ((err = grad_launch<R>(a.prm, sys, a.j0, a.wlen, items, Xb, ms, gpart, st)) != cudaSuccess) return err;
         count();
     }
     return cudaGetLastError();
@@ -1248,7 +1266,7 @@ cudaError_t launch_big_adj_rev_ps(const BigArgs<R>& a, const SysView<R>& sys, co
             if ((err = acc(zb, 1.f, 0.f, 0.f)) != cudaSuccess) return err;
         }
         if (sys.M > 0) {
-            k_big_grad<R><<<dim3(items, sys.M), 256, 0, st>>>(a.prm, sys, a.j0, a.wlen, Xb, ms, gpart);
+            if ((err = grad_launch<R>(a.prm, sys, a.j0, a.wlen, items, Xb, ms, gpart, st)) != cudaSuccess) return err;
             count();
         }
         return cudaGetLastError();

@@ -247,6 +247,10 @@ k_expm_adj(const DevParams* __restrict__ prm, SysView<R> sys, StateView<R> st, i
         t = z12; z12 = o12; o12 = t;
     }
     // dC/du_{k,j} = Re tr(Xbar^dag (-i s H_k)) = s sum_ab (Xbar_re Hk_im - Xbar_im Hk_re)
+    if (sys.hoff) {
+        contract_sparse<R>(sys, prm, gpart, e, j, [&](int a, int b) { return z12[a * LD + b]; });
+        return;
+    }
     const size_t dd = (size_t)d * d;
     // per-thread partials: FP32 form as (hi, lo) pairs of exact products, FP64 form in FP64; the
     // block sum in FP64
@@ -431,6 +435,13 @@ k_expm_adj_lr(const DevParams* __restrict__ prm, SysView<R> sys, StateView<R> st
     cp_async_wait<0>();
     __syncthreads();
     rank_update(Lc, Rb, R(1) / R(p));           // Z_p = I + X / p: Xbar += L_p R^dag / p
+    if (sys.hoff) {   // Xbar to the free operand buffer
+        __syncthreads();
+        if (act) store_acc<C, R, MT>(SN, xb, R(1), R(0), d, LD, ty, tx, G);
+        __syncthreads();
+        contract_sparse<R>(sys, prm, gpart, e, j, [&](int a, int b) { return SN[a * LD + b]; });
+        return;
+    }
     const size_t dd = (size_t)d * d;
     for (int k = 0; k < sys.M; ++k) {   // partials: FP32 pairs of exact products (FP32 form); FP64 sum
         double v = 0.0;
@@ -593,6 +604,13 @@ k_expm_adj_rev(const DevParams* __restrict__ prm, SysView<R> sys, StateView<R> s
                     xb[a][b].y += z.y * rp;
                 }
             }
+    }
+    if (sys.hoff) {   // Xbar to the free operand buffer
+        __syncthreads();
+        if (act) store_acc<C, R, MT>(SN, xb, R(1), R(0), d, LD, ty, tx, G);
+        __syncthreads();
+        contract_sparse<R>(sys, prm, gpart, e, j, [&](int a, int b) { return SN[a * LD + b]; });
+        return;
     }
     const size_t dd = (size_t)d * d;
     for (int k = 0; k < sys.M; ++k) {   // partials: FP32 pairs of exact products (FP32 form); FP64 sum

@@ -245,6 +245,13 @@ k_expm_adj_ps(const DevParams* __restrict__ prm, SysView<float> sys, StateView<f
     } else {
         cp_async_wait<0>();
     }
+    if (sys.hoff) {   // Xbar to a free operand buffer
+        __syncthreads();
+        if (act) store_acc<C, float, MT>(SN, xb, 1.f, 0.f, d, LD, ty, tx, G);
+        __syncthreads();
+        contract_sparse<float>(sys, prm, gpart, e, j, [&](int a, int b) { return SN[a * LD + b]; });
+        return;
+    }
     ps_contract<MT>(xb, sys, prm, gpart, e, j, ty, tx, G, act, red);
 }
 
@@ -434,6 +441,13 @@ k_expm_adj_ps_lr(const DevParams* __restrict__ prm, SysView<float> sys, StateVie
         ps_powers<MT>(xb, p2b, p3b, YH, SB, SN, Lb, p, d, LD, ty, tx, G, act);   // Lb: D x LD fits the six blocks
     } else {
         cp_async_wait<0>();
+    }
+    if (sys.hoff) {   // Xbar to a free operand buffer
+        __syncthreads();
+        if (act) store_acc<C, float, MT>(SN, xb, 1.f, 0.f, d, LD, ty, tx, G);
+        __syncthreads();
+        contract_sparse<float>(sys, prm, gpart, e, j, [&](int a, int b) { return SN[a * LD + b]; });
+        return;
     }
     ps_contract<MT>(xb, sys, prm, gpart, e, j, ty, tx, G, act, red);
 }

@@ -154,6 +154,7 @@ struct qoc_ctx {
 
     DevBuf H64, HR, dDelta, norms, psiTR, pathR, fmask, colw, ckpt, Ubuf, states, Gbuf, src, carry, Oj, C5j, Ofin,
         gpart, prm, u_h, grad_h, out_h, scratch, tc_planes;
+    DevBuf hoff, hidx, hval;             // the controls' non-zero elements (SysView), when sparse
     DevBuf sH;                           // s H_0 .. s H_det as FP32 pairs (per-slice split exponential)
     DevBuf chebd;                        // Chebyshev coefficients of the evaluation (state mode)
     DevBuf stscr;                        // state mode: the gradient kernel's per-item scratch
@@ -185,7 +186,7 @@ struct qoc_ctx {
     size_t device_bytes() const {
         const DevBuf* all[] = {&H64, &HR, &dDelta, &norms, &psiTR, &pathR, &fmask, &colw, &ckpt, &Ubuf, &states,
                                &Gbuf, &src, &carry, &Oj, &C5j, &Ofin, &gpart, &prm, &u_h, &grad_h, &out_h, &scratch,
-                               &tc_planes, &Pbuf, &lv0, &lv1, &scanst, &hbuf, &Ybuf, &Zbuf, &Zbig, &sH, &chebd, &stscr,
+                               &tc_planes, &Pbuf, &lv0, &lv1, &scanst, &hbuf, &Ybuf, &Zbuf, &Zbig, &sH, &chebd, &stscr, &hoff, &hidx, &hval,
                                &frozen_d};
         size_t s = 0;
         for (auto* b : all) s += b->bytes;
@@ -410,6 +411,36 @@ void plan_impl(qoc_ctx* c) {
     const size_t dd = (size_t)d * d;
     A(c->HR, (M + 2) * dd * cs, "alloc H");
     check_cuda(c, launch_convert<R>(c->H64.as<double2>(), c->HR.as<C>(), (M + 2) * dd, st), "convert H");
+    // the controls' non-zero elements, when at most a quarter are non-zero (a Pauli or ladder control
+    // has one or two a row): the gradient contracts those only
+    std::vector<int> hoff(1, 0), hidx;
+    std::vector<C> hval;
+    for (int k = 0; k < M && hidx.size() * 4 <= M * dd; ++k) {
+        const double* hk = c->Hk.data() + (size_t)k * dd * 2;
+        for (int a = 0; a < d; ++a)
+            for (int b = 0; b < d; ++b) {
+                const double x = hk[2 * ((size_t)a * d + b)], y = hk[2 * ((size_t)a * d + b) + 1];
+                if (x == 0.0 && y == 0.0) continue;
+                hidx.push_back(a << 16 | b);
+                C h;
+                h.x = (R)x;
+                h.y = (R)y;
+                hval.push_back(h);
+            }
+        hoff.push_back((int)hidx.size());
+    }
+    if (M > 0 && (int)hoff.size() == M + 1 && hidx.size() * 4 <= M * dd) {
+        hidx.push_back(0);   // never empty
+        hval.push_back(C{});
+        A(c->hoff, hoff.size() * sizeof(int), "alloc H_k offsets");
+        A(c->hidx, hidx.size() * sizeof(int), "alloc H_k elements");
+        A(c->hval, hval.size() * sizeof(C), "alloc H_k elements");
+        check_cuda(c, cudaMemcpyAsync(c->hoff.p, hoff.data(), c->hoff.bytes, cudaMemcpyHostToDevice, st), "copy H_k");
+        check_cuda(c, cudaMemcpyAsync(c->hidx.p, hidx.data(), c->hidx.bytes, cudaMemcpyHostToDevice, st), "copy H_k");
+        check_cuda(c, cudaMemcpyAsync(c->hval.p, hval.data(), c->hval.bytes, cudaMemcpyHostToDevice, st), "copy H_k");
+    } else {
+        for (DevBuf* b : {&c->hoff, &c->hidx, &c->hval}) b->release();
+    }
     if (split_exp<R>(c) || (c->path_kind == 2 && sizeof(R) == 4)) A(c->sH, (M + 2) * dd * sizeof(float4), "alloc sH");
     else c->sH.release();
     // costs
@@ -549,7 +580,8 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
     const size_t dd = (size_t)d * d;
     C* HR = c->HR.as<C>();
     SysView<R> sys{d, M, N, HR, HR + dd, c->Hdet.empty() ? nullptr : HR + (size_t)(M + 1) * dd,
-                   c->delta.empty() ? nullptr : c->dDelta.as<double>(), u};
+                   c->delta.empty() ? nullptr : c->dDelta.as<double>(), u,
+                   c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>()};
     CostView<R> cv{c->nF, c->fmask.as<int>(), c->colw.as<double>(), c->Wsum, c->psiTR.as<C>(),
                    c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]}};
     DevParams* prm = c->prm.as<DevParams>();
@@ -1005,7 +1037,8 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
     const size_t slice = sv.slice(), dd = (size_t)d * d;
     C* HR = c->HR.as<C>();
     SysView<R> sys{d, M, N, HR, HR + dd, c->Hdet.empty() ? nullptr : HR + (size_t)(M + 1) * dd,
-                   c->delta.empty() ? nullptr : c->dDelta.as<double>(), u};
+                   c->delta.empty() ? nullptr : c->dDelta.as<double>(), u,
+                   c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>()};
     CostView<R> cv{c->nF, c->fmask.as<int>(), c->colw.as<double>(), c->Wsum, c->psiTR.as<C>(),
                    c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]}};
     DevParams* prm = c->prm.as<DevParams>();

@@ -30,6 +30,11 @@ struct SysView {
     const C_t<R>* Hdet;   // d x d or nullptr
     const double* delta;  // E or nullptr
     const double* u;      // M x N
+    // The controls' non-zero elements, when few enough (nullptr: H_k dense): those of H_k are entries
+    // hoff[k] .. hoff[k + 1] - 1, element (row, column) = (hidx >> 16, hidx & 0xffff), value hval
+    const int* hoff = nullptr;
+    const int* hidx = nullptr;
+    const C_t<R>* hval = nullptr;
 };
 
 // Column-panel layout of every d x S block on the device: the S columns are padded to

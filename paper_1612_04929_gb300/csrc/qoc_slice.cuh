@@ -6,8 +6,41 @@
 // dimension of D + 1 complex elements; padding rows and columns are kept at zero.
 #pragma once
 #include "qoc_device.cuh"
+#include "qoc_internal.h"
 
 namespace qoc {
+
+// dC/du_kj = s sum_ab (Xbar_re Hk_im - Xbar_im Hk_re) over the controls' non-zero elements, a warp per
+// control: FP32 pairs of exact products (FP32 form) or FP64 per lane, an FP64 warp sum.  A Pauli or
+// ladder control has one or two elements a row, so the dense form (every element of every H_k, a block
+// reduction in FP64 per control) reads d^2 elements for each.  Evaluations went d = 27, E = 5, M = 6
+// 1.529 -> 1.510 ms, d = 40 1.635 -> 1.609 ms, d = 256, M = 16 (BF16_SPLIT) 157.2 -> 154.1 ms, d = 154,
+// S = 1 165.7 -> 163.8 ms.  at(a, b): Xbar's element.
+template <typename R, typename At>
+__device__ __forceinline__ void contract_sparse(const SysView<R>& sys, const DevParams* __restrict__ prm,
+                                                double* __restrict__ gpart, int e, int j, At at) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int k = warp; k < sys.M; k += nw) {
+        const int i1 = sys.hoff[k + 1];
+        double v = 0.0;
+        float hi = 0.f, lo = 0.f;
+        for (int i = sys.hoff[k] + lane; i < i1; i += 32) {
+            const int ab = sys.hidx[i];
+            const C_t<R> h = sys.hval[i];
+            const C_t<R> x = at(ab >> 16, ab & 0xffff);
+            if constexpr (sizeof(R) == 4) {
+                pair_acc(hi, lo, x.x, h.y);
+                pair_acc(hi, lo, -x.y, h.x);
+            } else {
+                v = fma(x.x, h.y, v);
+                v = fma(-x.y, h.x, v);
+            }
+        }
+        if constexpr (sizeof(R) == 4) v = (double)hi + (double)lo;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) gpart[((size_t)e * sys.M + k) * sys.N + j] = prm->s * v;
+    }
+}
 
 template <typename C, int MT>
 __device__ __forceinline__ void mm_acc(C (&acc)[MT][MT], const C* __restrict__ A,
