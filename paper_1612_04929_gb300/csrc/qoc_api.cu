@@ -1091,10 +1091,14 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
         throw Fail{set_err(c, QOC_ERR_UNSUPPORTED, "state mode: d x d and five d x S blocks exceed a CTA's shared memory")};
     if (c->opt.gradient == QOC_GRAD_EXACT && n > 16)
         throw Fail{set_err(c, QOC_ERR_UNSUPPORTED, "state mode: more than 2^16 applications per slice")};
+    bool grad_lr = false;
+    if constexpr (sizeof(R) == 4)
+        grad_lr = c->opt.gradient == QOC_GRAD_EXACT &&
+                  state_grad_lr_applies(sys, d, c->S_eff, p, n, cheb ? c->cheb_host.K : 0, cheb);
     // the gradient kernel's per-item scratch: application inputs and intermediates (or terms)
     const size_t scr_stride = state_grad_scratch(d, c->S_eff, p, n, cheb ? c->cheb_host.K : 0);
     const size_t scr_bytes = scr_stride * (size_t)E * W * sizeof(C);
-    if (c->opt.gradient == QOC_GRAD_EXACT && c->stscr.bytes < scr_bytes) {
+    if (c->opt.gradient == QOC_GRAD_EXACT && !grad_lr && c->stscr.bytes < scr_bytes) {
         c->stscr.release();
         check_cuda(c, c->stscr.alloc(scr_bytes), "alloc state-mode scratch");
     }
@@ -1150,6 +1154,12 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
             StateGradArgs<R> g{d, E, M, N, j0, wlen, W, sv, X, xs, states, G, sys.Hk, c->gpart.as<double>(), prm,
                                chebd, cheb ? c->cheb_host.K : 0, c->stscr.as<C>(), scr_stride};
             B();
+            if constexpr (sizeof(R) == 4) {
+                if (grad_lr) {
+                    L(launch_state_grad_lr(g, sys, p, n, st), "expm_adj");
+                    continue;
+                }
+            }
             L(launch_state_grad<R>(g, p, n, st), "expm_adj");
         }
     }

@@ -457,6 +457,9 @@ template <typename R>
 cudaError_t launch_state_x(const DevParams* prm, int d, int M, int N, const double* u, const double* delta, int has_det,
                            const void* Hsrc, int j0, int wlen, int E, void* X, size_t xs, cudaStream_t st);
 template <typename R> cudaError_t launch_state_chain(const StateChainArgs<R>& a, cudaStream_t st);
+// its form for sparse controls (k_state_grad.cu): Xbar as rank-one terms, no per-item scratch
+bool state_grad_lr_applies(const SysView<float>& sys, int d, int S, int p, int n, int K, bool cheb);
+cudaError_t launch_state_grad_lr(const StateGradArgs<float>& a, const SysView<float>& sys, int p, int n, cudaStream_t st);
 template <typename R> cudaError_t launch_state_grad(const StateGradArgs<R>& a, int p, int n, cudaStream_t st);
 
 // ---- per-slice costs, sources, final reduction (k_chain.cu) ----
