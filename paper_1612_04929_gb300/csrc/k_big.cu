@@ -17,6 +17,7 @@
 #include <utility>
 
 #include "qoc_device.cuh"
+#include "qoc_gemm.cuh"
 #include "qoc_internal.h"
 #include "qoc_slice.cuh"
 
@@ -49,14 +50,6 @@ template <typename E> __device__ __forceinline__ E ezero();
 template <> __device__ __forceinline__ float4 ezero<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 template <> __device__ __forceinline__ float2 ezero<float2>() { return make_float2(0.f, 0.f); }
 template <> __device__ __forceinline__ double2 ezero<double2>() { return make_double2(0.0, 0.0); }
-
-// Tile rows owned by a thread are ty + 16 x; rows at or past d (edge tiles) add nothing.  The
-// number of x a warp has to run: the largest over its lanes, so that the skip is warp-uniform.
-__device__ __forceinline__ int warp_rows(int valid, int ty, int MT) {
-    int xs = 0;
-    while (xs < MT && ty + 16 * xs < valid) ++xs;
-    return __reduce_max_sync(0xffffffffu, (unsigned)xs);
-}
 
 // ------------------------------------------------------------------------------------------
 // assembly: X = -i s H_j (+ delta_e H_det) from FP64 H; Z = I + X / p
@@ -180,122 +173,33 @@ struct PsAdd {
     float2 c0{0.f, 0.f}, c1{0.f, 0.f}, c2{0.f, 0.f};
 };
 
-template <typename E, int T, int MODE>   // MODE 0 plain, 1 split, 2 plain FP32 (E = float4)
-__global__ void __launch_bounds__(256)
+template <typename E, class Sh, int MODE>   // MODE 0 plain, 1 split, 2 plain FP32 (E = float4)
+__global__ void __launch_bounds__(Sh::NT, Sh::MB)
 k_big_mm(int d, const E* __restrict__ A, const E* __restrict__ B, E* __restrict__ Cm, size_t mstride, int kind, int i,
-         float magic, PsAdd ps) {
-    constexpr int MT = T / 16;
-    // two buffers of (As[T][KC + 1], Bs[KC][T + 1]): the next K-chunk is copied (cp.async) while
-    // the current one is multiplied
+         float magic, PsAdd ps, int ntn) {
+    constexpr int MT = Sh::MT, G = Sh::G;
     extern __shared__ __align__(16) unsigned char smraw[];
-    typedef E ATile[T][KC + 1];
-    typedef E BTile[KC][T + 1];
-    ATile* Abuf = reinterpret_cast<ATile*>(smraw);
-    BTile* Bbuf = reinterpret_cast<BTile*>(smraw + 2 * sizeof(ATile));
     const int item = blockIdx.y;
-    const int ntn = (d + T - 1) / T;
-    const int tm = blockIdx.x / ntn, tn = blockIdx.x - tm * ntn;
-    const int r0 = tm * T, c0 = tn * T;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int xw = warp_rows(d - r0, ty, MT);
+    const GemmPos<Sh> p(blockIdx.x, ntn, d);
     const E* Ai = A + (size_t)item * mstride;
     const E* Bi = B + (size_t)item * mstride;
-    // split accumulators: grid sums (re, im) exact, cross terms (re, im); MODE 2 uses [0], [1]
-    float sa[MT][MT][4];
-    E acc[MT][MT];
-#pragma unroll
-    for (int x = 0; x < MT; ++x)
-#pragma unroll
-        for (int y = 0; y < MT; ++y) {
-            sa[x][y][0] = sa[x][y][1] = sa[x][y][2] = sa[x][y][3] = 0.f;
-            acc[x][y] = ezero<E>();
-        }
-    auto issue = [&](int buf, int k0) {
-        for (int idx = tid; idx < T * KC; idx += 256) {
-            const int r = idx / KC, k = idx - r * KC;
-            const int gr = r0 + r, gk = k0 + k;
-            if (gr < d && gk < d) cp_async_elem(&Abuf[buf][r][k], &Ai[(size_t)gr * d + gk]);
-            else Abuf[buf][r][k] = ezero<E>();
-        }
-        for (int idx = tid; idx < KC * T; idx += 256) {
-            const int k = idx / T, c = idx - k * T;
-            const int gk = k0 + k, gc = c0 + c;
-            if (gk < d && gc < d) cp_async_elem(&Bbuf[buf][k][c], &Bi[(size_t)gk * d + gc]);
-            else Bbuf[buf][k][c] = ezero<E>();
-        }
+    std::conditional_t<MODE == 0, MacPlain<E, MT>, std::conditional_t<MODE == 1, MacSplit<MT>, MacFull<MT>>> mac;
+    auto& sa = mac.acc;
+    auto la = [&](int r, int k, E* dst) {
+        if (r < d && k < d) cp_async_elem(dst, &Ai[(size_t)r * d + k]);
+        else *dst = ezero<E>();
     };
-    const int nch = (d + KC - 1) / KC;
-    issue(0, 0);
-    cp_async_commit();
-    for (int ch = 0; ch < nch; ++ch) {
-        if (ch + 1 < nch) issue((ch + 1) & 1, (ch + 1) * KC);
-        cp_async_commit();
-        cp_async_wait<1>();   // chunk ch has landed
-        __syncthreads();
-        const ATile& As = Abuf[ch & 1];
-        const BTile& Bs = Bbuf[ch & 1];
-        const int kmax = min(KC, d - ch * KC);   // the last chunk may be partial (zero-padded)
-#pragma unroll 4
-        for (int k = 0; k < kmax; ++k) {
-            E a[MT], b[MT];
-#pragma unroll
-            for (int x = 0; x < MT; ++x) a[x] = As[ty + 16 * x][k];
-#pragma unroll
-            for (int y = 0; y < MT; ++y) b[y] = Bs[k][tx + 16 * y];
-            float2 bf[MT], af[MT];   // full values: of B (MODE 1), of A (MODE 2)
-#pragma unroll
-            for (int y = 0; y < MT; ++y) {
-                if constexpr (MODE == 1) {
-                    const float4 bv = *reinterpret_cast<const float4*>(&b[y]);
-                    bf[y] = make_float2(bv.x + bv.z, bv.y + bv.w);
-                }
-                if constexpr (MODE == 2) {
-                    const float4 av = *reinterpret_cast<const float4*>(&a[y]);
-                    af[y] = make_float2(av.x + av.z, av.y + av.w);
-                }
-            }
-#pragma unroll
-            for (int x = 0; x < MT; ++x) {
-                if (x >= xw) break;   // rows past d in every lane of this warp
-#pragma unroll
-                for (int y = 0; y < MT; ++y) {
-                    if constexpr (MODE == 1) {
-                        const float4 av = *reinterpret_cast<const float4*>(&a[x]);
-                        const float4 bv = *reinterpret_cast<const float4*>(&b[y]);
-                        float* c = sa[x][y];
-                        c[0] = fmaf(av.x, bv.x, c[0]);
-                        c[0] = fmaf(-av.y, bv.y, c[0]);
-                        c[1] = fmaf(av.x, bv.y, c[1]);
-                        c[1] = fmaf(av.y, bv.x, c[1]);
-                        c[2] = fmaf(av.x, bv.z, c[2]);
-                        c[2] = fmaf(-av.y, bv.w, c[2]);
-                        c[2] = fmaf(av.z, bf[y].x, c[2]);
-                        c[2] = fmaf(-av.w, bf[y].y, c[2]);
-                        c[3] = fmaf(av.x, bv.w, c[3]);
-                        c[3] = fmaf(av.y, bv.z, c[3]);
-                        c[3] = fmaf(av.z, bf[y].y, c[3]);
-                        c[3] = fmaf(av.w, bf[y].x, c[3]);
-                    } else if constexpr (MODE == 2) {
-                        const float4 bv = *reinterpret_cast<const float4*>(&b[y]);
-                        float* c = sa[x][y];
-                        c[0] = fmaf(af[x].x, bv.x, c[0]);
-                        c[0] = fmaf(-af[x].y, bv.y, c[0]);
-                        c[1] = fmaf(af[x].x, bv.y, c[1]);
-                        c[1] = fmaf(af[x].y, bv.x, c[1]);
-                    } else {
-                        cfma(acc[x][y], a[x], b[y]);
-                    }
-                }
-            }
-        }
-        __syncthreads();   // before this buffer is refilled
-    }
+    auto lb = [&](int k, int c, E* dst) {
+        if (k < d && c < d) cp_async_elem(dst, &Bi[(size_t)k * d + c]);
+        else *dst = ezero<E>();
+    };
+    gemm_loop<E>(smraw, p, d, la, lb, mac);
     E* Ci = Cm + (size_t)item * mstride;
 #pragma unroll
     for (int x = 0; x < MT; ++x)
 #pragma unroll
         for (int y = 0; y < MT; ++y) {
-            const int r = r0 + ty + 16 * x, c = c0 + tx + 16 * y;
+            const int r = p.r0 + p.ty + G * x, c = p.c0 + p.tx + G * y;
             if (r >= d || c >= d) continue;
             const bool diag = (kind == 0) && (r == c);
             E out;
@@ -342,7 +246,7 @@ k_big_mm(int d, const E* __restrict__ A, const E* __restrict__ B, E* __restrict_
                 }
                 out = *reinterpret_cast<E*>(&o);
             } else {
-                out = acc[x][y];
+                out = sa[x][y];
                 if (kind == 0) {
                     using S = decltype(out.x);
                     const S ri = S(1) / S(i);
@@ -693,115 +597,52 @@ struct RevOps {
     const C* p[4];          // A1, B1, A2, B2
     size_t s[4];            // item strides
 };
-template <typename C, int T>
-__global__ void __launch_bounds__(256)
-k_big_rev(int d, RevOps<C> ops, C* __restrict__ O1, C* __restrict__ O2, size_t mstride, int mode, int i) {
-    constexpr int MT = T / 16;
+template <typename C, class Sh>
+__global__ void __launch_bounds__(Sh::NT, Sh::MB)
+k_big_rev(int d, RevOps<C> ops, C* __restrict__ O1, C* __restrict__ O2, size_t mstride, int mode, int i, int ntn) {
+    constexpr int MT = Sh::MT, G = Sh::G;
     extern __shared__ __align__(16) unsigned char smraw[];
-    typedef C ATile[T][KC + 1];
-    typedef C BTile[KC][T + 1];
-    ATile* A1b = reinterpret_cast<ATile*>(smraw);
-    ATile* A2b = A1b + 2;
-    BTile* B1b = reinterpret_cast<BTile*>(smraw + 4 * sizeof(ATile));
-    BTile* B2b = B1b + 2;
     const int item = blockIdx.y;
-    const int ntn = (d + T - 1) / T;
-    const int tm = blockIdx.x / ntn, tn = blockIdx.x - tm * ntn;
-    const int r0 = tm * T, c0 = tn * T;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int xw = warp_rows(d - r0, ty, MT);
-    const C* A1 = ops.p[0] + (size_t)item * ops.s[0];
-    const C* B1 = ops.p[1] + (size_t)item * ops.s[1];
-    const C* A2 = ops.p[2] + (size_t)item * ops.s[2];
-    const C* B2 = ops.p[3] + (size_t)item * ops.s[3];
-    C acc1[MT][MT], acc2[MT][MT];
-#pragma unroll
-    for (int x = 0; x < MT; ++x)
-#pragma unroll
-        for (int y = 0; y < MT; ++y) acc1[x][y] = acc2[x][y] = czero<C>();
-    auto issue = [&](int buf, int k0) {
-        for (int idx = tid; idx < T * KC; idx += 256) {
-            const int r = idx / KC, k = idx - r * KC;
-            const int gr = r0 + r, gk = k0 + k;
-            if (gr < d && gk < d) {
-                cp_async_elem(&A1b[buf][r][k], &A1[(size_t)gr * d + gk]);
-                cp_async_elem(&A2b[buf][r][k], &A2[(size_t)gr * d + gk]);
-            } else {
-                A1b[buf][r][k] = czero<C>();
-                A2b[buf][r][k] = czero<C>();
-            }
-        }
-        for (int idx = tid; idx < KC * T; idx += 256) {
-            const int k = idx / T, c = idx - k * T;
-            const int gk = k0 + k, gc = c0 + c;
-            if (gk < d && gc < d) {
-                cp_async_elem(&B1b[buf][k][c], &B1[(size_t)gk * d + gc]);
-                cp_async_elem(&B2b[buf][k][c], &B2[(size_t)gk * d + gc]);
-            } else {
-                B1b[buf][k][c] = czero<C>();
-                B2b[buf][k][c] = czero<C>();
-            }
-        }
+    const GemmPos<Sh> p(blockIdx.x, ntn, d);
+    const size_t off = (size_t)item * mstride;
+    using S = decltype(ops.p[0]->x);
+    const S ri = (mode == 0) ? S(1) / S(i) : S(1);
+    MacPlain<C, MT> mac;
+    auto mul = [&](int q) {   // acc += operands q, q + 1
+        const C* A = ops.p[q] + (size_t)item * ops.s[q];
+        const C* B = ops.p[q + 1] + (size_t)item * ops.s[q + 1];
+        auto la = [&](int r, int k, C* dst) {
+            if (r < d && k < d) cp_async_elem(dst, &A[(size_t)r * d + k]);
+            else *dst = czero<C>();
+        };
+        auto lb = [&](int k, int c, C* dst) {
+            if (k < d && c < d) cp_async_elem(dst, &B[(size_t)k * d + c]);
+            else *dst = czero<C>();
+        };
+        gemm_loop<C>(smraw, p, d, la, lb, mac);
     };
-    const int nch = (d + KC - 1) / KC;
-    issue(0, 0);
-    cp_async_commit();
-    for (int ch = 0; ch < nch; ++ch) {
-        if (ch + 1 < nch) issue((ch + 1) & 1, (ch + 1) * KC);
-        cp_async_commit();
-        cp_async_wait<1>();   // chunk ch has landed
-        __syncthreads();
-        const ATile& A1s = A1b[ch & 1];
-        const ATile& A2s = A2b[ch & 1];
-        const BTile& B1s = B1b[ch & 1];
-        const BTile& B2s = B2b[ch & 1];
-        const int kmax = min(KC, d - ch * KC);   // the last chunk may be partial (zero-padded)
-#pragma unroll 4
-        for (int k = 0; k < kmax; ++k) {
-            C a1[MT], a2[MT], b1[MT], b2[MT];
+    auto store = [&](C* O, bool add) {
 #pragma unroll
-            for (int x = 0; x < MT; ++x) {
-                a1[x] = A1s[ty + 16 * x][k];
-                a2[x] = A2s[ty + 16 * x][k];
-            }
+        for (int x = 0; x < MT; ++x)
 #pragma unroll
             for (int y = 0; y < MT; ++y) {
-                b1[y] = B1s[k][tx + 16 * y];
-                b2[y] = B2s[k][tx + 16 * y];
+                const int r = p.r0 + p.ty + G * x, c = p.c0 + p.tx + G * y;
+                if (r >= d || c >= d) continue;
+                C v = add ? O[off + (size_t)r * d + c] : czero<C>();
+                v.x += mac.acc[x][y].x * ri;
+                v.y += mac.acc[x][y].y * ri;
+                O[off + (size_t)r * d + c] = v;
             }
-#pragma unroll
-            for (int x = 0; x < MT; ++x) {
-                if (x >= xw) break;   // rows past d in every lane of this warp
-#pragma unroll
-                for (int y = 0; y < MT; ++y) {
-                    cfma(acc1[x][y], a1[x], b1[y]);
-                    if (mode == 0) cfma(acc2[x][y], a2[x], b2[y]);
-                    else cfma(acc1[x][y], a2[x], b2[y]);
-                }
-            }
-        }
-        __syncthreads();   // before this buffer is refilled
+    };
+    // one accumulator tile at a time: mode 0 the two outputs one after the other, mode 1 both products
+    // into one
+    mul(0);
+    if (mode == 0) {
+        store(O1, false);
+        mac = MacPlain<C, MT>{};
     }
-    using S = decltype(acc1[0][0].x);
-    const S ri = (mode == 0) ? S(1) / S(i) : S(1);
-    const size_t off = (size_t)item * mstride;
-#pragma unroll
-    for (int x = 0; x < MT; ++x)
-#pragma unroll
-        for (int y = 0; y < MT; ++y) {
-            const int r = r0 + ty + 16 * x, c = c0 + tx + 16 * y;
-            if (r >= d || c >= d) continue;
-            C v1 = acc1[x][y];
-            v1.x *= ri;
-            v1.y *= ri;
-            O1[off + (size_t)r * d + c] = v1;
-            if (mode == 0) {
-                C v2 = O2[off + (size_t)r * d + c];
-                v2.x += acc2[x][y].x * ri;
-                v2.y += acc2[x][y].y * ri;
-                O2[off + (size_t)r * d + c] = v2;
-            }
-        }
+    mul(2);
+    store(mode == 0 ? O2 : O1, mode == 0);
 }
 
 // Xbar += Zbar / p (the last Horner factor Z_p = I + X / p)
@@ -828,26 +669,34 @@ static int big_tile(int d) { return d <= 96 ? 32 : 64; }
 template <typename E, int T> constexpr size_t mm_smem() { return 2 * sizeof(E) * ((size_t)T * (KC + 1) + (size_t)KC * (T + 1)); }
 template <typename E, int T> constexpr size_t blk_smem() { return 2 * mm_smem<E, T>(); }
 
-template <typename E, int T, int MODE>
+template <typename E, class Sh, int MODE>
 static cudaError_t mm_launch_t(int d, int items, const E* A, const E* B, E* Cm, size_t mstride, int kind, int i,
                                float magic, cudaStream_t st, const PsAdd& ps) {
-    constexpr size_t smem = mm_smem<E, T>();
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_big_mm<E, T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    const int nt = ((d + T - 1) / T) * ((d + T - 1) / T);
-    k_big_mm<E, T, MODE><<<dim3(nt, items), 256, smem, st>>>(d, A, B, Cm, mstride, kind, i, magic, ps);
+    constexpr size_t smem = Sh::template smem<E>();
+    cudaError_t e = cudaFuncSetAttribute(k_big_mm<E, Sh, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int n = Sh::tiles(d);
+    k_big_mm<E, Sh, MODE><<<dim3(n * n, items), Sh::NT, smem, st>>>(d, A, B, Cm, mstride, kind, i, magic, ps, n);
     return cudaGetLastError();
 }
-
 template <typename E, int MODE>
 static cudaError_t mm_launch(int d, int items, const E* A, const E* B, E* Cm, size_t mstride, int kind, int i,
                              cudaStream_t st, float magic = 0.f, const PsAdd& ps = PsAdd{}) {
-    if (big_tile(d) == 32) return mm_launch_t<E, 32, MODE>(d, items, A, B, Cm, mstride, kind, i, magic, st, ps);
-    return mm_launch_t<E, 64, MODE>(d, items, A, B, Cm, mstride, kind, i, magic, st, ps);
+#define QOC_MM(Sh) return mm_launch_t<E, Sh, MODE>(d, items, A, B, Cm, mstride, kind, i, magic, st, ps)
+    if constexpr (sizeof(E) == 16 && MODE == 0) {          // FP64
+        QOC_MM(GemmWide);
+    } else if constexpr (sizeof(E) == 16) {
+        QOC_MM(GemmSplit);
+    } else {
+        switch (gemm_plain_mt(d)) {
+            case 4:
+                if (d % GemmPlain4::T == 0) QOC_MM(GemmPlain4F);
+                QOC_MM(GemmPlain4);
+            case 5: QOC_MM(GemmPlain5);
+            default: QOC_MM(GemmPlain6);
+        }
+    }
+#undef QOC_MM
 }
 
 template <typename C, int T>
@@ -1104,19 +953,30 @@ cudaError_t launch_big_adj(const BigArgs<R>& a, const SysView<R>& sys, const Sta
     return cudaGetLastError();
 }
 
-template <typename C, int T>
+template <typename C, class Sh>
 static cudaError_t rev_launch_t(int d, int items, const RevOps<C>& ops, C* O1, C* O2, size_t ms, int mode, int i,
                                 cudaStream_t st) {
-    constexpr size_t smem = blk_smem<C, T>();
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_big_rev<C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    const int nt = ((d + T - 1) / T) * ((d + T - 1) / T);
-    k_big_rev<C, T><<<dim3(nt, items), 256, smem, st>>>(d, ops, O1, O2, ms, mode, i);
+    constexpr size_t smem = Sh::template smem<C>();
+    cudaError_t e = cudaFuncSetAttribute(k_big_rev<C, Sh>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int n = Sh::tiles(d);
+    k_big_rev<C, Sh><<<dim3(n * n, items), Sh::NT, smem, st>>>(d, ops, O1, O2, ms, mode, i, n);
     return cudaGetLastError();
+}
+template <typename C>
+static cudaError_t rev_launch(int d, int items, const RevOps<C>& ops, C* O1, C* O2, size_t ms, int mode, int i,
+                              cudaStream_t st) {
+    if constexpr (sizeof(C) == 16) {
+        return rev_launch_t<C, GemmWide>(d, items, ops, O1, O2, ms, mode, i, st);
+    } else {
+        switch (gemm_plain_mt(d)) {
+            case 4:
+                if (d % GemmPlain4::T == 0) return rev_launch_t<C, GemmPlain4F>(d, items, ops, O1, O2, ms, mode, i, st);
+                return rev_launch_t<C, GemmPlain4>(d, items, ops, O1, O2, ms, mode, i, st);
+            case 5: return rev_launch_t<C, GemmPlain5>(d, items, ops, O1, O2, ms, mode, i, st);
+            default: return rev_launch_t<C, GemmPlain6>(d, items, ops, O1, O2, ms, mode, i, st);
+        }
+    }
 }
 
 template <typename R>
@@ -1143,7 +1003,6 @@ cudaError_t launch_big_adj_rev(const BigArgs<R>& a, const SysView<R>& sys, const
     if ((err = mm_launch<C, 0>(d, items, Zb, Xb, Za, ms, 1, 0, st)) != cudaSuccess) return err;
     count();
     if ((err = cudaMemsetAsync(Xb, 0, (size_t)items * ms * sizeof(C), st)) != cudaSuccess) return err;
-    const int T = (sizeof(C) == 16) ? 32 : big_tile(d);
     C *zb = Za, *zo = Zb;
     // tensor-core products (BF16_SPLIT): X^dag is sliced once for the wave
     int xh_sliced = 0;
@@ -1163,8 +1022,7 @@ cudaError_t launch_big_adj_rev(const BigArgs<R>& a, const SysView<R>& sys, const
                 return e2;
             }
         }
-        e2 = (T == 32) ? rev_launch_t<C, 32>(d, items, ops, zo, O2, ms, mode, i, st)
-                       : rev_launch_t<C, 64>(d, items, ops, zo, O2, ms, mode, i, st);
+        e2 = rev_launch<C>(d, items, ops, zo, O2, ms, mode, i, st);
         count();
         std::swap(zb, zo);
         return e2;
@@ -1219,7 +1077,6 @@ cudaError_t launch_big_adj_rev_ps(const BigArgs<R>& a, const SysView<R>& sys, co
         if ((err = mm_launch<C, 0>(d, items, Zb, Xb, Za, ms, 1, 0, st)) != cudaSuccess) return err;
         count();
         if ((err = cudaMemsetAsync(Xb, 0, 3 * (size_t)items * ms * sizeof(C), st)) != cudaSuccess) return err;
-        const int T = big_tile(d);
         C *zb = Za, *zo = Zb;
         int xh_sliced = 0;
         OzRev tc{};
@@ -1234,8 +1091,7 @@ cudaError_t launch_big_adj_rev_ps(const BigArgs<R>& a, const SysView<R>& sys, co
                 const float2* o4[4] = {ops.p[0], ops.p[1], ops.p[2], ops.p[3]};
                 e2 = oz_rev_step(tc, o4, ops.s, zo, O2, ms, mode, 1, st, launches);
             } else {
-                e2 = (T == 32) ? rev_launch_t<C, 32>(d, items, ops, zo, O2, ms, mode, 1, st)
-                               : rev_launch_t<C, 64>(d, items, ops, zo, O2, ms, mode, 1, st);
+                e2 = rev_launch<C>(d, items, ops, zo, O2, ms, mode, 1, st);
                 count();
             }
             std::swap(zb, zo);
