@@ -193,7 +193,7 @@ k_big_mm(int d, const E* __restrict__ A, const E* __restrict__ B, E* __restrict_
         if (k < d && c < d) cp_async_elem(dst, &Bi[(size_t)k * d + c]);
         else *dst = ezero<E>();
     };
-    gemm_loop<E>(smraw, p, d, la, lb, mac);
+    gemm_loop<E, Sh>(smraw, p, d, la, lb, mac);
     E* Ci = Cm + (size_t)item * mstride;
 #pragma unroll
     for (int x = 0; x < MT; ++x)
@@ -619,7 +619,7 @@ k_big_rev(int d, RevOps<C> ops, C* __restrict__ O1, C* __restrict__ O2, size_t m
             if (k < d && c < d) cp_async_elem(dst, &B[(size_t)k * d + c]);
             else *dst = czero<C>();
         };
-        gemm_loop<C>(smraw, p, d, la, lb, mac);
+        gemm_loop<C, Sh>(smraw, p, d, la, lb, mac);
     };
     auto store = [&](C* O, bool add) {
 #pragma unroll

@@ -364,7 +364,8 @@ k_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, const C_t<R>* __r
     const C* psi = states + ((size_t)e * (wmax + 1) + jl + 1) * slice;
     const C* T = cv.path ? cv.path + (size_t)j * slice : cv.psiT;
     const bool last = (j == N - 1), forb = cv.nF > 0;
-    const int rows = ts / cb, a0 = t0 / cb, s0 = t0 - a0 * cb;
+    // panels wider than the threads (one panel of all columns) are walked in chunks of ts columns
+    const int cw = cb < ts ? cb : ts, rows = ts / cw, a0 = t0 / cw, sc = t0 - a0 * cw;
     RunSum<R> so[2], sf[2], s5;
     double ore = 0, oim = 0, c5 = 0, fre = 0, fim = 0, w = 0.0;
     auto flush = [&]() {
@@ -377,7 +378,9 @@ k_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, const C_t<R>* __r
         }
     };
     if (a0 < rows)
-        for (int kb = 0; kb < sv.ncb; ++kb) {
+        for (int ch = 0, nch = (cb + cw - 1) / cw; ch < sv.ncb * nch; ++ch) {
+            const int kb = ch / nch, s0 = (ch - kb * nch) * cw + sc;
+            if (s0 >= cb) continue;
             const double wk = cv.w[kb * cb + s0];
             if (wk != w) {
                 if (w != 0.0) flush();

@@ -141,6 +141,8 @@ struct qoc_ctx {
     int W = 0, nw = 0, seg = 0, nseg_total = 0, path_kind = 0;
     int Spad = 0, cb = 0, ncb = 0, pstride = 0, S_eff = 0;
     bool scan = false;                   // segmented-scan form of the two recursions
+    bool tree = false;                   // both recursions over the wave's binary tree (k_tree.cu)
+    float tree_mo[2] = {0.f, 0.f};       // its grids: of the states (norms of Psi_0), of the costates (Psi_T)
     double theta_max = 0.0;              // in effect (the option, or the path's default)
     bool ps = false;                     // Paterson-Stockmeyer form of the per-slice FP32 exponential
     int nzmax = 0;                       // checkpoint segments per wave
@@ -154,6 +156,7 @@ struct qoc_ctx {
 
     DevBuf H64, HR, dDelta, norms, psiTR, pathR, fmask, colw, ckpt, Ubuf, states, Gbuf, src, carry, Oj, C5j, Ofin,
         gpart, prm, u_h, grad_h, out_h, scratch, tc_planes;
+    DevBuf tnodes, tcarry, tcoef, tgtK;  // tree form: nodes (two wave sets), carried blocks, coefficients, Psi_T
     DevBuf hoff, hidx, hval;             // the controls' non-zero elements (SysView), when sparse
     DevBuf sH;                           // s H_0 .. s H_det as FP32 pairs (per-slice split exponential)
     DevBuf chebd;                        // Chebyshev coefficients of the evaluation (state mode)
@@ -187,6 +190,7 @@ struct qoc_ctx {
         const DevBuf* all[] = {&H64, &HR, &dDelta, &norms, &psiTR, &pathR, &fmask, &colw, &ckpt, &Ubuf, &states,
                                &Gbuf, &src, &carry, &Oj, &C5j, &Ofin, &gpart, &prm, &u_h, &grad_h, &out_h, &scratch,
                                &tc_planes, &Pbuf, &lv0, &lv1, &scanst, &hbuf, &Ybuf, &Zbuf, &Zbig, &sH, &chebd, &stscr, &hoff, &hidx, &hval,
+                               &tnodes, &tcarry, &tcoef, &tgtK,
                                &frozen_d};
         size_t s = 0;
         for (auto* b : all) s += b->bytes;
@@ -327,6 +331,31 @@ void plan_impl(qoc_ctx* c) {
         }
         seg = best_seg;
     }
+    // Full unitaries with a cost on the final state alone: both recursions as batched products over the
+    // wave's tree, from d = 48 on (below, a chain step costs a few us and the tree's launches more).
+    // The blocks are then one panel of all columns (row-major).
+    c->tree = sizeof(R) == 4 && c->scan && S == d && d >= kTreeMinD && (c->nF == 0 || c->alpha[3] == 0.0) &&
+              c->alpha[4] == 0.0;
+    if (c->tree) {
+        auto grid_of = [&](const std::vector<double>& psi) {   // 2^e bounds the propagated columns' norms
+            double mx = 0.0;
+            for (int s : c->cols) {
+                double n2 = 0.0;
+                for (int a = 0; a < d; ++a)
+                    for (int q = 0; q < 2; ++q) {
+                        const double v = psi[((size_t)a * c->S + s) * 2 + q];
+                        n2 += v * v;
+                    }
+                mx = std::max(mx, n2);
+            }
+            const double b = 1.0625 * std::sqrt(mx);
+            const int e = b > 0.0 ? std::max(-100, std::min(100, (int)std::ceil(std::log2(b)))) : -100;
+            return std::ldexp(1.5f, e + 11);
+        };
+        c->tree_mo[0] = grid_of(c->psi0);
+        c->tree_mo[1] = grid_of(c->psiT);
+        cbw = S;
+    }
     c->cb = std::min(cbw, S);
     c->ncb = (S + c->cb - 1) / c->cb;
     c->Spad = c->ncb * c->cb;
@@ -350,7 +379,8 @@ void plan_impl(qoc_ctx* c) {
         if (c->path_kind == 1) per += big_scratch_per_item(d, sizeof(R) == 8, c->ps);
         if (use_tc(c)) per += tc_scratch_floats(d, 1) * sizeof(float);
         if (use_oz(c)) per += std::max(oz_scratch_bytes(d, 1), oz_fwd_on(c) ? oz_fwd_scratch_bytes(d, 1) : 0);
-        if (c->scan) per += dd0 * ks + (2 * (size_t)c->ustride * ks + seg - 1) / seg;
+        if (c->tree) per += 2 * dd0 * ks + slice * ks;                        // nodes (two sets), carried blocks
+        else if (c->scan) per += dd0 * ks + (2 * (size_t)c->ustride * ks + seg - 1) / seg;
         if (c->path_kind == 0 && c->opt.gradient == QOC_GRAD_EXACT && c->opt.adjoint == QOC_ADJ_AUTO)
             per += 2 * (size_t)kZCap * ((dd0 + 31) / 32 * 32) * cs;
         per *= (size_t)E;
@@ -525,7 +555,18 @@ void plan_impl(qoc_ctx* c) {
     } else {
         c->Zbuf.release();
     }
-    if (c->scan) {
+    if (c->tree) {
+        A(c->tnodes, 2 * (size_t)E * tree_nodes(W) * dd * sizeof(float4), "alloc tree nodes");
+        A(c->tcarry, (size_t)E * (W + 1) * slice * sizeof(float4), "alloc tree blocks");
+        A(c->tcoef, (size_t)E * S * sizeof(float4), "alloc tree coefficients");
+        A(c->tgtK, slice * sizeof(K_t<R>), "alloc carried target");
+        check_cuda(c, cudaStreamSynchronize(st), "sync");
+        check_cuda(c, cudaMemcpyAsync(stage.p, psiTp.data(), blk, cudaMemcpyHostToDevice, st), "copy target");
+        check_cuda(c, launch_to_carry<R>(stage.as<double2>(), c->tgtK.as<K_t<R>>(), d, S, sv, 1, slice, st), "carried target");
+    } else {
+        for (DevBuf* b : {&c->tnodes, &c->tcarry, &c->tcoef, &c->tgtK}) b->release();
+    }
+    if (c->scan && !c->tree) {
         const size_t nz = (size_t)c->nzmax, ks = sizeof(K_t<R>);
         const size_t half = (size_t)((seg + 1) / 2);
         A(c->Pbuf, 2 * (size_t)E * nz * c->ustride * ks, "alloc segment products");
@@ -798,6 +839,76 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
         a.prm = prm;
         return a;
     };
+    if constexpr (sizeof(R) == 4) if (c->tree) {
+        // ---- the tree's passes and the per-slice costs on sx, the exponentials and adjoints on st ----
+        auto targs = [&](int w) {
+            return TreeArgs{d, E, sv.S, std::min(W, N - w * W), W, Ub(w), c->ustride,
+                            c->tnodes.as<float4>() + (size_t)(w & 1) * E * tree_nodes(W) * dd, c->tcarry.as<float4>(),
+                            slice, prm};
+        };
+        const size_t ck_e = (size_t)c->nseg_total * slice;
+        auto ck = [&](int w) { return c->ckpt.as<K>() + (size_t)(w * W / seg) * slice; };   // first block of wave w
+        auto forward = [&](int w, bool hand_on) {
+            int n_l = 0;
+            B(sx);
+            cudaError_t e = launch_tree_up(targs(w), sx, &n_l);
+            L(e, "seg_products", sx);
+            extra += n_l - 1;
+            n_l = 0;
+            B(sx);
+            const bool next = hand_on && w + 1 < nw;
+            e = launch_tree_forward(targs(w), ck(w), ck_e, next ? ck(w + 1) : nullptr, ck_e, Sb(w), (size_t)(W + 1) * slice,
+                                    c->tree_mo[0], sx, &n_l);
+            L(e, "chain (replay)", sx);
+            extra += n_l - 1;
+        };
+        for (int w = 0; w < nw; ++w) {
+            const int j0 = w * W, wlen = std::min(W, N - j0);
+            if (w >= 2) wait(st, ev_fwd[w - 2]);           // set w % 2 released by wave w - 2
+            B(st);
+            L(expm_fwd(w), "expm_fwd", st);
+            rec(ev_exp[w], st);
+            wait(sx, ev_exp[w]);
+            forward(w, true);
+            B(sx);
+            L(launch_slice_costs<R>(d, sv, j0, wlen, N, E, Sb(w), W, cv, c->Oj.as<double2>(), c->C5j.as<double>(),
+                                    c->Ofin.as<double2>(), sx),
+              "slice_costs", sx);
+            rec(ev_fwd[w], sx);
+        }
+        B(sx);
+        L(launch_tree_coef(cv, E, sv.S, c->Ofin.as<double2>(), c->tcoef.as<float4>(), sx), "sources", sx);
+        for (int w = nw - 1; w >= 0; --w) {
+            if (w < nw - 2) {                              // recomputed: the states too
+                wait(sx, ev_rep[w]);
+                forward(w, false);
+            }
+            int n_l = 0;
+            B(sx);
+            const cudaError_t e = launch_tree_costate(targs(w), w == nw - 1 ? c->tgtK.as<float4>() : c->carry.as<float4>(),
+                                                      w == nw - 1 ? 0 : slice, w > 0 ? c->carry.as<float4>() : nullptr, slice,
+                                                      Gb(w), (size_t)W * slice, c->tcoef.as<float4>(), c->tree_mo[1], sx, &n_l);
+            L(e, "costate (final)", sx);
+            extra += n_l - 1;
+            rec(ev_cost[w], sx);
+            if (w >= 1 && w - 1 < nw - 2) {                // set (w - 1) % 2: wave w + 1's, whose adjoint is on st
+                B(st);
+                L(expm_fwd(w - 1), "expm_fwd (recompute)", st);
+                rec(ev_rep[w - 1], st);
+            }
+            wait(st, ev_cost[w]);
+            B(st);
+            L(expm_adj(w), "expm_adj", st);
+        }
+        rec(ev_join, sx);
+        wait(st, ev_join);
+        B(st);
+        L(launch_finalize(E, M, N, u, c->alpha, c->Oj.as<double2>(), c->C5j.as<double>(), c->Ofin.as<double2>(),
+                          c->gpart.as<double>(), grad, out, prm, st),
+          "finalize", st);
+        c->launches = launches + extra;
+        return;
+    }
     if (!c->scan) {
         // ---- forward: exponentials on st, propagation and per-slice costs on sx ----
         for (int w = 0; w < nw; ++w) {

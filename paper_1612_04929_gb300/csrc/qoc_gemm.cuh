@@ -76,7 +76,8 @@ struct GemmPos {
 // `mac.run(a, b, xw)` for every k, with the MT operands of each side.  la(row, k, dst) and lb(k, column,
 // dst) bring one element of an operand into shared memory (zero past its edge).  The caller has passed
 // a barrier since the ring was last read; ends with a barrier.
-template <typename E, class Sh, typename LA, typename LB, typename Mac>
+// AT: A's elements are brought row-fastest (the caller reads A transposed).
+template <typename E, class Sh, bool AT = false, typename LA, typename LB, typename Mac>
 __device__ __forceinline__ void gemm_loop(unsigned char* smraw, const GemmPos<Sh>& p, int kd, LA la, LB lb, Mac& mac) {
     constexpr int MT = Sh::MT, G = Sh::G, T = Sh::T, ST = Sh::ST, NT = Sh::NT;
     constexpr int asz = T * (kGemmK + 1), bsz = kGemmK * (T + 1), per = T * kGemmK / NT;
@@ -89,8 +90,13 @@ __device__ __forceinline__ void gemm_loop(unsigned char* smraw, const GemmPos<Sh
         const int k = threadIdx.x % kGemmK;
 #pragma unroll
         for (int q = 0; q < per; ++q) {
-            const int r = threadIdx.x / kGemmK + q * (NT / kGemmK);
-            la(p.r0 + r, k0 + k, as + r * (kGemmK + 1) + k);
+            if constexpr (AT) {
+                const int idx = threadIdx.x + q * NT, kt = idx / T, r = idx - kt * T;
+                la(p.r0 + r, k0 + kt, as + r * (kGemmK + 1) + kt);
+            } else {
+                const int r = threadIdx.x / kGemmK + q * (NT / kGemmK);
+                la(p.r0 + r, k0 + k, as + r * (kGemmK + 1) + k);
+            }
         }
 #pragma unroll
         for (int q = 0; q < per; ++q) {

@@ -462,6 +462,30 @@ bool state_grad_lr_applies(const SysView<float>& sys, int d, int S, int p, int n
 cudaError_t launch_state_grad_lr(const StateGradArgs<float>& a, const SysView<float>& sys, int p, int n, cudaStream_t st);
 template <typename R> cudaError_t launch_state_grad(const StateGradArgs<R>& a, int p, int n, cudaStream_t st);
 
+// ---- full-unitary recursions over a binary tree of the wave (k_tree.cu, FP32 forms) ----
+// Blocks are d x S row-major (one panel of width S), slice elements apart.
+struct TreeArgs {
+    int d, E, S, wlen, W;   // slices of this wave; the most a wave has (strides)
+    const float2* U;        // propagators of the wave: U_j at U + (e W + j) ustride, U_j^dag at + ustride / 2
+    long long ustride;
+    float4* nodes;          // tree_nodes(W) d x d matrices per member, grid-split
+    float4* carry;          // W + 1 blocks per member: the pass's states or costates, grid-split
+    size_t slice;
+    const DevParams* prm;
+};
+constexpr int kTreeMinD = 48;
+int tree_levels(int wlen);
+size_t tree_nodes(int W);   // per member
+cudaError_t launch_tree_up(const TreeArgs& a, cudaStream_t st, int* launches);
+// states Psi_0 .. Psi_wlen of the wave (rounded) from its first block (pairs); the last one also to next
+cudaError_t launch_tree_forward(const TreeArgs& a, const float4* start, size_t start_e, float4* next, size_t next_e,
+                                float2* states, size_t states_e, float mo, cudaStream_t st, int* launches);
+cudaError_t launch_tree_coef(const CostView<float>& cv, int E, int S, const double2* Ofin, float4* coef, cudaStream_t st);
+// costates G_1 .. G_wlen (block j - 1 of G), coef times the block propagated from start; the block below
+// the wave's first slice to next (or nullptr)
+cudaError_t launch_tree_costate(const TreeArgs& a, const float4* start, size_t start_e, float4* next, size_t next_e,
+                                float2* G, size_t G_e, const float4* coef, float mo, cudaStream_t st, int* launches);
+
 // ---- per-slice costs, sources, final reduction (k_chain.cu) ----
 template <typename R>
 cudaError_t launch_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* states,
