@@ -39,14 +39,18 @@
 // warp 0 issues the TMA loads of a three-stage ring (one stage: the eight slice planes of A and
 // of B for a 16-wide K chunk, SWIZZLE_32B, 64 KB), warp 1 issues the tcgen05.mma (kind::f16,
 // BF16 in, FP32 accumulators in tensor memory: leading re, leading im, rest re, rest im, 128
-// columns each) and commits each stage back to the producer, warps 2-5 read tensor memory with
-// tcgen05.ld, stage the scaled tile in the idle ring and write it with coalesced stores.  Every mbarrier wait is bounded; a wait that runs out sets
+// columns each) and commits each stage back to the producer, warps 2-9 read tensor memory with
+// tcgen05.ld, stage the scaled tile in the idle ring and write it with coalesced stores; what the tile
+// is added to (the accumulated output, the Paterson-Stockmeyer block) they hold in registers by then,
+// read while the products ran.  With four epilogue warps that read it after the products, a tile spent
+// half its time outside the MMAs (d = 256: 61 us a forward tile, its MMAs about 31).  Every mbarrier wait is bounded; a wait that runs out sets
 // kErrTimeout in DevParams.err and the CTA stops issuing, waits (bounded) for its copies in
 // flight, frees its tensor memory and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "qoc_device.cuh"
 #include "qoc_internal.h"
@@ -57,7 +61,8 @@ namespace {
 
 constexpr int BM = 128, BK = 16;                   // BK in BF16 elements: 32-byte rows
 constexpr int SBITS = 7;
-constexpr int NTHREADS = 192;                      // producer warp, MMA warp, four epilogue warps
+constexpr int EPI_WARPS = 8;                       // two per tensor-memory lane quarter
+constexpr int NTHREADS = 64 + 32 * EPI_WARPS;      // producer warp, MMA warp, epilogue warps
 
 // One product configuration: NS slices per value, BN-wide tiles, NLEV accumulator levels (every
 // level below NLEV - 1 exact, the last one taking the remaining slice pairs), NST stages.
@@ -120,17 +125,27 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
                  : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
+// 16 columns of this lane's row; the values may be read after tmem_wait
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
         "[%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]),
+          "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
         : "r"(taddr));
+}
+// the loads before it have landed; their values pass through an empty asm after the wait, so no use of
+// them can move above it
+__device__ __forceinline__ void tmem_pass(float (&r)[16]) {
+    asm volatile("" : "+f"(r[0]), "+f"(r[1]), "+f"(r[2]), "+f"(r[3]), "+f"(r[4]), "+f"(r[5]), "+f"(r[6]), "+f"(r[7]),
+                 "+f"(r[8]), "+f"(r[9]), "+f"(r[10]), "+f"(r[11]), "+f"(r[12]), "+f"(r[13]), "+f"(r[14]), "+f"(r[15]));
+}
+__device__ __forceinline__ void tmem_wait(float (&a)[16], float (&b)[16], float (&c)[16], float (&d)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
+    tmem_pass(a);
+    tmem_pass(b);
+    tmem_pass(c);
+    tmem_pass(d);
 }
 
 // exponent e with |x| < 2^e for the largest |x| of a row or column (0 for an all-zero one)
@@ -434,6 +449,42 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
             s_ok = 0;
         }
     }
+    // Epilogue warp: 32 tile rows (the lane quarter of tensor memory it may read) and half the columns.
+    // While the products run it brings what its outputs are added to into registers, in the order it
+    // writes them (row rw, column lane + 32 j of its half): the accumulated output (beta), or the
+    // Paterson-Stockmeyer block c0 I + c1 X + c2 X^2 in pair arithmetic.
+    constexpr int HC = BN / 2, JC = HC / 32;           // columns per epilogue warp, per lane
+    const int q4 = warp & 3, ch0 = c0 + ((warp - 2) >> 2) * HC;
+    const int row0 = r0 + q4 * 32, nrows = min(32, d - row0), ncols = min(HC, d - ch0);
+    using Add = std::conditional_t<FWD, float4, float2>;
+    constexpr int PRE = FWD ? 20 : 22;                 // rows held (registers), the others are read when written
+    Add add[PRE][JC];
+    const bool has_add = FWD ? fe.kind == 2 : jb.beta != 0;
+    auto read_add = [&](int rw, int j) -> Add {
+        const int c = lane + 32 * j;
+        const bool in = rw < nrows && c < ncols;
+        if constexpr (FWD) {
+            const size_t o = (size_t)item * fe.ostride + (size_t)(row0 + rw) * d + ch0 + c;
+            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 xv = in ? fe.X[o] : z4, yv = in ? fe.X2[o] : z4;
+            float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+            pair_fma(rh, rl, fe.c1, xv.x, xv.z);
+            pair_fma(ih, il, fe.c1, xv.y, xv.w);
+            pair_fma(rh, rl, fe.c2, yv.x, yv.z);
+            pair_fma(ih, il, fe.c2, yv.y, yv.w);
+            if (row0 + rw == ch0 + c) df_addc(rh, rl, fe.c0);
+            return make_float4(rh, ih, rl, il);
+        } else {
+            const float2* out = jb.out + (size_t)item * jb.ostride;
+            return in ? out[(size_t)(row0 + rw) * d + ch0 + c] : make_float2(0.f, 0.f);
+        }
+    };
+    if (warp >= 2 && has_add) {
+#pragma unroll
+        for (int rw = 0; rw < PRE; ++rw)
+#pragma unroll
+            for (int j = 0; j < JC; ++j) add[rw][j] = read_add(rw, j);
+    }
     __syncthreads();
     const bool fin = mbar_wait(&done, 0, limit);
     if (!fin && tid == 0) atomicOr(&prm->err, kErrTimeout);
@@ -441,18 +492,14 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
     const bool go = __syncthreads_and(fin && s_ok != 0) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (go && warp >= 2) {
-        // Each epilogue warp owns 32 tile rows (the TMEM lane quarter it may read).  It scales
-        // its rows into a staging area of the idle stage ring (every copy has landed and every
-        // MMA has read its operands once `done` completed), then writes them row by row with
-        // the lanes along the columns, so the global stores (and the reads of beta) coalesce.
-        constexpr int SROW = BN + 1;                   // padded row: fewer bank conflicts
-        const int q4 = warp & 3;
-        const int r = r0 + q4 * 32 + lane;
-        const int ncols = min(BN, d - c0);
+        // Each epilogue warp scales its part of the tile into a staging area of the idle stage ring (every
+        // copy has landed and every MMA has read its operands once `done` completed), then writes it
+        // row by row with the lanes along the columns, so the global stores coalesce.
+        constexpr int SROW = HC + 1;                   // padded row: fewer bank conflicts
+        const int r = row0 + lane;
         const int eA = r < d ? exps[((size_t)item * kOzMats + jb.a_mat) * d + r] : 0;
         const int* eBp = exps + ((size_t)item * kOzMats + jb.b_mat) * d;
-        const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16);
-        const int nrows = min(32, d - (r0 + q4 * 32));
+        const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(ch0 - c0);
         if constexpr (!FWD) {
             float2* stg = reinterpret_cast<float2*>(base) + (size_t)(warp - 2) * 32 * SROW;
             for (int cc = 0; cc < ncols; cc += 16) {
@@ -461,45 +508,37 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                 tmem_ld16(lane_base + (uint32_t)(BN + cc), li);
                 tmem_ld16(lane_base + (uint32_t)(2 * BN + cc), rr);
                 tmem_ld16(lane_base + (uint32_t)(3 * BN + cc), ri);
+                tmem_wait(lr, li, rr, ri);
 #pragma unroll
                 for (int q = 0; q < 16; ++q) {
-                    const int c = c0 + cc + q;
+                    const int c = ch0 + cc + q;
                     const float sc = ldexpf(jb.alpha, eA + (c < d ? eBp[c] : 0) - 3 * SBITS);
                     stg[lane * SROW + cc + q] = make_float2((lr[q] + rr[q]) * sc, (li[q] + ri[q]) * sc);
                 }
             }
             __syncwarp();
-            // eight rows at a time, each lane four columns (c = lane + 32 j): the 32 reads of the
-            // accumulated output (beta) are in flight together
             float2* out = jb.out + (size_t)item * jb.ostride;
-            for (int rw0 = 0; rw0 < nrows; rw0 += 8) {
-                float2 old[8][BN / 32];
-                if (jb.beta) {
+            float2 rest[32 - PRE][JC];
+            if (has_add)
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
+                for (int rw = PRE; rw < 32; ++rw)
 #pragma unroll
-                        for (int j = 0; j < BN / 32; ++j) {
-                            const int rw = rw0 + u, c = lane + 32 * j;
-                            old[u][j] = (rw < nrows && c < ncols) ? out[(size_t)(r0 + q4 * 32 + rw) * d + c0 + c]
-                                                                  : make_float2(0.f, 0.f);
-                        }
-                }
+                    for (int j = 0; j < JC; ++j) rest[rw - PRE][j] = read_add(rw, j);
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
+            for (int rw = 0; rw < 32; ++rw)
 #pragma unroll
-                    for (int j = 0; j < BN / 32; ++j) {
-                        const int rw = rw0 + u, c = lane + 32 * j;
-                        if (rw >= nrows || c >= ncols) continue;
-                        const int row = r0 + q4 * 32 + rw;
-                        float2 v = stg[rw * SROW + c];
-                        if (jb.beta) {
-                            v.x += old[u][j].x;
-                            v.y += old[u][j].y;
-                        }
-                        if (jb.ident && row == c0 + c) v.x += 1.0f;
-                        out[(size_t)row * d + c0 + c] = v;
+                for (int j = 0; j < JC; ++j) {
+                    const int c = lane + 32 * j;
+                    if (rw >= nrows || c >= ncols) continue;
+                    float2 v = stg[rw * SROW + c];
+                    if (has_add) {
+                        const float2 q = rw < PRE ? add[rw < PRE ? rw : 0][j] : rest[rw < PRE ? 0 : rw - PRE][j];
+                        v.x += q.x;
+                        v.y += q.y;
                     }
-            }
+                    if (jb.ident && row0 + rw == ch0 + c) v.x += 1.0f;
+                    out[(size_t)(row0 + rw) * d + ch0 + c] = v;
+                }
         } else {
             // value pairs (re_hi, im_hi, re_lo, im_lo): the three exact levels summed without
             // error, the remainder level added to the low part; every scaling is by a power of two
@@ -513,9 +552,10 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                     tmem_ld16(lane_base + (uint32_t)((2 + part) * BN + cc), a1);
                     tmem_ld16(lane_base + (uint32_t)((4 + part) * BN + cc), a2);
                     tmem_ld16(lane_base + (uint32_t)((6 + part) * BN + cc), a3);
+                    tmem_wait(a0, a1, a2, a3);
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
-                        const int c = c0 + cc + q;
+                        const int c = ch0 + cc + q;
                         const float sc = ldexpf(1.0f, eA + (c < d ? eBp[c] : 0) - 3 * SBITS);
                         float h, l, h2, l2;
                         two_sum(a0[q] * sc, a1[q] * sc, h, l);
@@ -534,45 +574,31 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                 }
             }
             __syncwarp();
-            // four rows at a time, each lane BN / 32 columns; the block terms' reads in flight together
             float4* out = fe.out + (size_t)item * fe.ostride;
-            const size_t ioff = (size_t)item * fe.ostride;
-            for (int rw0 = 0; rw0 < nrows; rw0 += 4) {
-                float4 xv[4][BN / 32], yv[4][BN / 32];
-                if (fe.kind == 2) {
+            float4 rest[32 - PRE][JC];
+            if (has_add)
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
+                for (int rw = PRE; rw < 32; ++rw)
 #pragma unroll
-                        for (int j = 0; j < BN / 32; ++j) {
-                            const int rw = rw0 + u, c = lane + 32 * j;
-                            const bool in = rw < nrows && c < ncols;
-                            const size_t o = ioff + (size_t)(r0 + q4 * 32 + rw) * d + c0 + c;
-                            xv[u][j] = in ? fe.X[o] : make_float4(0.f, 0.f, 0.f, 0.f);
-                            yv[u][j] = in ? fe.X2[o] : make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-                }
+                    for (int j = 0; j < JC; ++j) rest[rw - PRE][j] = read_add(rw, j);
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
+            for (int rw = 0; rw < 32; ++rw)
 #pragma unroll
-                    for (int j = 0; j < BN / 32; ++j) {
-                        const int rw = rw0 + u, c = lane + 32 * j;
-                        if (rw >= nrows || c >= ncols) continue;
-                        const int row = r0 + q4 * 32 + rw;
-                        const float4 v = stg[rw * SROW + c];
-                        float rh = v.x, rl = v.z, ih = v.y, il = v.w;
-                        if (fe.kind == 2) {
-                            pair_fma(rh, rl, fe.c1, xv[u][j].x, xv[u][j].z);
-                            pair_fma(ih, il, fe.c1, xv[u][j].y, xv[u][j].w);
-                            pair_fma(rh, rl, fe.c2, yv[u][j].x, yv[u][j].z);
-                            pair_fma(ih, il, fe.c2, yv[u][j].y, yv[u][j].w);
-                            if (row == c0 + c) df_addc(rh, rl, fe.c0);
-                        }
-                        float4 o;
-                        grid_split(rh, rl, fe.magic, o.x, o.z);
-                        grid_split(ih, il, fe.magic, o.y, o.w);
-                        out[(size_t)row * d + c0 + c] = o;
+                for (int j = 0; j < JC; ++j) {
+                    const int c = lane + 32 * j;
+                    if (rw >= nrows || c >= ncols) continue;
+                    const float4 v = stg[rw * SROW + c];
+                    float rh = v.x, rl = v.z, ih = v.y, il = v.w;
+                    if (has_add) {
+                        const float4 q = rw < PRE ? add[rw < PRE ? rw : 0][j] : rest[rw < PRE ? 0 : rw - PRE][j];
+                        df_addc(rh, rl, make_float2(q.x, q.z));
+                        df_addc(ih, il, make_float2(q.y, q.w));
                     }
-            }
+                    float4 o;
+                    grid_split(rh, rl, fe.magic, o.x, o.z);
+                    grid_split(ih, il, fe.magic, o.y, o.w);
+                    out[(size_t)(row0 + rw) * d + ch0 + c] = o;
+                }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
