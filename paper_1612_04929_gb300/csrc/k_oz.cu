@@ -35,15 +35,13 @@
 // accumulators within the tensor memory, and the epilogue adds the Paterson-Stockmeyer block in
 // pair arithmetic and writes grid-split value pairs.
 //
-// k_oz_mm computes one 128 x 128 tile of C = alpha A B (+ C) (+ I) for one job and one wave item:
+// k_oz_mm computes 128 x 128 tiles of C = alpha A B (+ C) (+ I), a persistent CTA per SM:
 // warp 0 issues the TMA loads of a three-stage ring (one stage: the eight slice planes of A and
-// of B for a 16-wide K chunk, SWIZZLE_32B, 64 KB), warp 1 issues the tcgen05.mma (kind::f16,
+// of B for a 16-wide K chunk, four to a SWIZZLE_128B tile, 64 KB), warp 1 issues the tcgen05.mma (kind::f16,
 // BF16 in, FP32 accumulators in tensor memory: leading re, leading im, rest re, rest im, 128
 // columns each) and commits each stage back to the producer, warps 2-9 read tensor memory with
-// tcgen05.ld, stage the scaled tile in the idle ring and write it with coalesced stores; what the tile
-// is added to (the accumulated output, the Paterson-Stockmeyer block) they hold in registers by then,
-// read while the products ran.  With four epilogue warps that read it after the products, a tile spent
-// half its time outside the MMAs (d = 256: 61 us a forward tile, its MMAs about 31).  Every mbarrier wait is bounded; a wait that runs out sets
+// tcgen05.ld into registers, hand it back to the MMA warp and then add and write the tile while the next
+// one's products run.  Every mbarrier wait is bounded; a wait that runs out sets
 // kErrTimeout in DevParams.err and the CTA stops issuing, waits (bounded) for its copies in
 // flight, frees its tensor memory and returns.
 #include <cuda.h>
@@ -59,7 +57,8 @@ namespace qoc {
 
 namespace {
 
-constexpr int BM = 128, BK = 16;                   // BK in BF16 elements: 32-byte rows
+constexpr int BM = 128, BK = 16;                   // BK in BF16 elements
+constexpr int GRP = 4;                             // planes side by side in a 128-byte row (per K chunk)
 constexpr int SBITS = 7;
 constexpr int EPI_WARPS = 8;                       // two per tensor-memory lane quarter
 constexpr int NTHREADS = 64 + 32 * EPI_WARPS;      // producer warp, MMA warp, epilogue warps
@@ -70,9 +69,11 @@ template <int NS_, int BN_, int NLEV_, int NST_>
 struct OzCfg {
     static constexpr int NS = NS_, BN = BN_, NLEV = NLEV_, NST = NST_;
     static constexpr int NPART = 2 * NS;                      // re slices, then im slices
-    static constexpr int TILE_A = BM * BK * 2;                // one A plane tile, 4 KB
-    static constexpr int TILE_B = BN * BK * 2;                // one B plane tile
-    static constexpr int STAGE = NPART * (TILE_A + TILE_B);
+    static constexpr int NG = NPART / GRP;                    // groups of planes
+    static constexpr int TILE_A = BM * BK * 2 * GRP;          // one group's A tile, 16 KB
+    static constexpr int TILE_B = BN * BK * 2 * GRP;          // one group's B tile
+    static constexpr int STAGE = NG * (TILE_A + TILE_B);
+    static_assert(NPART % GRP == 0, "whole groups");
     static constexpr int SMEM = NST * STAGE + 1024;           // + alignment slack
     static constexpr uint32_t TMEM_COLS = 512;
 };
@@ -109,18 +110,37 @@ __device__ __forceinline__ void tma_3d(void* smem, const CUtensorMap* map, int x
         "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(su32(bar))
         : "memory");
 }
-// UMMA shared-memory descriptor: K-major, SWIZZLE_32B (one 32-byte row per M / N index, 8-row
-// groups 256 bytes apart), descriptor version 1
-__device__ __forceinline__ uint64_t sdesc(const void* smem) {
-    const uint64_t a = su32(smem);
-    return ((a >> 4) & 0x3FFFull) | (1ull << 16) | ((uint64_t)(256 >> 4) << 32) | (1ull << 46) | (6ull << 61);
+// UMMA shared-memory descriptor: K-major, SWIZZLE_128B (one 128-byte row per M / N index holding the
+// K chunk of four planes, 8-row groups 1024 bytes apart), descriptor version 1.  lo: sdesc_lo of the
+// group's tile (1024-byte aligned) plus 2 per plane (its 32 bytes), in units of 16 bytes.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t smem) { return ((smem >> 4) & 0x3FFFu) | (1u << 16); }
+__device__ __forceinline__ uint64_t sdesc(uint32_t lo) {
+    return ((uint64_t)((1024u >> 4) | (1u << 14) | (2u << 29)) << 32) | lo;
 }
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
+// one lane of a converged warp: the MMA operands are in uniform registers, which the compiler finds by
+// itself only where the choice of the lane is this instruction and all around it is uniform.  (Under
+// `lane == 0` an MMA took 72 cycles to issue whatever its size: 1200 us a forward product of 450 items
+// at d = 256, 939 with the choice alone by elect.)
+__device__ __forceinline__ bool elect() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
 }
+// One MMA of a run that shares its A operand (and its descriptor): the first of the run fills the A
+// collector from shared memory, the others read A from it
+enum { A_FILL, A_USE, A_LAST, A_NONE };
+#define QOC_MMA(OP)                                                                                                   \
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"                                                        \
+                 " tcgen05.mma.cta_group::1.kind::f16.collector::a::" OP " [%0], %1, %2, %3, p;\n}" ::"r"(tmem),       \
+                 "l"(a), "l"(b), "r"(idesc), "r"(acc)                                                                 \
+                 : "memory")
+__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc, int use) {
+    if (use == A_FILL) QOC_MMA("fill");
+    else if (use == A_USE) QOC_MMA("use");
+    else if (use == A_LAST) QOC_MMA("lastuse");
+    else QOC_MMA("discard");
+}
+#undef QOC_MMA
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
                  : "memory");
@@ -183,19 +203,24 @@ __device__ __forceinline__ float4 as_pairs(float4 v) { return make_float4(v.x, v
 
 }  // namespace
 
-// plane (item, matrix, part) in a plane array of NPART planes per matrix
+// Planes are stored in groups of four: a row of a group holds, for each 16-wide K chunk, the chunk of the
+// group's four planes side by side (128 bytes), so one SWIZZLE_128B tile brings four planes of a chunk.
+// (With a plane per tile and 32-byte rows a forward product of 150 items at d = 256 took 477 us instead of
+// 458 and an adjoint one 269 instead of 250; the slicer pays 5 % for it.)  Group (item, matrix, g):
 template <int NPART>
-__host__ __device__ inline size_t oz_plane(int item, int mat, int part) {
-    return ((size_t)item * kOzMats + mat) * NPART + part;
+__host__ __device__ inline size_t oz_group(int item, int mat, int g) {
+    return ((size_t)item * kOzMats + mat) * (NPART / GRP) + g;
 }
+__host__ __device__ inline int oz_row(int d) { return (d + BK - 1) / BK * BK * GRP; }   // elements of a group's row
+// element k of plane `part` within a row of its group
+__device__ __forceinline__ size_t oz_at(int part, int k) { return (size_t)(k / BK) * (BK * GRP) + (part % GRP) * BK + k % BK; }
 
 // ------------------------------------------------------------------------------------------
 // slicing: FP32 complex d x d matrices (row-major, item-strided) -> exponents and BF16 planes
 // ------------------------------------------------------------------------------------------
 // Row layout (A operand): plane row r = row r of M, exponent per row.  Column layout (B operand,
 // K-major): plane row c = column c of M, exponent per column (no conjugation is applied).
-// Eight consecutive elements of one plane row, as one 16-byte store (the plane rows are padded to
-// a multiple of eight elements and start on 16-byte boundaries)
+// Eight consecutive elements of one plane row (half a K chunk), as one 16-byte store
 __device__ __forceinline__ void store8(__nv_bfloat16* dst, const float (&v)[8]) {
     uint4 w;
     __nv_bfloat162 h;
@@ -210,11 +235,11 @@ __device__ __forceinline__ void store8(__nv_bfloat16* dst, const float (&v)[8]) 
     *reinterpret_cast<uint4*>(dst) = w;
 }
 
-// the slices of eight consecutive elements of one plane row (k0 .. k0 + 7; zero past d), written
-// as 16-byte stores into the row's 2 NS planes
+// the slices of eight consecutive elements k0 .. k0 + 7 of plane row `row` (zero past d), written as
+// 16-byte stores into the row's 2 NS planes; gsz: elements of a group (d rows)
 template <int NS>
-__device__ __forceinline__ void put8(__nv_bfloat16* __restrict__ planes, size_t pbase, size_t psz, size_t rowoff,
-                                     const float4 (&q)[8], int e, bool role_a) {
+__device__ __forceinline__ void put8(__nv_bfloat16* __restrict__ planes, size_t pbase, size_t gsz, int row, int rowlen,
+                                     int k0, const float4 (&q)[8], int e, bool role_a) {
     float sr[8][NS], si[8][NS];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -229,14 +254,15 @@ __device__ __forceinline__ void put8(__nv_bfloat16* __restrict__ planes, size_t 
             vr[i] = sr[i][s];
             vi[i] = si[i][s];
         }
-        store8(planes + (pbase + s) * psz + rowoff, vr);
-        store8(planes + (pbase + NS + s) * psz + rowoff, vi);
+        __nv_bfloat16* pr = planes + (size_t)row * rowlen;
+        store8(pr + (pbase + s / GRP) * gsz + oz_at(s, k0), vr);
+        store8(pr + (pbase + (NS + s) / GRP) * gsz + oz_at(NS + s, k0), vi);
     }
 }
 
 template <int NS, typename In>
 __global__ void __launch_bounds__(256)
-k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict__ exps, int d, int ldp) {
+k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict__ exps, int d) {
     constexpr int NPART = 2 * NS;
     constexpr int KT = 64;                       // rows of M per staged tile (column layout)
     __shared__ float4 tile[KT][33];
@@ -245,8 +271,9 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
     const OzSliceJob jb = jobs.job[blockIdx.z];
     const int item = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const In* M = static_cast<const In*>(jb.src) + (size_t)item * jb.stride;
-    const size_t psz = (size_t)d * ldp;
-    const size_t pbase = oz_plane<NPART>(item, jb.mat, 0);
+    const int rowlen = oz_row(d), dk = rowlen / GRP;   // dk: d rounded up to whole K chunks
+    const size_t gsz = (size_t)d * rowlen;
+    const size_t pbase = oz_group<NPART>(item, jb.mat, 0);
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     // the exponent comes from the rounded values |re|, |im| (a pair's sum rounded up to 2^e only
     // raises e: conservative)
@@ -272,7 +299,7 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
 #pragma unroll
         for (int ch = 0; ch < 2; ++ch) {
             const int b0 = ch * 256 + lane * 8;
-            if (b0 < d) put8<NS>(planes, pbase, psz, (size_t)r * ldp + b0, v[ch], e, true);
+            if (b0 < dk) put8<NS>(planes, pbase, gsz, r, rowlen, b0, v[ch], e, true);
         }
         return;
     }
@@ -303,11 +330,11 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
         }
         __syncthreads();
         const int cc = c0 + tc, kk = k0 + tk;
-        if (cc < d && kk < d) {
+        if (cc < d && kk < dk) {
             float4 q8[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) q8[i] = tile[tk + i][tc];
-            put8<NS>(planes, pbase, psz, (size_t)cc * ldp + kk, q8, cexp[tc], false);
+            put8<NS>(planes, pbase, gsz, cc, rowlen, kk, q8, cexp[tc], false);
         }
         __syncthreads();
     }
@@ -326,34 +353,36 @@ struct OzFwdEpi {
 };
 
 // ------------------------------------------------------------------------------------------
-// one 128 x BN output tile for job blockIdx.z, item blockIdx.y: adjoint products (FWD false)
-// C = alpha A B (+ beta C) (+ I) in FP32; forward products (FWD true) as value pairs (OzFwdEpi)
+// 128 x BN output tiles of the jobs' items: adjoint products (FWD false) C = alpha A B (+ beta C) (+ I)
+// in FP32; forward products (FWD true) as value pairs (OzFwdEpi).  A persistent CTA per SM takes tiles
+// blockIdx.x, + gridDim.x, ..: while the epilogue warps add and write one tile, the products of the next
+// run, and only the read-out of tensor memory stands between the products of two tiles.
+// A forward product at d = 256 (450 items, us): 1375 with a CTA per tile; 1204 persistent; 929 with the
+// MMAs' operands in uniform registers (elect); 742 with A read once per run by the collector, 60 % of the
+// tensor rate at 1.9 GHz.  What is left: the copies alone (4.2 GB of plane tiles through L2 a launch, 2.8 GB of HBM traffic) take 599,
+// the MMAs 530.  An adjoint product (mean of single and double launches): 750, 622, 608, 583, the copies
+// alone 490.
 // ------------------------------------------------------------------------------------------
 template <class Cfg, bool FWD>
 __global__ void __launch_bounds__(NTHREADS, 1)
-k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, OzJobs jobs,
-        OzFwdEpi fe, const int* __restrict__ exps, int d, DevParams* __restrict__ prm) {
+k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, OzJobs jobs, int njobs,
+        int items, OzFwdEpi fe, const int* __restrict__ exps, int d, DevParams* __restrict__ prm) {
     constexpr int NS = Cfg::NS, BN = Cfg::BN, NLEV = Cfg::NLEV, NST = Cfg::NST, NPART = Cfg::NPART;
-    constexpr int TILE_A = Cfg::TILE_A, TILE_B = Cfg::TILE_B, STAGE = Cfg::STAGE;
+    constexpr int TILE_A = Cfg::TILE_A, TILE_B = Cfg::TILE_B, STAGE = Cfg::STAGE, NG = Cfg::NG;
     extern __shared__ __align__(1024) unsigned char smraw[];
     unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full[NST], empty[NST], done;
+    __shared__ __align__(8) uint64_t full[NST], empty[NST], acc_full, acc_empty;
     __shared__ uint32_t tmem_holder;
-    __shared__ int skip, s_ok;
+    __shared__ int skip;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // once a wait has run out in this evaluation, later launches skip their work (the result is
     // reported as QOC_ERR_TIMEOUT); thread 0 decides for the whole CTA
-    if (tid == 0) {
-        skip = (*(volatile int*)&prm->err & kErrTimeout) != 0;
-        s_ok = 1;
-    }
+    if (tid == 0) skip = (*(volatile int*)&prm->err & kErrTimeout) != 0;
     __syncthreads();
     if (skip) return;
     const uint32_t limit = jobs.fault ? WAIT_LIMIT_TEST : WAIT_LIMIT;
-    const int item = blockIdx.y;
-    const OzJob jb = jobs.j[blockIdx.z];
-    const int ntn = (d + BN - 1) / BN;
-    const int r0 = (blockIdx.x / ntn) * BM, c0 = (blockIdx.x % ntn) * BN;
+    const int ntn = (d + BN - 1) / BN, per_item = ((d + BM - 1) / BM) * ntn;
+    const int per_job = per_item * items, total = per_job * njobs;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_holder)),
                      "r"(Cfg::TMEM_COLS)
@@ -365,7 +394,8 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
             mbar_init(&full[b], 1);
             mbar_init(&empty[b], 1);
         }
-        mbar_init(&done, 1);
+        mbar_init(&acc_full, 1);
+        mbar_init(&acc_empty, EPI_WARPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -373,232 +403,227 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_holder;
     const int nk = (d + BK - 1) / BK;
+    auto job_of = [&](int t) { return jobs.j[t / per_job]; };
 
     if (warp == 0 && lane == 0) {
-        // ---- producer: the NPART A planes and NPART B planes of one K chunk per stage ----
+        // ---- producer: the plane groups of A and of B for one K chunk per stage ----
         bool ok = true;
         int last_issued[NST];
 #pragma unroll
         for (int b = 0; b < NST; ++b) last_issued[b] = -1;
-        for (int s = 0; s < nk; ++s) {
-            const int b = s % NST;
-            if (s >= NST && !mbar_wait(&empty[b], (uint32_t)((s / NST - 1) & 1), limit)) {
-                ok = false;
-                break;
+        int g = 0;   // stages so far, over all tiles
+        for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+            const OzJob jb = job_of(t);
+            const int rest = t % per_job, item = rest / per_item, tile = rest - item * per_item;
+            const int r0 = (tile / ntn) * BM, c0 = (tile % ntn) * BN;
+            for (int s = 0; s < nk; ++s, ++g) {
+                const int b = g % NST;
+                if (g >= NST && !mbar_wait(&empty[b], (uint32_t)((g / NST - 1) & 1), limit)) {
+                    ok = false;
+                    break;
+                }
+                if (jobs.fault && g == 0) continue;   // fault injection: the first copy is withheld
+                unsigned char* st = base + b * STAGE;
+                mbar_expect_tx(&full[b], STAGE);
+                for (int q = 0; q < NG; ++q) {
+                    tma_3d(st + q * TILE_A, &mapA, s * BK * GRP, r0, (int)oz_group<NPART>(item, jb.a_mat, q), &full[b]);
+                    tma_3d(st + NG * TILE_A + q * TILE_B, &mapB, s * BK * GRP, c0,
+                           (int)oz_group<NPART>(item, jb.b_mat, q), &full[b]);
+                }
+                last_issued[b] = g;
             }
-            if (jobs.fault && s == 0) continue;   // fault injection: the first copy is withheld
-            unsigned char* st = base + b * STAGE;
-            mbar_expect_tx(&full[b], STAGE);
-            for (int part = 0; part < NPART; ++part) {
-                tma_3d(st + part * TILE_A, &mapA, s * BK, r0, (int)oz_plane<NPART>(item, jb.a_mat, part), &full[b]);
-                tma_3d(st + NPART * TILE_A + part * TILE_B, &mapB, s * BK, c0,
-                       (int)oz_plane<NPART>(item, jb.b_mat, part), &full[b]);
-            }
-            last_issued[b] = s;
         }
-        if (!ok) {
-            atomicOr(&prm->err, kErrTimeout);
-            s_ok = 0;
-        }
+        if (!ok) atomicOr(&prm->err, kErrTimeout);
         // every copy issued into this CTA's shared memory lands before the CTA can leave (bounded)
         for (int b = 0; b < NST; ++b)
             if (last_issued[b] >= 0) mbar_wait(&full[b], (uint32_t)((last_issued[b] / NST) & 1), limit);
-    } else if (warp == 1 && lane == 0) {
-        // ---- MMA issuer ----
+    } else if (warp == 1) {
+        // ---- MMA issuer: the whole warp goes through the waits, one lane issues ----
         // instruction descriptor: D f32, A/B bf16, both K-major, N = BN, M = 128
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
         const uint32_t idesc_nA = idesc | (1u << 13);   // negate A
+        const uint32_t acc0 = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t lo0 = sdesc_lo((su32(smraw) + 1023) & ~1023u);
         bool ok = true;
-        for (int s = 0; s < nk; ++s) {
-            const int b = s % NST;
-            if (!mbar_wait(&full[b], (uint32_t)((s / NST) & 1), limit)) {
-                ok = false;
+        int b = 0, n = 0;        // stage, tiles so far
+        uint32_t par = 0;        // the stage's phase
+        for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++n) {
+            if (n > 0) ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty, (uint32_t)((n - 1) & 1), limit));   // read out
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int s = 0; s < nk && ok; ++s) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&full[b], par, limit));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (elect()) {
+                    const uint32_t lo = lo0 + (uint32_t)b * (STAGE >> 4);
+                    // plane p: group p / 4, 32 bytes per plane within its rows
+                    auto dA = [&](int p) { return sdesc(lo + (uint32_t)((p / GRP) * TILE_A + (p % GRP) * (BK * 2)) / 16); };
+                    auto dB = [&](int p) {
+                        return sdesc(lo + (uint32_t)(NG * TILE_A + (p / GRP) * TILE_B + (p % GRP) * (BK * 2)) / 16);
+                    };
+#pragma unroll
+                    for (int sa = 0; sa < NS; ++sa) {
+                        // slice level sa + sb goes to its own accumulators below NLEV - 1, the rest to the last
+                        const int nb = NS - sa;
+                        auto acc = [&](int sb) { return acc0 + (uint32_t)(2 * min(sa + sb, NLEV - 1) * BN); };
+                        // re += Ar Br, im += Ar Bi: one run of A operand Ar.  The first MMA into each accumulator
+                        // (sa = 0, sb = its level) overwrites it
+#pragma unroll
+                        for (int sb = 0; sb < nb; ++sb) {
+                            const uint32_t en = (s > 0 || sa > 0 || sb > NLEV - 1) ? 1u : 0u;
+                            mma_bf16(acc(sb), dA(sa), dB(sb), idesc, en, sb == 0 ? A_FILL : A_USE);
+                            mma_bf16(acc(sb) + BN, dA(sa), dB(NS + sb), idesc, en, sb == nb - 1 ? A_LAST : A_USE);
+                        }
+                        // re -= Ai Bi, then im += Ai Br: the negation goes with A, so a run each
+#pragma unroll
+                        for (int neg = 1; neg >= 0; --neg)
+#pragma unroll
+                            for (int sb = 0; sb < nb; ++sb) {
+                                const int use = nb == 1 ? A_NONE : sb == 0 ? A_FILL : sb == nb - 1 ? A_LAST : A_USE;
+                                mma_bf16(acc(sb) + (neg ? 0 : BN), dA(NS + sa), dB(neg ? NS + sb : sb),
+                                         neg ? idesc_nA : idesc, 1, use);
+                            }
+                    }
+                    mma_commit(&empty[b]);   // the stage is free once these MMAs have read it
+                    if (s == nk - 1) mma_commit(&acc_full);
+                }
+                __syncwarp();
+                if (++b == NST) {
+                    b = 0;
+                    par ^= 1;
+                }
+            }
+        }
+        if (!ok && lane == 0) atomicOr(&prm->err, kErrTimeout);
+    } else if (warp >= 2) {
+        // ---- epilogue warp: 32 tile rows (the lane quarter of tensor memory it may read, a row a lane)
+        // and half the columns, in registers from the read-out on; a lane's columns are consecutive in
+        // memory, so its 16-byte (8-byte) accesses fill the sectors of its row one after another, under
+        // the next tile's products ----
+        constexpr int HC = BN / 2;
+        const int q4 = warp & 3, half = (warp - 2) >> 2;
+        int n = 0;
+        for (int t = blockIdx.x; t < total; t += gridDim.x, ++n) {
+            const OzJob jb = job_of(t);
+            const int rest = t % per_job, item = rest / per_item, tile = rest - item * per_item;
+            const int row = (tile / ntn) * BM + q4 * 32 + lane, ch0 = (tile % ntn) * BN + half * HC;
+            const int ncols = min(HC, d - ch0);
+            const int* eBp = exps + ((size_t)item * kOzMats + jb.b_mat) * d;
+            const int eA = row < d ? exps[((size_t)item * kOzMats + jb.a_mat) * d + row] : 0;
+            int eB[HC / 32];   // this lane's columns' exponents, broadcast by shuffle
+#pragma unroll
+            for (int j = 0; j < HC / 32; ++j) eB[j] = ch0 + 32 * j + lane < d ? eBp[ch0 + 32 * j + lane] : 0;
+            if (!__all_sync(0xffffffffu, mbar_wait(&acc_full, (uint32_t)(n & 1), limit))) {
+                if (lane == 0) atomicOr(&prm->err, kErrTimeout);
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const unsigned char* st = base + b * STAGE;
-            uint64_t Ar[NS], Ai[NS], Br[NS], Bi[NS];
+            const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(half * HC);
+            std::conditional_t<FWD, float4, float2> res[HC];   // FWD: (re_hi, im_hi, re_lo, im_lo)
 #pragma unroll
-            for (int q = 0; q < NS; ++q) {
-                Ar[q] = sdesc(st + q * TILE_A);
-                Ai[q] = sdesc(st + (NS + q) * TILE_A);
-                Br[q] = sdesc(st + NPART * TILE_A + q * TILE_B);
-                Bi[q] = sdesc(st + NPART * TILE_A + (NS + q) * TILE_B);
-            }
-#pragma unroll
-            for (int sa = 0; sa < NS; ++sa)
-#pragma unroll
-                for (int sb = 0; sb + sa < NS; ++sb) {
-                    // slice level sa + sb goes to its own accumulator below NLEV - 1, the rest to the
-                    // last; the first MMA into each accumulator (sa = 0, sb = its level) overwrites it
-                    const int lev = sa + sb < NLEV ? sa + sb : NLEV - 1;
-                    const bool first = sa == 0 && sb == lev;
-                    const uint32_t en = (s > 0 || !first) ? 1u : 0u;
-                    const uint32_t acc_re = tmem + (uint32_t)(2 * lev * BN), acc_im = acc_re + BN;
-                    // re += Ar Br - Ai Bi ;  im += Ar Bi + Ai Br
-                    mma_bf16(acc_re, Ar[sa], Br[sb], idesc, en);
-                    mma_bf16(acc_re, Ai[sa], Bi[sb], idesc_nA, 1);
-                    mma_bf16(acc_im, Ar[sa], Bi[sb], idesc, en);
-                    mma_bf16(acc_im, Ai[sa], Br[sb], idesc, 1);
-                }
-            mma_commit(&empty[b]);   // the stage is free once these MMAs have read it
-        }
-        mma_commit(&done);
-        if (!ok) {
-            atomicOr(&prm->err, kErrTimeout);
-            s_ok = 0;
-        }
-    }
-    // Epilogue warp: 32 tile rows (the lane quarter of tensor memory it may read) and half the columns.
-    // While the products run it brings what its outputs are added to into registers, in the order it
-    // writes them (row rw, column lane + 32 j of its half): the accumulated output (beta), or the
-    // Paterson-Stockmeyer block c0 I + c1 X + c2 X^2 in pair arithmetic.
-    constexpr int HC = BN / 2, JC = HC / 32;           // columns per epilogue warp, per lane
-    const int q4 = warp & 3, ch0 = c0 + ((warp - 2) >> 2) * HC;
-    const int row0 = r0 + q4 * 32, nrows = min(32, d - row0), ncols = min(HC, d - ch0);
-    using Add = std::conditional_t<FWD, float4, float2>;
-    constexpr int PRE = FWD ? 20 : 22;                 // rows held (registers), the others are read when written
-    Add add[PRE][JC];
-    const bool has_add = FWD ? fe.kind == 2 : jb.beta != 0;
-    auto read_add = [&](int rw, int j) -> Add {
-        const int c = lane + 32 * j;
-        const bool in = rw < nrows && c < ncols;
-        if constexpr (FWD) {
-            const size_t o = (size_t)item * fe.ostride + (size_t)(row0 + rw) * d + ch0 + c;
-            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4 xv = in ? fe.X[o] : z4, yv = in ? fe.X2[o] : z4;
-            float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-            pair_fma(rh, rl, fe.c1, xv.x, xv.z);
-            pair_fma(ih, il, fe.c1, xv.y, xv.w);
-            pair_fma(rh, rl, fe.c2, yv.x, yv.z);
-            pair_fma(ih, il, fe.c2, yv.y, yv.w);
-            if (row0 + rw == ch0 + c) df_addc(rh, rl, fe.c0);
-            return make_float4(rh, ih, rl, il);
-        } else {
-            const float2* out = jb.out + (size_t)item * jb.ostride;
-            return in ? out[(size_t)(row0 + rw) * d + ch0 + c] : make_float2(0.f, 0.f);
-        }
-    };
-    if (warp >= 2 && has_add) {
-#pragma unroll
-        for (int rw = 0; rw < PRE; ++rw)
-#pragma unroll
-            for (int j = 0; j < JC; ++j) add[rw][j] = read_add(rw, j);
-    }
-    __syncthreads();
-    const bool fin = mbar_wait(&done, 0, limit);
-    if (!fin && tid == 0) atomicOr(&prm->err, kErrTimeout);
-    // the epilogue's TMEM loads are warp-collective: the decision is the same for every thread
-    const bool go = __syncthreads_and(fin && s_ok != 0) != 0;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (go && warp >= 2) {
-        // Each epilogue warp scales its part of the tile into a staging area of the idle stage ring (every
-        // copy has landed and every MMA has read its operands once `done` completed), then writes it
-        // row by row with the lanes along the columns, so the global stores coalesce.
-        constexpr int SROW = HC + 1;                   // padded row: fewer bank conflicts
-        const int r = row0 + lane;
-        const int eA = r < d ? exps[((size_t)item * kOzMats + jb.a_mat) * d + r] : 0;
-        const int* eBp = exps + ((size_t)item * kOzMats + jb.b_mat) * d;
-        const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(ch0 - c0);
-        if constexpr (!FWD) {
-            float2* stg = reinterpret_cast<float2*>(base) + (size_t)(warp - 2) * 32 * SROW;
-            for (int cc = 0; cc < ncols; cc += 16) {
-                float lr[16], li[16], rr[16], ri[16];
-                tmem_ld16(lane_base + (uint32_t)cc, lr);
-                tmem_ld16(lane_base + (uint32_t)(BN + cc), li);
-                tmem_ld16(lane_base + (uint32_t)(2 * BN + cc), rr);
-                tmem_ld16(lane_base + (uint32_t)(3 * BN + cc), ri);
-                tmem_wait(lr, li, rr, ri);
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int c = ch0 + cc + q;
-                    const float sc = ldexpf(jb.alpha, eA + (c < d ? eBp[c] : 0) - 3 * SBITS);
-                    stg[lane * SROW + cc + q] = make_float2((lr[q] + rr[q]) * sc, (li[q] + ri[q]) * sc);
-                }
-            }
-            __syncwarp();
-            float2* out = jb.out + (size_t)item * jb.ostride;
-            float2 rest[32 - PRE][JC];
-            if (has_add)
-#pragma unroll
-                for (int rw = PRE; rw < 32; ++rw)
-#pragma unroll
-                    for (int j = 0; j < JC; ++j) rest[rw - PRE][j] = read_add(rw, j);
-#pragma unroll
-            for (int rw = 0; rw < 32; ++rw)
-#pragma unroll
-                for (int j = 0; j < JC; ++j) {
-                    const int c = lane + 32 * j;
-                    if (rw >= nrows || c >= ncols) continue;
-                    float2 v = stg[rw * SROW + c];
-                    if (has_add) {
-                        const float2 q = rw < PRE ? add[rw < PRE ? rw : 0][j] : rest[rw < PRE ? 0 : rw - PRE][j];
-                        v.x += q.x;
-                        v.y += q.y;
-                    }
-                    if (jb.ident && row0 + rw == ch0 + c) v.x += 1.0f;
-                    out[(size_t)(row0 + rw) * d + ch0 + c] = v;
-                }
-        } else {
-            // value pairs (re_hi, im_hi, re_lo, im_lo): the three exact levels summed without
-            // error, the remainder level added to the low part; every scaling is by a power of two
-            static_assert(NLEV == 4, "three exact levels and a remainder");
-            float4* stg = reinterpret_cast<float4*>(base) + (size_t)(warp - 2) * 32 * SROW;
-            for (int cc = 0; cc < ncols; cc += 16) {
-#pragma unroll
-                for (int part = 0; part < 2; ++part) {   // re, then im
-                    float a0[16], a1[16], a2[16], a3[16];
-                    tmem_ld16(lane_base + (uint32_t)(part * BN + cc), a0);
-                    tmem_ld16(lane_base + (uint32_t)((2 + part) * BN + cc), a1);
-                    tmem_ld16(lane_base + (uint32_t)((4 + part) * BN + cc), a2);
-                    tmem_ld16(lane_base + (uint32_t)((6 + part) * BN + cc), a3);
-                    tmem_wait(a0, a1, a2, a3);
+            for (int cc = 0; cc < HC; cc += 16) {
+                if constexpr (!FWD) {
+                    float lr[16], li[16], rr[16], ri[16];
+                    tmem_ld16(lane_base + (uint32_t)cc, lr);
+                    tmem_ld16(lane_base + (uint32_t)(BN + cc), li);
+                    tmem_ld16(lane_base + (uint32_t)(2 * BN + cc), rr);
+                    tmem_ld16(lane_base + (uint32_t)(3 * BN + cc), ri);
+                    tmem_wait(lr, li, rr, ri);
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
-                        const int c = ch0 + cc + q;
-                        const float sc = ldexpf(1.0f, eA + (c < d ? eBp[c] : 0) - 3 * SBITS);
-                        float h, l, h2, l2;
-                        two_sum(a0[q] * sc, a1[q] * sc, h, l);
-                        two_sum(h, a2[q] * sc, h2, l2);
-                        h = h2;
-                        l = fmaf(a3[q], sc, l + l2);
-                        float4& o = stg[lane * SROW + cc + q];
-                        if (part == 0) {
-                            o.x = h;
-                            o.z = l;
-                        } else {
-                            o.y = h;
-                            o.w = l;
+                        const int e = __shfl_sync(0xffffffffu, eB[(cc + q) / 32], (cc + q) % 32);
+                        const float sc = ldexpf(jb.alpha, eA + e - 3 * SBITS);
+                        res[cc + q] = make_float2((lr[q] + rr[q]) * sc, (li[q] + ri[q]) * sc);
+                    }
+                } else {
+                    // the three exact levels summed without error, the remainder level added to the low
+                    // part; every scaling is by a power of two
+                    static_assert(!FWD || NLEV == 4, "three exact levels and a remainder");
+#pragma unroll
+                    for (int part = 0; part < 2; ++part) {   // re, then im
+                        float a0[16], a1[16], a2[16], a3[16];
+                        tmem_ld16(lane_base + (uint32_t)(part * BN + cc), a0);
+                        tmem_ld16(lane_base + (uint32_t)((2 + part) * BN + cc), a1);
+                        tmem_ld16(lane_base + (uint32_t)((4 + part) * BN + cc), a2);
+                        tmem_ld16(lane_base + (uint32_t)((6 + part) * BN + cc), a3);
+                        tmem_wait(a0, a1, a2, a3);
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            float h, l, h2, l2;
+                            two_sum(a0[q], a1[q], h, l);
+                            two_sum(h, a2[q], h2, l2);
+                            l = l + l2 + a3[q];
+                            if (part == 0) {
+                                res[cc + q].x = h2;
+                                res[cc + q].z = l;
+                            } else {
+                                res[cc + q].y = h2;
+                                res[cc + q].w = l;
+                            }
                         }
                     }
                 }
             }
+            // tensor memory is read: the next tile's products may start
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            float4* out = fe.out + (size_t)item * fe.ostride;
-            float4 rest[32 - PRE][JC];
-            if (has_add)
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acc_empty)) : "memory");
+            if constexpr (!FWD) {
+                float2* out = jb.out + (size_t)item * jb.ostride + (size_t)row * d + ch0;
 #pragma unroll
-                for (int rw = PRE; rw < 32; ++rw)
+                for (int c8 = 0; c8 < HC; c8 += 8) {
+                    float2 old[8];
+                    if (jb.beta) {
 #pragma unroll
-                    for (int j = 0; j < JC; ++j) rest[rw - PRE][j] = read_add(rw, j);
-#pragma unroll
-            for (int rw = 0; rw < 32; ++rw)
-#pragma unroll
-                for (int j = 0; j < JC; ++j) {
-                    const int c = lane + 32 * j;
-                    if (rw >= nrows || c >= ncols) continue;
-                    const float4 v = stg[rw * SROW + c];
-                    float rh = v.x, rl = v.z, ih = v.y, il = v.w;
-                    if (has_add) {
-                        const float4 q = rw < PRE ? add[rw < PRE ? rw : 0][j] : rest[rw < PRE ? 0 : rw - PRE][j];
-                        df_addc(rh, rl, make_float2(q.x, q.z));
-                        df_addc(ih, il, make_float2(q.y, q.w));
+                        for (int q = 0; q < 8; ++q)
+                            old[q] = (row < d && c8 + q < ncols) ? out[c8 + q] : make_float2(0.f, 0.f);
                     }
-                    float4 o;
-                    grid_split(rh, rl, fe.magic, o.x, o.z);
-                    grid_split(ih, il, fe.magic, o.y, o.w);
-                    out[(size_t)(row0 + rw) * d + ch0 + c] = o;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        if (row >= d || c8 + q >= ncols) continue;
+                        float2 v = res[c8 + q];
+                        if (jb.beta) {
+                            v.x += old[q].x;
+                            v.y += old[q].y;
+                        }
+                        if (jb.ident && row == ch0 + c8 + q) v.x += 1.0f;
+                        out[c8 + q] = v;
+                    }
                 }
+            } else {
+                const size_t o0 = (size_t)item * fe.ostride + (size_t)row * d + ch0;
+#pragma unroll
+                for (int c4 = 0; c4 < HC; c4 += 4) {
+                    float4 xv[4], yv[4];
+                    if (fe.kind == 2) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const bool in = row < d && c4 + q < ncols;
+                            xv[q] = in ? fe.X[o0 + c4 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
+                            yv[q] = in ? fe.X2[o0 + c4 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int e = __shfl_sync(0xffffffffu, eB[0], c4 + q);
+                        if (row >= d || c4 + q >= ncols) continue;
+                        const float sc = ldexpf(1.0f, eA + e - 3 * SBITS);
+                        const float4 v = res[c4 + q];
+                        float rh = v.x * sc, rl = v.z * sc, ih = v.y * sc, il = v.w * sc;
+                        if (fe.kind == 2) {
+                            pair_fma(rh, rl, fe.c1, xv[q].x, xv[q].z);
+                            pair_fma(ih, il, fe.c1, xv[q].y, xv[q].w);
+                            pair_fma(rh, rl, fe.c2, yv[q].x, yv[q].z);
+                            pair_fma(ih, il, fe.c2, yv[q].y, yv[q].w);
+                            if (row == ch0 + c4 + q) df_addc(rh, rl, fe.c0);
+                        }
+                        float4 o;
+                        grid_split(rh, rl, fe.magic, o.x, o.z);
+                        grid_split(ih, il, fe.magic, o.y, o.w);
+                        fe.out[o0 + c4 + q] = o;
+                    }
+                }
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -628,7 +653,7 @@ static EncodeTiledFn oz_encode_fn() {
 
 template <class Cfg>
 static size_t plane_bytes(int d, int items) {
-    return (size_t)items * kOzMats * Cfg::NPART * (size_t)d * oz_ld(d) * 2;
+    return (size_t)items * kOzMats * Cfg::NG * (size_t)d * oz_row(d) * 2;
 }
 template <class Cfg>
 static size_t scratch_bytes(int d, int items) {
@@ -643,17 +668,17 @@ template <class Cfg>
 static cudaError_t make_maps(void* planes, int d, int items, TcMaps* maps) {
     EncodeTiledFn enc = oz_encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    const int ld = oz_ld(d);
-    // x: K (d columns of a plane row), y: plane rows (d), z: planes; reads beyond d fill zeros
-    cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)d, (cuuint64_t)items * kOzMats * Cfg::NPART};
-    cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)ld * d * 2};
+    const int row = oz_row(d);
+    // x: the row of a group, y: plane rows (d), z: groups; rows beyond d fill zeros
+    cuuint64_t dims[3] = {(cuuint64_t)row, (cuuint64_t)d, (cuuint64_t)items * kOzMats * Cfg::NG};
+    cuuint64_t strides[2] = {(cuuint64_t)row * 2, (cuuint64_t)row * d * 2};
     cuuint32_t estr[3] = {1, 1, 1};
-    cuuint32_t boxA[3] = {BK, BM, 1}, boxB[3] = {BK, (cuuint32_t)Cfg::BN, 1};
+    cuuint32_t boxA[3] = {BK * GRP, BM, 1}, boxB[3] = {BK * GRP, (cuuint32_t)Cfg::BN, 1};
     CUresult r1 = enc(reinterpret_cast<CUtensorMap*>(maps->a), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, planes, dims,
-                      strides, boxA, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+                      strides, boxA, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     CUresult r2 = enc(reinterpret_cast<CUtensorMap*>(maps->b), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, planes, dims,
-                      strides, boxB, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+                      strides, boxB, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return (r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS) ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -664,8 +689,7 @@ static cudaError_t slice_launch(const OzSliceJobs& jobs, int njobs, int d, int i
     if (njobs < 1 || njobs > 4 || items > cap) return cudaErrorInvalidValue;
     __nv_bfloat16* planes = reinterpret_cast<__nv_bfloat16*>(scratch);
     const int gx = std::max((d + 7) / 8, (d + 31) / 32);
-    k_oz_slice<Cfg::NS, In><<<dim3(gx, items, njobs), 256, 0, st>>>(jobs, planes, exps_of<Cfg>(scratch, d, cap), d,
-                                                                    oz_ld(d));
+    k_oz_slice<Cfg::NS, In><<<dim3(gx, items, njobs), 256, 0, st>>>(jobs, planes, exps_of<Cfg>(scratch, d, cap), d);
     return cudaGetLastError();
 }
 
@@ -679,10 +703,15 @@ static cudaError_t mm_launch(const OzJobs& jobs, int njobs, const OzFwdEpi& fe, 
         attr = true;
     }
     if (njobs < 1 || njobs > 2 || d > kMaxD || items > cap) return cudaErrorInvalidValue;
-    const int ntiles = ((d + BM - 1) / BM) * ((d + Cfg::BN - 1) / Cfg::BN);
-    k_oz_mm<Cfg, FWD><<<dim3(ntiles, items, njobs), NTHREADS, Cfg::SMEM, st>>>(
-        *reinterpret_cast<const CUtensorMap*>(maps.a), *reinterpret_cast<const CUtensorMap*>(maps.b), jobs, fe,
-        exps_of<Cfg>(scratch, d, cap), d, prm);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return cudaErrorInvalidDevice;
+    const long long ntiles = (long long)((d + BM - 1) / BM) * ((d + Cfg::BN - 1) / Cfg::BN) * items * njobs;
+    if (ntiles > 0x7fffffffll - sms) return cudaErrorInvalidValue;
+    k_oz_mm<Cfg, FWD><<<(int)std::min<long long>(ntiles, sms), NTHREADS, Cfg::SMEM, st>>>(
+        *reinterpret_cast<const CUtensorMap*>(maps.a), *reinterpret_cast<const CUtensorMap*>(maps.b), jobs, njobs, items,
+        fe, exps_of<Cfg>(scratch, d, cap), d, prm);
     return cudaGetLastError();
 }
 

@@ -535,8 +535,8 @@ void plan_impl(qoc_ctx* c) {
         c->scratch.release();
     }
     if (use_oz(c)) {
-        // the tensor maps cover exactly d x d of every plane (reads past d fill zeros), so the
-        // padding columns of the planes are never read and need no clearing
+        // the slicer writes whole K chunks (zero past d) and the tensor maps end at row d (reads past
+        // it fill zeros), so the planes need no clearing
         // the forward's and the adjoint's products run on one stream and share the plane array
         A(c->tc_planes, std::max(oz_scratch_bytes(d, E * W), oz_fwd_on(c) ? oz_fwd_scratch_bytes(d, E * W) : 0),
           "alloc tensor-core slices");

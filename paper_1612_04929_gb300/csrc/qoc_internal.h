@@ -269,7 +269,6 @@ constexpr int kOzFwdSlices = 6;  // seven-bit slices per value (forward products
 constexpr int kOzFwdMinD = 128;  // d range whose forward products BF16_SPLIT runs on the tensor cores
 constexpr int kOzFwdMaxD = 384;  // (the three exact slice levels stay exact up to here)
 constexpr int kOzMats = 5;       // sliced matrices per item: A1, B1, A2, B2 of a reverse step, X^dag
-inline int oz_ld(int d) { return (d + 7) / 8 * 8; }   // plane row stride (BF16): 16-byte rows for TMA
 struct OzSliceJob {
     const void* src;        // d x d row-major complex matrices, item i at src + i * stride elements:
                             // float2 (adjoint) or float4 value pairs (forward)
