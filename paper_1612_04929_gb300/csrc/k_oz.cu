@@ -52,6 +52,7 @@
 
 #include "qoc_device.cuh"
 #include "qoc_internal.h"
+#include "qoc_tree.cuh"
 
 namespace qoc {
 
@@ -208,8 +209,8 @@ __device__ __forceinline__ float4 as_pairs(float4 v) { return make_float4(v.x, v
 // (With a plane per tile and 32-byte rows a forward product of 150 items at d = 256 took 477 us instead of
 // 458 and an adjoint one 269 instead of 250; the slicer pays 5 % for it.)  Group (item, matrix, g):
 template <int NPART>
-__host__ __device__ inline size_t oz_group(int item, int mat, int g) {
-    return ((size_t)item * kOzMats + mat) * (NPART / GRP) + g;
+__host__ __device__ inline size_t oz_group(int item, int mats, int mat, int g) {
+    return ((size_t)item * mats + mat) * (NPART / GRP) + g;
 }
 __host__ __device__ inline int oz_row(int d) { return (d + BK - 1) / BK * BK * GRP; }   // elements of a group's row
 // element k of plane `part` within a row of its group
@@ -219,7 +220,8 @@ __device__ __forceinline__ size_t oz_at(int part, int k) { return (size_t)(k / B
 // slicing: FP32 complex d x d matrices (row-major, item-strided) -> exponents and BF16 planes
 // ------------------------------------------------------------------------------------------
 // Row layout (A operand): plane row r = row r of M, exponent per row.  Column layout (B operand,
-// K-major): plane row c = column c of M, exponent per column (no conjugation is applied).
+// K-major): plane row c = column c of M, exponent per column (no conjugation is applied).  Conjugated
+// column layout: M^dag as an A operand, plane row c = conjugated column c of M.
 // Eight consecutive elements of one plane row (half a K chunk), as one 16-byte store
 __device__ __forceinline__ void store8(__nv_bfloat16* dst, const float (&v)[8]) {
     uint4 w;
@@ -270,10 +272,11 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
     __shared__ int cexp[32];
     const OzSliceJob jb = jobs.job[blockIdx.z];
     const int item = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const In* M = static_cast<const In*>(jb.src) + (size_t)item * jb.stride;
+    const int it = jobs.item0 + item, se = jobs.count ? it / jobs.count : 0;   // member, and its item
+    const In* M = static_cast<const In*>(jb.src) + se * jb.estride + (size_t)(it - se * jobs.count) * jb.stride;
     const int rowlen = oz_row(d), dk = rowlen / GRP;   // dk: d rounded up to whole K chunks
     const size_t gsz = (size_t)d * rowlen;
-    const size_t pbase = oz_group<NPART>(item, jb.mat, 0);
+    const size_t pbase = oz_group<NPART>(item, jobs.mats, jb.mat, 0);
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     // the exponent comes from the rounded values |re|, |im| (a pair's sum rounded up to 2^e only
     // raises e: conservative)
@@ -295,7 +298,7 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
             }
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         const int e = scale_exp(m);
-        if (lane == 0) exps[((size_t)item * kOzMats + jb.mat) * d + r] = e;
+        if (lane == 0) exps[((size_t)item * jobs.mats + jb.mat) * d + r] = e;
 #pragma unroll
         for (int ch = 0; ch < 2; ++ch) {
             const int b0 = ch * 256 + lane * 8;
@@ -317,7 +320,7 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
         for (int w = 1; w < 8; ++w) mm = fmaxf(mm, cmax[w][lane]);
         const int e = scale_exp(mm);
         cexp[lane] = e;
-        if (c < d) exps[((size_t)item * kOzMats + jb.mat) * d + c] = e;
+        if (c < d) exps[((size_t)item * jobs.mats + jb.mat) * d + c] = e;
     }
     __syncthreads();
     // tiles of KT rows: staged with the lanes along the columns (coalesced reads), then thread t
@@ -333,8 +336,11 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
         if (cc < d && kk < dk) {
             float4 q8[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) q8[i] = tile[tk + i][tc];
-            put8<NS>(planes, pbase, gsz, cc, rowlen, kk, q8, cexp[tc], false);
+            for (int i = 0; i < 8; ++i) {
+                q8[i] = tile[tk + i][tc];
+                if (jb.col == 2) q8[i].z = -q8[i].z, q8[i].w = -q8[i].w;
+            }
+            put8<NS>(planes, pbase, gsz, cc, rowlen, kk, q8, cexp[tc], jb.col == 2);
         }
         __syncthreads();
     }
@@ -352,9 +358,17 @@ struct OzFwdEpi {
     float2 c0, c1, c2;
 };
 
+struct OzAdjEpi {};
+// The tree's epilogue: out = A B grid-split with the magic mo (0: of the propagators' exponent), the
+// optional second output and the optional rounded (scaled) value of TreeMm
+struct OzTreeEpi {
+    TreeMm t;
+    int item0;
+};
+
 // ------------------------------------------------------------------------------------------
-// 128 x BN output tiles of the jobs' items: adjoint products (FWD false) C = alpha A B (+ beta C) (+ I)
-// in FP32; forward products (FWD true) as value pairs (OzFwdEpi).  A persistent CTA per SM takes tiles
+// 128 x BN output tiles of the jobs' items: adjoint products (OzAdjEpi) C = alpha A B (+ beta C) (+ I)
+// in FP32; forward products (OzFwdEpi) and the tree's (OzTreeEpi) as value pairs.  A persistent CTA per SM takes tiles
 // blockIdx.x, + gridDim.x, ..: while the epilogue warps add and write one tile, the products of the next
 // run, and only the read-out of tensor memory stands between the products of two tiles.
 // A forward product at d = 256 (450 items, us): 1375 with a CTA per tile; 1204 persistent; 929 with the
@@ -363,10 +377,11 @@ struct OzFwdEpi {
 // the MMAs 530.  An adjoint product (mean of single and double launches): 750, 622, 608, 583, the copies
 // alone 490.
 // ------------------------------------------------------------------------------------------
-template <class Cfg, bool FWD>
+template <class Cfg, class Epi>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, OzJobs jobs, int njobs,
-        int items, OzFwdEpi fe, const int* __restrict__ exps, int d, DevParams* __restrict__ prm) {
+        int items, Epi fe, const int* __restrict__ exps, int d, DevParams* __restrict__ prm) {
+    constexpr bool FWD = !std::is_same_v<Epi, OzAdjEpi>;
     constexpr int NS = Cfg::NS, BN = Cfg::BN, NLEV = Cfg::NLEV, NST = Cfg::NST, NPART = Cfg::NPART;
     constexpr int TILE_A = Cfg::TILE_A, TILE_B = Cfg::TILE_B, STAGE = Cfg::STAGE, NG = Cfg::NG;
     extern __shared__ __align__(1024) unsigned char smraw[];
@@ -426,9 +441,9 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                 unsigned char* st = base + b * STAGE;
                 mbar_expect_tx(&full[b], STAGE);
                 for (int q = 0; q < NG; ++q) {
-                    tma_3d(st + q * TILE_A, &mapA, s * BK * GRP, r0, (int)oz_group<NPART>(item, jb.a_mat, q), &full[b]);
+                    tma_3d(st + q * TILE_A, &mapA, s * BK * GRP, r0, (int)oz_group<NPART>(item, jobs.mats, jb.a_mat, q), &full[b]);
                     tma_3d(st + NG * TILE_A + q * TILE_B, &mapB, s * BK * GRP, c0,
-                           (int)oz_group<NPART>(item, jb.b_mat, q), &full[b]);
+                           (int)oz_group<NPART>(item, jobs.mats, jb.b_mat, q), &full[b]);
                 }
                 last_issued[b] = g;
             }
@@ -508,8 +523,8 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
             const int rest = t % per_job, item = rest / per_item, tile = rest - item * per_item;
             const int row = (tile / ntn) * BM + q4 * 32 + lane, ch0 = (tile % ntn) * BN + half * HC;
             const int ncols = min(HC, d - ch0);
-            const int* eBp = exps + ((size_t)item * kOzMats + jb.b_mat) * d;
-            const int eA = row < d ? exps[((size_t)item * kOzMats + jb.a_mat) * d + row] : 0;
+            const int* eBp = exps + ((size_t)item * jobs.mats + jb.b_mat) * d;
+            const int eA = row < d ? exps[((size_t)item * jobs.mats + jb.a_mat) * d + row] : 0;
             int eB[HC / 32];   // this lane's columns' exponents, broadcast by shuffle
 #pragma unroll
             for (int j = 0; j < HC / 32; ++j) eB[j] = ch0 + 32 * j + lane < d ? eBp[ch0 + 32 * j + lane] : 0;
@@ -590,6 +605,18 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                         out[c8 + q] = v;
                     }
                 }
+            } else if constexpr (std::is_same_v<Epi, OzTreeEpi>) {
+                const TreeMm& tm = fe.t;
+                const int it = fe.item0 + item, te = it / tm.count, ti = it - te * tm.count;
+                const float mo = tm.mo == 0.f ? grid_magic(prm->eu) : tm.mo;
+                const size_t o0 = (size_t)row * d + ch0;
+#pragma unroll
+                for (int q = 0; q < HC; ++q) {
+                    const int e = __shfl_sync(0xffffffffu, eB[0], q);
+                    if (row >= d || q >= ncols) continue;
+                    const float sc = ldexpf(1.0f, eA + e - 3 * SBITS);
+                    tree_store(tm, te, ti, o0 + q, ch0 + q, make_float4(res[q].x * sc, res[q].y * sc, res[q].z * sc, res[q].w * sc), mo);
+                }
             } else {
                 const size_t o0 = (size_t)item * fe.ostride + (size_t)row * d + ch0;
 #pragma unroll
@@ -652,25 +679,25 @@ static EncodeTiledFn oz_encode_fn() {
 }
 
 template <class Cfg>
-static size_t plane_bytes(int d, int items) {
-    return (size_t)items * kOzMats * Cfg::NG * (size_t)d * oz_row(d) * 2;
+static size_t plane_bytes(int d, int items, int mats = kOzMats) {
+    return (size_t)items * mats * Cfg::NG * (size_t)d * oz_row(d) * 2;
 }
 template <class Cfg>
-static size_t scratch_bytes(int d, int items) {
-    return (plane_bytes<Cfg>(d, items) + 255) / 256 * 256 + (size_t)items * kOzMats * d * 4;
+static size_t scratch_bytes(int d, int items, int mats = kOzMats) {
+    return (plane_bytes<Cfg>(d, items, mats) + 255) / 256 * 256 + (size_t)items * mats * d * 4;
 }
 template <class Cfg>
-static int* exps_of(unsigned char* scratch, int d, int cap) {
-    return reinterpret_cast<int*>(scratch + (plane_bytes<Cfg>(d, cap) + 255) / 256 * 256);
+static int* exps_of(unsigned char* scratch, int d, int cap, int mats) {
+    return reinterpret_cast<int*>(scratch + (plane_bytes<Cfg>(d, cap, mats) + 255) / 256 * 256);
 }
 
 template <class Cfg>
-static cudaError_t make_maps(void* planes, int d, int items, TcMaps* maps) {
+static cudaError_t make_maps(void* planes, int d, int items, TcMaps* maps, int mats = kOzMats) {
     EncodeTiledFn enc = oz_encode_fn();
     if (!enc) return cudaErrorNotSupported;
     const int row = oz_row(d);
     // x: the row of a group, y: plane rows (d), z: groups; rows beyond d fill zeros
-    cuuint64_t dims[3] = {(cuuint64_t)row, (cuuint64_t)d, (cuuint64_t)items * kOzMats * Cfg::NG};
+    cuuint64_t dims[3] = {(cuuint64_t)row, (cuuint64_t)d, (cuuint64_t)items * mats * Cfg::NG};
     cuuint64_t strides[2] = {(cuuint64_t)row * 2, (cuuint64_t)row * d * 2};
     cuuint32_t estr[3] = {1, 1, 1};
     cuuint32_t boxA[3] = {BK * GRP, BM, 1}, boxB[3] = {BK * GRP, (cuuint32_t)Cfg::BN, 1};
@@ -689,16 +716,16 @@ static cudaError_t slice_launch(const OzSliceJobs& jobs, int njobs, int d, int i
     if (njobs < 1 || njobs > 4 || items > cap) return cudaErrorInvalidValue;
     __nv_bfloat16* planes = reinterpret_cast<__nv_bfloat16*>(scratch);
     const int gx = std::max((d + 7) / 8, (d + 31) / 32);
-    k_oz_slice<Cfg::NS, In><<<dim3(gx, items, njobs), 256, 0, st>>>(jobs, planes, exps_of<Cfg>(scratch, d, cap), d);
+    k_oz_slice<Cfg::NS, In><<<dim3(gx, items, njobs), 256, 0, st>>>(jobs, planes, exps_of<Cfg>(scratch, d, cap, jobs.mats), d);
     return cudaGetLastError();
 }
 
-template <class Cfg, bool FWD>
-static cudaError_t mm_launch(const OzJobs& jobs, int njobs, const OzFwdEpi& fe, int d, int items, int cap,
+template <class Cfg, class Epi>
+static cudaError_t mm_launch(const OzJobs& jobs, int njobs, const Epi& fe, int d, int items, int cap,
                              unsigned char* scratch, const TcMaps& maps, DevParams* prm, cudaStream_t st) {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_oz_mm<Cfg, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+        cudaError_t e = cudaFuncSetAttribute(k_oz_mm<Cfg, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
         if (e != cudaSuccess) return e;
         attr = true;
     }
@@ -709,9 +736,9 @@ static cudaError_t mm_launch(const OzJobs& jobs, int njobs, const OzFwdEpi& fe, 
         return cudaErrorInvalidDevice;
     const long long ntiles = (long long)((d + BM - 1) / BM) * ((d + Cfg::BN - 1) / Cfg::BN) * items * njobs;
     if (ntiles > 0x7fffffffll - sms) return cudaErrorInvalidValue;
-    k_oz_mm<Cfg, FWD><<<(int)std::min<long long>(ntiles, sms), NTHREADS, Cfg::SMEM, st>>>(
+    k_oz_mm<Cfg, Epi><<<(int)std::min<long long>(ntiles, sms), NTHREADS, Cfg::SMEM, st>>>(
         *reinterpret_cast<const CUtensorMap*>(maps.a), *reinterpret_cast<const CUtensorMap*>(maps.b), jobs, njobs, items,
-        fe, exps_of<Cfg>(scratch, d, cap), d, prm);
+        fe, exps_of<Cfg>(scratch, d, cap, jobs.mats), d, prm);
     return cudaGetLastError();
 }
 
@@ -727,7 +754,7 @@ cudaError_t launch_oz_slice(const OzSliceJobs& jobs, int njobs, int d, int items
 
 cudaError_t launch_oz_mm(const OzJobs& jobs, int njobs, int d, int items, int cap, unsigned char* scratch,
                          const TcMaps& maps, DevParams* prm, cudaStream_t st) {
-    return mm_launch<AdjCfg, false>(jobs, njobs, OzFwdEpi{}, d, items, cap, scratch, maps, prm, st);
+    return mm_launch<AdjCfg>(jobs, njobs, OzAdjEpi{}, d, items, cap, scratch, maps, prm, st);
 }
 
 size_t oz_fwd_scratch_bytes(int d, int items) { return scratch_bytes<FwdCfg>(d, items); }
@@ -753,9 +780,50 @@ cudaError_t oz_fwd_product(const OzFwd& z, const float4* a_src, int a_mat, const
     jobs.fault = z.fault;
     jobs.j[0] = {a_mat, b_mat, nullptr, 0, 1.0f, 0, 0};
     OzFwdEpi fe{out, (long long)ms, kind, magic, X, X2, c0, c1, c2};
-    e = mm_launch<FwdCfg, true>(jobs, 1, fe, z.d, z.items, z.cap, z.scratch, z.maps, z.prm, st);
+    e = mm_launch<FwdCfg>(jobs, 1, fe, z.d, z.items, z.cap, z.scratch, z.maps, z.prm, st);
     count();
     return e;
+}
+
+size_t oz_tree_scratch_bytes(int d, int items) { return scratch_bytes<FwdCfg>(d, items, 2); }
+cudaError_t oz_tree_make_maps(void* planes, int d, int items, TcMaps* maps) {
+    return make_maps<FwdCfg>(planes, d, items, maps, 2);
+}
+
+cudaError_t oz_tree_product(const OzTree& z, const TreeMm& t, int ak, bool bl, DevParams* prm, cudaStream_t st, int* launches) {
+    const int total = t.E * t.count;
+    for (int i0 = 0; i0 < total; i0 += z.cap) {   // the planes hold cap items at a time
+        const int items = std::min(z.cap, total - i0);
+        OzSliceJobs sa{}, sb{};
+        sa.mats = sb.mats = 2;
+        sa.count = sb.count = t.count;
+        sa.item0 = sb.item0 = i0;
+        sa.job[0] = {t.a, t.ai, 0, ak == 2 ? 2 : 0, t.ae};
+        sb.job[0] = {t.b, t.bi, 1, 1, t.be};
+        cudaError_t e;
+        if ((ak == 1) == bl) {   // operands of one type: one launch
+            sa.job[1] = sb.job[0];
+            e = bl ? slice_launch<FwdCfg, float2>(sa, 2, t.d, items, z.cap, z.scratch, st)
+                   : slice_launch<FwdCfg, float4>(sa, 2, t.d, items, z.cap, z.scratch, st);
+        } else {
+            e = ak == 1 ? slice_launch<FwdCfg, float2>(sa, 1, t.d, items, z.cap, z.scratch, st)
+                        : slice_launch<FwdCfg, float4>(sa, 1, t.d, items, z.cap, z.scratch, st);
+            if (e != cudaSuccess) return e;
+            ++*launches;
+            e = bl ? slice_launch<FwdCfg, float2>(sb, 1, t.d, items, z.cap, z.scratch, st)
+                   : slice_launch<FwdCfg, float4>(sb, 1, t.d, items, z.cap, z.scratch, st);
+        }
+        if (e != cudaSuccess) return e;
+        ++*launches;
+        OzJobs jobs{};
+        jobs.mats = 2;
+        jobs.fault = z.fault;
+        jobs.j[0] = {0, 1, nullptr, 0, 1.0f, 0, 0};
+        e = mm_launch<FwdCfg>(jobs, 1, OzTreeEpi{t, i0}, t.d, items, z.cap, z.scratch, z.maps, prm, st);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t oz_rev_step(const OzRev& z, const float2* const ops[4], const size_t strides[4], float2* O1, float2* O2,

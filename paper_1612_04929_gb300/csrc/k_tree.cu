@@ -17,23 +17,22 @@
 // coefficient -2 a_fid O_N w_s / (E W) where G_j is written.
 // Measured on GB300 (evaluation): d = 128, N = 500 11.7 -> 8.3 ms; d = 64,
 // N = 2000 7.05 -> 6.13 ms; d = 256, N = 2000 (BF16_SPLIT) 153 -> 142 ms.
+//
+// BF16_SPLIT with 128 <= d <= 384 runs the same products on the tensor cores (k_oz.cu: both operands cut
+// into six seven-bit slices, accurate as the split product; the epilogue writes what k_tree_mm writes):
+// 7.6 -> 2.7 us a product of d = 256 with its slicing, the evaluation above 124 -> 94.6 ms, error against
+// 64 bits unchanged.  All levels, though a single product is no faster there (62 us either way).
 #include <algorithm>
 #include <cmath>
 
 #include "qoc_device.cuh"
 #include "qoc_gemm.cuh"
 #include "qoc_internal.h"
+#include "qoc_tree.cuh"
 
 namespace qoc {
 
 namespace {
-
-__device__ __forceinline__ float4 tree_split(const float4 v, float m) {
-    float4 o;
-    grid_split(v.x, v.z, m, o.x, o.z);
-    grid_split(v.y, v.w, m, o.y, o.w);
-    return o;
-}
 
 // acc += conj(A) B for A given transposed (a product with A^dag)
 template <int MT>
@@ -61,25 +60,6 @@ struct MacSplitConj {
             }
         }
     }
-};
-
-// One batched product of a level.  Item (e, i): A = a + e ae + i ai (matrices d x d), B = b + e be + i bi
-// (d x cols), out likewise.  A or B may be the slice propagators (float2, rounded; split here).
-struct TreeMm {
-    int d, cols, E, count, tiles_r, tiles_c;
-    const void* a;
-    size_t ae, ai;
-    const void* b;
-    size_t be, bi;
-    float4* out;              // grid-split with mo
-    size_t oe, oi;
-    float4* copy;             // optional second carried output (the block handed to the next wave)
-    size_t ce;
-    float2* round;            // optional rounded output: states, or costates scaled by coef
-    size_t re, ri;
-    const float4* coef;       // per member and column (re, im hi; re, im lo), or nullptr
-    float mo;
-    const DevParams* prm;     // exponent eu of the propagators (and of out when mo is 0)
 };
 
 // AK: 0 A carried, 1 A rounded propagators, 2 A carried and taken as A^dag; BL: B rounded propagators
@@ -121,8 +101,6 @@ __global__ void __launch_bounds__(GemmSplit::NT, GemmSplit::MB) k_tree_mm(TreeMm
     };
     std::conditional_t<AK == 2, MacSplitConj<MT>, MacSplit<MT>> mac;
     gemm_loop<float4, Sh, AK == 2>(smraw, p, d, la, lb, mac);
-    float4* out = t.out + e * t.oe + i * t.oi;
-    float2* rnd = t.round ? t.round + e * t.re + i * t.ri : nullptr;
 #pragma unroll
     for (int x = 0; x < MT; ++x)
 #pragma unroll
@@ -133,22 +111,7 @@ __global__ void __launch_bounds__(GemmSplit::NT, GemmSplit::MB) k_tree_mm(TreeMm
             two_sum(mac.acc[x][y][0], mac.acc[x][y][2], v.x, v.z);
             two_sum(mac.acc[x][y][1], mac.acc[x][y][3], v.y, v.w);
             const size_t o = (size_t)r * cols + c;
-            const float4 g = tree_split(v, mo);
-            out[o] = g;
-            if (t.copy) t.copy[e * t.ce + o] = g;
-            if (rnd) {
-                if (t.coef) {
-                    const float4 q = t.coef[(size_t)e * cols + c];
-                    float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
-                    pair_fma(xh, xl, make_float2(q.x, q.z), v.x, v.z);
-                    pair_fma(xh, xl, make_float2(-q.y, -q.w), v.y, v.w);
-                    pair_fma(yh, yl, make_float2(q.x, q.z), v.y, v.w);
-                    pair_fma(yh, yl, make_float2(q.y, q.w), v.x, v.z);
-                    rnd[o] = make_float2(xh + xl, yh + yl);
-                } else {
-                    rnd[o] = make_float2(v.x + v.z, v.y + v.w);
-                }
-            }
+            tree_store(t, e, i, o, c, v, mo);
         }
 }
 
@@ -206,7 +169,8 @@ __global__ void k_tree_coef(CostView<float> cv, int E, int cols, const double2* 
 int tree_ew_blocks(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 64); }
 
 template <int AK, bool BL>
-cudaError_t mm(const TreeMm& t, cudaStream_t st, int* launches) {
+cudaError_t mm(const TreeArgs& a, const TreeMm& t, cudaStream_t st, int* launches) {
+    if (a.oz) return oz_tree_product(*a.oz, t, AK, BL, a.prm, st, launches);
     constexpr size_t smem = GemmSplit::smem<float4>();
     cudaError_t e = cudaFuncSetAttribute(k_tree_mm<AK, BL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -270,7 +234,7 @@ cudaError_t launch_tree_up(const TreeArgs& a, cudaStream_t st, int* launches) {
             t.out = lev;
             t.oe = ne;
             t.oi = dd;
-            if ((err = l == 1 ? mm<1, true>(t, st, launches) : mm<0, false>(t, st, launches)) != cudaSuccess) return err;
+            if ((err = l == 1 ? mm<1, true>(a, t, st, launches) : mm<0, false>(a, t, st, launches)) != cudaSuccess) return err;
         }
         if (below & 1) {
             const void* s;
@@ -305,7 +269,7 @@ cudaError_t launch_tree_forward(const TreeArgs& a, const float4* start, size_t s
         t.round = states + (size_t)a.wlen * a.slice;
         t.re = states_e;
         t.mo = mo;
-        if ((err = L == 0 ? mm<1, false>(t, st, launches) : mm<0, false>(t, st, launches)) != cudaSuccess) return err;
+        if ((err = L == 0 ? mm<1, false>(a, t, st, launches) : mm<0, false>(a, t, st, launches)) != cudaSuccess) return err;
     }
     for (int l = L - 1; l >= 0; --l) {
         const int step = 1 << l;
@@ -322,7 +286,7 @@ cudaError_t launch_tree_forward(const TreeArgs& a, const float4* start, size_t s
         t.re = states_e;
         t.ri = t.bi;
         t.mo = mo;
-        if ((err = l == 0 ? mm<1, false>(t, st, launches) : mm<0, false>(t, st, launches)) != cudaSuccess) return err;
+        if ((err = l == 0 ? mm<1, false>(a, t, st, launches) : mm<0, false>(a, t, st, launches)) != cudaSuccess) return err;
     }
     return cudaSuccess;
 }
@@ -351,7 +315,7 @@ cudaError_t launch_tree_costate(const TreeArgs& a, const float4* start, size_t s
         t.out = next;
         t.oe = next_e;
         t.mo = mo;
-        if ((err = L == 0 ? mm<1, false>(t, st, launches) : mm<2, false>(t, st, launches)) != cudaSuccess) return err;
+        if ((err = L == 0 ? mm<1, false>(a, t, st, launches) : mm<2, false>(a, t, st, launches)) != cudaSuccess) return err;
     }
     for (int l = L - 1; l >= 0; --l) {
         const int step = 1 << l, cnt = (a.wlen - 1 - step) / (2 * step) + 1;
@@ -374,7 +338,7 @@ cudaError_t launch_tree_costate(const TreeArgs& a, const float4* start, size_t s
             t.ri = t.bi;
             t.coef = coef;
             t.mo = mo;
-            if ((err = l == 0 ? mm<1, false>(t, st, launches) : mm<2, false>(t, st, launches)) != cudaSuccess) return err;
+            if ((err = l == 0 ? mm<1, false>(a, t, st, launches) : mm<2, false>(a, t, st, launches)) != cudaSuccess) return err;
         }
     }
     return cudaSuccess;

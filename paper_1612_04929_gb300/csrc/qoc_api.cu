@@ -156,6 +156,9 @@ struct qoc_ctx {
 
     DevBuf H64, HR, dDelta, norms, psiTR, pathR, fmask, colw, ckpt, Ubuf, states, Gbuf, src, carry, Oj, C5j, Ofin,
         gpart, prm, u_h, grad_h, out_h, scratch, tc_planes;
+    DevBuf tplanes;                      // tree form: its operands' slices on the tensor cores
+    TcMaps tree_maps;
+    int tree_cap = 0;                    // items they hold (0: the products run on the FP32 pipes)
     DevBuf tnodes, tcarry, tcoef, tgtK;  // tree form: nodes (two wave sets), carried blocks, coefficients, Psi_T
     DevBuf hoff, hidx, hval;             // the controls' non-zero elements (SysView), when sparse
     DevBuf sH;                           // s H_0 .. s H_det as FP32 pairs (per-slice split exponential)
@@ -190,7 +193,7 @@ struct qoc_ctx {
         const DevBuf* all[] = {&H64, &HR, &dDelta, &norms, &psiTR, &pathR, &fmask, &colw, &ckpt, &Ubuf, &states,
                                &Gbuf, &src, &carry, &Oj, &C5j, &Ofin, &gpart, &prm, &u_h, &grad_h, &out_h, &scratch,
                                &tc_planes, &Pbuf, &lv0, &lv1, &scanst, &hbuf, &Ybuf, &Zbuf, &Zbig, &sH, &chebd, &stscr, &hoff, &hidx, &hval,
-                               &tnodes, &tcarry, &tcoef, &tgtK,
+                               &tplanes, &tnodes, &tcarry, &tcoef, &tgtK,
                                &frozen_d};
         size_t s = 0;
         for (auto* b : all) s += b->bytes;
@@ -566,6 +569,14 @@ void plan_impl(qoc_ctx* c) {
     } else {
         for (DevBuf* b : {&c->tnodes, &c->tcarry, &c->tcoef, &c->tgtK}) b->release();
     }
+    c->tree_cap = 0;
+    if (c->tree && use_oz(c) && d >= kOzFwdMinD && d <= kOzFwdMaxD) {
+        c->tree_cap = std::min(E * (W / 2 + 1), kOzTreeItems);
+        A(c->tplanes, oz_tree_scratch_bytes(d, c->tree_cap), "alloc tree slices");
+        check_cuda(c, oz_tree_make_maps(c->tplanes.p, d, c->tree_cap, &c->tree_maps), "tensor maps");
+    } else {
+        c->tplanes.release();
+    }
     if (c->scan && !c->tree) {
         const size_t nz = (size_t)c->nzmax, ks = sizeof(K_t<R>);
         const size_t half = (size_t)((seg + 1) / 2);
@@ -841,10 +852,11 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
     };
     if constexpr (sizeof(R) == 4) if (c->tree) {
         // ---- the tree's passes and the per-slice costs on sx, the exponentials and adjoints on st ----
+        const OzTree ozt{c->opt.fault_inject, c->tree_cap, c->tplanes.as<unsigned char>(), c->tree_maps};
         auto targs = [&](int w) {
             return TreeArgs{d, E, sv.S, std::min(W, N - w * W), W, Ub(w), c->ustride,
                             c->tnodes.as<float4>() + (size_t)(w & 1) * E * tree_nodes(W) * dd, c->tcarry.as<float4>(),
-                            slice, prm};
+                            slice, prm, c->tree_cap ? &ozt : nullptr};
         };
         const size_t ck_e = (size_t)c->nseg_total * slice;
         auto ck = [&](int w) { return c->ckpt.as<K>() + (size_t)(w * W / seg) * slice; };   // first block of wave w

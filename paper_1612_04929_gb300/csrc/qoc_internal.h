@@ -274,9 +274,15 @@ struct OzSliceJob {
                             // float2 (adjoint) or float4 value pairs (forward)
     size_t stride;
     int mat;                // plane matrix to write
-    int col;                // 0: row layout (A operand), 1: column layout (B operand)
+    int col;                // 0: row layout (A operand), 1: column layout (B operand), 2: M^dag as A operand
+    size_t estride = 0;     // of members, when the items are count per member
 };
-struct OzSliceJobs { OzSliceJob job[4]; };
+struct OzSliceJobs {
+    OzSliceJob job[4];
+    int mats = kOzMats;     // plane matrices per item
+    int count = 0;          // items per member (0: one member)
+    int item0 = 0;          // first item
+};
 struct OzJob {              // out = alpha A B (+ out if beta) (+ I if ident), per item
     int a_mat, b_mat;
     float2* out;
@@ -287,6 +293,7 @@ struct OzJob {              // out = alpha A B (+ out if beta) (+ I if ident), p
 struct OzJobs {
     OzJob j[2];
     int fault;              // withhold the first operand copy (test of the bounded wait)
+    int mats = kOzMats;     // plane matrices per item
 };
 // the reverse-mode adjoint's products on the tensor cores: state of one wave
 struct OzRev {
@@ -463,6 +470,20 @@ template <typename R> cudaError_t launch_state_grad(const StateGradArgs<R>& a, i
 
 // ---- full-unitary recursions over a binary tree of the wave (k_tree.cu, FP32 forms) ----
 // Blocks are d x S row-major (one panel of width S), slice elements apart.
+// the tree's products on the tensor cores (BF16_SPLIT): planes of the two operands of cap items
+struct OzTree {
+    int fault, cap;
+    unsigned char* scratch; // oz_tree_scratch_bytes(d, cap)
+    TcMaps maps;            // oz_tree_make_maps
+};
+struct TreeMm;
+size_t oz_tree_scratch_bytes(int d, int items);
+cudaError_t oz_tree_make_maps(void* planes, int d, int items, TcMaps* maps);
+// one level (k_tree.cu); ak, bl: the forms of its operands as in k_tree_mm
+cudaError_t oz_tree_product(const OzTree& z, const TreeMm& t, int ak, bool bl, DevParams* prm, cudaStream_t st, int* launches);
+// items sliced at once: d = 256, N = 2000 takes 97.1 ms with 76, 95.8 with 152, 94.6 with 304 (0.95 GB of
+// planes), 94.3 with 608
+constexpr int kOzTreeItems = 304;
 struct TreeArgs {
     int d, E, S, wlen, W;   // slices of this wave; the most a wave has (strides)
     const float2* U;        // propagators of the wave: U_j at U + (e W + j) ustride, U_j^dag at + ustride / 2
@@ -470,7 +491,8 @@ struct TreeArgs {
     float4* nodes;          // tree_nodes(W) d x d matrices per member, grid-split
     float4* carry;          // W + 1 blocks per member: the pass's states or costates, grid-split
     size_t slice;
-    const DevParams* prm;
+    DevParams* prm;
+    const OzTree* oz;       // or nullptr
 };
 constexpr int kTreeMinD = 48;
 int tree_levels(int wlen);
