@@ -979,6 +979,29 @@ static cudaError_t rev_launch(int d, int items, const RevOps<C>& ops, C* O1, C* 
     }
 }
 
+// Ubar = G Psi^dag into out.  A tiled product of the staged factors Zf, Xf; with oz a product on the tensor
+// cores (FP32-grade as the others of the reverse mode), and full unitaries in one panel are read where
+// they are: 1390 -> 700 us for 450 items at d = 256, S = 256 (staging or slicing included).
+template <typename R>
+static cudaError_t ubar_launch(const BigArgs<R>& a, const StateView<R>& sv, const C_t<R>* states, const C_t<R>* Gbuf,
+                               C_t<R>* Zf, C_t<R>* Xf, C_t<R>* out, cudaStream_t st, int* launches, const OzRev* oz) {
+    using C = C_t<R>;
+    const int d = a.d, items = a.wlen * a.E;
+    const size_t ms = a.mstride, slice = sv.slice();
+    if (sizeof(C) == 8 && oz && sv.S == d && sv.cb == d)
+        return oz_ubar(*oz, {Gbuf, slice, 0, 0, a.wmax * slice}, {states, slice, 1, 3, (a.wmax + 1) * slice}, a.wlen,
+                       reinterpret_cast<float2*>(out), ms, st, launches);
+    k_big_ubar_factors<C><<<dim3(ew_blocks((size_t)d * d), items), 256, 0, st>>>(d, sv, a.wlen, states, Gbuf, a.wmax, Zf, Xf, ms);
+    if (launches) ++*launches;
+    cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    if (sizeof(C) == 8 && oz)
+        return oz_ubar(*oz, {Zf, ms, 0, 0}, {Xf, ms, 1, 1}, 0, reinterpret_cast<float2*>(out), ms, st, launches);
+    err = mm_launch<C, 0>(d, items, Zf, Xf, out, ms, 1, 0, st);
+    if (launches) ++*launches;
+    return err;
+}
+
 template <typename R>
 cudaError_t launch_big_adj_rev(const BigArgs<R>& a, const SysView<R>& sys, const StateView<R>& sv, const C_t<R>* states,
                                const C_t<R>* Gbuf, double* gpart, int p, int n, const C_t<R>* zst, cudaStream_t st,
@@ -997,11 +1020,7 @@ cudaError_t launch_big_adj_rev(const BigArgs<R>& a, const SysView<R>& sys, const
     count();
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_big_ubar_factors<C><<<dim3(eb, items), 256, 0, st>>>(d, sv, a.wlen, states, Gbuf, a.wmax, Zb, Xb, ms);
-    count();
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    if ((err = mm_launch<C, 0>(d, items, Zb, Xb, Za, ms, 1, 0, st)) != cudaSuccess) return err;
-    count();
+    if ((err = ubar_launch<R>(a, sv, states, Gbuf, Zb, Xb, Za, st, launches, oz)) != cudaSuccess) return err;
     if ((err = cudaMemsetAsync(Xb, 0, (size_t)items * ms * sizeof(C), st)) != cudaSuccess) return err;
     C *zb = Za, *zo = Zb;
     // tensor-core products (BF16_SPLIT): X^dag is sliced once for the wave
@@ -1071,11 +1090,7 @@ cudaError_t launch_big_adj_rev_ps(const BigArgs<R>& a, const SysView<R>& sys, co
         C* X2b = Xb + (size_t)items * ms;
         C* Yb = X2b + (size_t)items * ms;
         cudaError_t err;
-        k_big_ubar_factors<C><<<dim3(eb, items), 256, 0, st>>>(d, sv, a.wlen, states, Gbuf, a.wmax, Zb, Xb, ms);
-        count();
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        if ((err = mm_launch<C, 0>(d, items, Zb, Xb, Za, ms, 1, 0, st)) != cudaSuccess) return err;
-        count();
+        if ((err = ubar_launch<R>(a, sv, states, Gbuf, Zb, Xb, Za, st, launches, oz)) != cudaSuccess) return err;
         if ((err = cudaMemsetAsync(Xb, 0, 3 * (size_t)items * ms * sizeof(C), st)) != cudaSuccess) return err;
         C *zb = Za, *zo = Zb;
         int xh_sliced = 0;

@@ -221,7 +221,8 @@ __device__ __forceinline__ size_t oz_at(int part, int k) { return (size_t)(k / B
 // ------------------------------------------------------------------------------------------
 // Row layout (A operand): plane row r = row r of M, exponent per row.  Column layout (B operand,
 // K-major): plane row c = column c of M, exponent per column (no conjugation is applied).  Conjugated
-// column layout: M^dag as an A operand, plane row c = conjugated column c of M.
+// column layout: M^dag as an A operand, plane row c = conjugated column c of M.  Conjugated row layout:
+// M^dag as a B operand.
 // Eight consecutive elements of one plane row (half a K chunk), as one 16-byte store
 __device__ __forceinline__ void store8(__nv_bfloat16* dst, const float (&v)[8]) {
     uint4 w;
@@ -281,7 +282,7 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
     // the exponent comes from the rounded values |re|, |im| (a pair's sum rounded up to 2^e only
     // raises e: conservative)
     auto mag = [](float4 q) { return fmaxf(fabsf(q.x + q.y), fabsf(q.z + q.w)); };
-    if (!jb.col) {
+    if (jb.col == 0 || jb.col == 3) {
         // row layout: one warp per row, each lane eight consecutive columns per 256-column chunk
         // (d <= 512: at most two chunks, held in registers between the maximum and the slicing)
         const int r = blockIdx.x * 8 + warp;
@@ -302,7 +303,12 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
 #pragma unroll
         for (int ch = 0; ch < 2; ++ch) {
             const int b0 = ch * 256 + lane * 8;
-            if (b0 < dk) put8<NS>(planes, pbase, gsz, r, rowlen, b0, v[ch], e, true);
+            if (b0 >= dk) continue;
+            if (jb.col == 3) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[ch][i].z = -v[ch][i].z, v[ch][i].w = -v[ch][i].w;
+            }
+            put8<NS>(planes, pbase, gsz, r, rowlen, b0, v[ch], e, jb.col != 3);
         }
         return;
     }
@@ -824,6 +830,23 @@ cudaError_t oz_tree_product(const OzTree& z, const TreeMm& t, int ak, bool bl, D
         ++*launches;
     }
     return cudaSuccess;
+}
+
+cudaError_t oz_ubar(const OzRev& z, const OzSliceJob& G, const OzSliceJob& P, int count, float2* out, size_t ms,
+                    cudaStream_t st, int* launches) {
+    OzSliceJobs sj{};
+    sj.count = count;
+    sj.job[0] = G;
+    sj.job[1] = P;
+    cudaError_t e = launch_oz_slice(sj, 2, z.d, z.items, z.cap, z.scratch, st);
+    if (launches) ++*launches;
+    if (e != cudaSuccess) return e;
+    OzJobs jobs{};
+    jobs.fault = z.fault;
+    jobs.j[0] = {G.mat, P.mat, out, (long long)ms, 1.0f, 0, 0};
+    e = launch_oz_mm(jobs, 1, z.d, z.items, z.cap, z.scratch, z.maps, z.prm, st);
+    if (launches) ++*launches;
+    return e;
 }
 
 cudaError_t oz_rev_step(const OzRev& z, const float2* const ops[4], const size_t strides[4], float2* O1, float2* O2,

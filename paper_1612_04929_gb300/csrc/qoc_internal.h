@@ -274,7 +274,7 @@ struct OzSliceJob {
                             // float2 (adjoint) or float4 value pairs (forward)
     size_t stride;
     int mat;                // plane matrix to write
-    int col;                // 0: row layout (A operand), 1: column layout (B operand), 2: M^dag as A operand
+    int col;                // 0: row layout (A operand), 1: column layout (B operand), 2, 3: M^dag as A, B operand
     size_t estride = 0;     // of members, when the items are count per member
 };
 struct OzSliceJobs {
@@ -316,6 +316,10 @@ cudaError_t launch_oz_mm(const OzJobs& jobs, int njobs, int d, int items, int ca
 // O2 += A2 B2 / i; mode 1 (squaring) O1 = A1 B1 + A2 B2; ops = {A1, B1, A2, B2} with item strides
 cudaError_t oz_rev_step(const OzRev& z, const float2* const ops[4], const size_t strides[4], float2* O1, float2* O2,
                         size_t ms, int mode, int i, cudaStream_t st, int* launches);
+
+// Ubar = A B of the operands that G and P describe (count items a member), into out
+cudaError_t oz_ubar(const OzRev& z, const OzSliceJob& G, const OzSliceJob& P, int count, float2* out, size_t ms,
+                    cudaStream_t st, int* launches);
 
 // The forward products of the Paterson-Stockmeyer form on the tensor cores (BF16_SPLIT, batched
 // path): six seven-bit slices of the value pairs, the leading two slice levels accumulated exactly
