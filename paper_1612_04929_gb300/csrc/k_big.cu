@@ -723,7 +723,8 @@ static int ew_blocks(size_t dd) {
 // products): X^2 and X^3, the top block element-wise, the chain W_q = B_q + X^3 W_{q+1} with B_q
 // added in the product's epilogue (split products for q <= (m_split - 1) / 3, plain FP32 above),
 // then the squarings.  Scratch per item: X, X^2, X^3 and the W ping-pong (five float4 matrices).
-// Stored operands (conjugate transposes) in the slot layout of ps_slots.
+// Stored operands (conjugate transposes) in the slot layout of ps_slots; those that a tensor-core product
+// makes are stored by its epilogue (a pass each before, 143 us for 450 items at d = 256).
 static cudaError_t big_expm_ps(const BigArgs<float>& a, const DevParams& hp, cudaStream_t st, int* launches,
                                float2* zst, const OzFwd* ozf) {
     const int p = hp.p, n = hp.n, d = a.d, items = a.wlen * a.E;
@@ -759,26 +760,27 @@ static cudaError_t big_expm_ps(const BigArgs<float>& a, const DevParams& hp, cud
     // squarings (1 keeps X for X^3), 2 X^2, 3 X^3 (once for the whole chain), 4 the chain operand.
     const PsAdd none{};
     auto tc = [&](const float4* A, int am, const float4* B, int bm, float4* O, int kind, float mg,
-                  const PsAdd& ps) -> cudaError_t {
+                  const PsAdd& ps, int slot) -> cudaError_t {   // slot: the output's, or -1
         int n_l = 0;
+        float2* ct = zst && slot >= 0 ? zst + (size_t)slot * ms : nullptr;
         const cudaError_t e2 = oz_fwd_product(*ozf, A, am, B, bm, O, ms, kind, mg, ps.X, ps.X2, ps.c0, ps.c1, ps.c2,
-                                              st, &n_l);
+                                              ct, (size_t)cap * ms, st, &n_l);
         if (launches) *launches += n_l;
         return e2;
     };
     if (p >= 2) {
-        err = ozf ? tc(X, 0, X, 1, X2, 1, magic(hp.e2), none)
+        err = ozf ? tc(X, 0, X, 1, X2, 1, magic(hp.e2), none, 0)
                   : mm_launch<float4, 1>(d, items, X, X, X2, ms, 1, 0, st, magic(hp.e2));
         if (!ozf) count();
         if (err != cudaSuccess) return err;
-        if ((err = store(X2, 0)) != cudaSuccess) return err;
+        if (!ozf && (err = store(X2, 0)) != cudaSuccess) return err;
     }
     if (p >= 3) {
-        err = ozf ? tc(X2, 2, nullptr, 1, X3, 1, magic(hp.e3), none)
+        err = ozf ? tc(X2, 2, nullptr, 1, X3, 1, magic(hp.e3), none, 1)
                   : mm_launch<float4, 1>(d, items, X2, X, X3, ms, 1, 0, st, magic(hp.e3));
         if (!ozf) count();
         if (err != cudaSuccess) return err;
-        if ((err = store(X3, 1)) != cudaSuccess) return err;
+        if (!ozf && (err = store(X3, 1)) != cudaSuccess) return err;
     }
     auto form_of = [&](int q) { return ozf ? (q == 0 ? hp.eu : hp.ew[q]) : form_w(q); };
     k_big_ps_top<<<dim3(eb, items), 256, 0, st>>>(d, X, X2, X3, win, ms, coef(3 * qt), coef(3 * qt + 1),
@@ -786,7 +788,7 @@ static cudaError_t big_expm_ps(const BigArgs<float>& a, const DevParams& hp, cud
     count();
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     for (int q = qt - 1; q >= 0; --q) {
-        if ((err = store(win, 2 + (qt - 1 - q))) != cudaSuccess) return err;
+        if ((!ozf || q == qt - 1) && (err = store(win, 2 + (qt - 1 - q))) != cudaSuccess) return err;
         PsAdd ps;
         ps.X = X;
         ps.X2 = X2;
@@ -796,7 +798,7 @@ static cudaError_t big_expm_ps(const BigArgs<float>& a, const DevParams& hp, cud
         const int f = form_of(q);
         const float mg = f == kFullForm ? 0.f : magic(f);
         if (ozf) {
-            err = tc(q == qt - 1 ? X3 : nullptr, 3, win, 4, wout, 2, mg, ps);
+            err = tc(q == qt - 1 ? X3 : nullptr, 3, win, 4, wout, 2, mg, ps, q > 0 || n > 0 ? 2 + qt - q : -1);
         } else {
             err = (q <= qs) ? mm_launch<float4, 1>(d, items, X3, win, wout, ms, 2, 0, st, mg, ps)
                             : mm_launch<float4, 2>(d, items, X3, win, wout, ms, 2, 0, st, mg, ps);
@@ -806,9 +808,9 @@ static cudaError_t big_expm_ps(const BigArgs<float>& a, const DevParams& hp, cud
         std::swap(win, wout);
     }
     for (int m = 0; m < n; ++m) {
-        if ((err = store(win, qt + 2 + m)) != cudaSuccess) return err;
+        if ((!ozf || (m == 0 && qt == 0)) && (err = store(win, qt + 2 + m)) != cudaSuccess) return err;
         if (ozf) {
-            err = tc(win, 0, win, 1, wout, 1, magic(hp.eu), none);
+            err = tc(win, 0, win, 1, wout, 1, magic(hp.eu), none, m + 1 < n ? qt + 3 + m : -1);
         } else {
             err = mm_launch<float4, 1>(d, items, win, win, wout, ms, 1, 0, st, magic(hp.eu));
             count();

@@ -362,6 +362,8 @@ struct OzFwdEpi {
     const float4* X;
     const float4* X2;
     float2 c0, c1, c2;
+    float2* ct;             // optional: the output's rounded conjugate transpose (item stride cts)
+    size_t cts;
 };
 
 struct OzAdjEpi {};
@@ -654,6 +656,9 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                         grid_split(rh, rl, fe.magic, o.x, o.z);
                         grid_split(ih, il, fe.magic, o.y, o.w);
                         fe.out[o0 + c4 + q] = o;
+                        if (fe.ct)   // the lanes' rows are consecutive there
+                            fe.ct[(size_t)item * fe.cts + (size_t)(ch0 + c4 + q) * d + row] =
+                                make_float2(o.x + o.z, -(o.y + o.w));
                     }
                 }
             }
@@ -770,7 +775,7 @@ cudaError_t oz_fwd_make_maps(void* planes, int d, int items, TcMaps* maps) {
 
 cudaError_t oz_fwd_product(const OzFwd& z, const float4* a_src, int a_mat, const float4* b_src, int b_mat,
                            float4* out, size_t ms, int kind, float magic, const float4* X, const float4* X2, float2 c0,
-                           float2 c1, float2 c2, cudaStream_t st, int* launches) {
+                           float2 c1, float2 c2, float2* ct, size_t cts, cudaStream_t st, int* launches) {
     auto count = [&]() { if (launches) ++*launches; };
     if (magic == 0.f || (kind == 2 && (!X || !X2))) return cudaErrorInvalidValue;
     OzSliceJobs sj{};
@@ -785,7 +790,7 @@ cudaError_t oz_fwd_product(const OzFwd& z, const float4* a_src, int a_mat, const
     OzJobs jobs{};
     jobs.fault = z.fault;
     jobs.j[0] = {a_mat, b_mat, nullptr, 0, 1.0f, 0, 0};
-    OzFwdEpi fe{out, (long long)ms, kind, magic, X, X2, c0, c1, c2};
+    OzFwdEpi fe{out, (long long)ms, kind, magic, X, X2, c0, c1, c2, ct, cts};
     e = mm_launch<FwdCfg>(jobs, 1, fe, z.d, z.items, z.cap, z.scratch, z.maps, z.prm, st);
     count();
     return e;

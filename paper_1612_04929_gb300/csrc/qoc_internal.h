@@ -335,10 +335,11 @@ size_t oz_fwd_scratch_bytes(int d, int items);
 cudaError_t oz_fwd_make_maps(void* planes, int d, int items, TcMaps* maps);
 // out = A B (kind 1) or A B + c0 I + c1 X + c2 X^2 (kind 2, the chain product), written as value
 // pairs grid-split with `magic`; a_src / b_src (item stride ms) are sliced into matrices a_mat /
-// b_mat first, or null when that matrix already holds the operand's slices
+// b_mat first, or null when that matrix already holds the operand's slices; ct (or nullptr): the
+// output's rounded conjugate transpose, item stride cts
 cudaError_t oz_fwd_product(const OzFwd& z, const float4* a_src, int a_mat, const float4* b_src, int b_mat,
                            float4* out, size_t ms, int kind, float magic, const float4* X, const float4* X2, float2 c0,
-                           float2 c1, float2 c2, cudaStream_t st, int* launches);
+                           float2 c1, float2 c2, float2* ct, size_t cts, cudaStream_t st, int* launches);
 
 // ---- serial sweeps (k_serial.cu) ----
 // mode 0: forward propagation of one wave (grid z = 1) from checkpoint `seg0`, storing the
