@@ -370,7 +370,11 @@ def roofline_of(prob, precision, info, prof, K, peaks, traffic_key=None):
     slices = prob.N if top_name != "expm_fwd (recompute)" else prob.N - last
     flops = per_slice[top_name] * slices * prob.E * K
     achieved = flops / (top_ms / 1e3) / 1e12
-    tensor = precision == "bf16" and top_name == "expm_adj" and info["kernel_path"] == 1
+    # the form's tensor-core products: the adjoint's, and the forward's for 128 <= d <= 384
+    mmas = OZ_MMA_PER_COMPLEX_PRODUCT["fwd" if top_name.startswith("expm_fwd") else "adj"]
+    tensor = (precision == "bf16" and info["kernel_path"] == 1 and
+              (top_name == "expm_adj" or (top_name.startswith("expm_fwd") and 128 <= prob.d <= 384 and
+                                          info["taylor_scheme"] == 1)))
     if tensor:
         peak, bound, src = peaks["bf16_tflops"], "tensor", peaks["tensor_source"] + ", BF16 burst"
     elif precision == "fp64":
@@ -386,9 +390,9 @@ def roofline_of(prob, precision, info, prof, K, peaks, traffic_key=None):
             "traffic_source": ("dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of this kernel at "
                                "this workload, per slice, times this run's average slices per launch") if traffic else None}
     if tensor:
-        roof["executed_mma_tflops"] = achieved * OZ_MMA_PER_COMPLEX_PRODUCT / 4.0
+        roof["executed_mma_tflops"] = achieved * mmas / 4.0
         roof["note"] = ("algorithmic flops count 8 d^3 per complex product; the exact-accumulation tensor-core "
-                        "products issue %d real BF16 GEMMs of d^3 per complex product" % OZ_MMA_PER_COMPLEX_PRODUCT)
+                        "products issue %d real BF16 GEMMs of d^3 per complex product" % mmas)
     elif precision != "fp64" and top_name.startswith("expm_fwd") and info["kernel_path"] == 0:
         roof["note"] = ("algorithmic flops (8 d^3 per complex product); the FP32 form's grid-split products "
                         "execute 12 FMAs per complex multiply-add (3.25 per algorithmic one), so the split "
@@ -403,10 +407,10 @@ def state_matvecs_per_slice(info):
 
 
 def state_roofline(prob, precision, info, prof, K, peaks):
-    """State mode: the dominant kernel is one of the serial chains (forward or costate), one CTA per
-    (panel, member); its algorithmic flops are 8 d^2 S per matrix-vector product (complex), one
+    """State mode: the dominant kernel is one of the serial chains (forward or costate), one cluster of
+    CTAs per (panel, member); its algorithmic flops are 8 d^2 S per matrix-vector product (complex), one
     product per Horner step or Chebyshev term.  The peak is the FP32 (FP64) FMA peak of the whole
-    GPU although the chain runs on one SM per (panel, member): the fraction shows how far a single
+    GPU although the chain runs on a few SMs per (panel, member): the fraction shows how far a single
     trajectory is from the GPU's throughput."""
     cands = {k: v for k, v in prof.items() if k.startswith("state_chain")}
     if not cands:
@@ -418,12 +422,12 @@ def state_roofline(prob, precision, info, prof, K, peaks):
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": None, "kernel": top_name, "launches": top_launches, "avg_launch_ms": top_ms / top_launches,
             "peak_source": peaks["fp_source"] + " (of measured)",
-            "note": "serial chain: one CTA per (column panel, member), so at most E * panels SMs are busy"}
+            "note": "serial chain: a cluster of up to 16 CTAs per (column panel, member), one dependent product after another"}
 
 
-# real BF16 GEMMs of d^3 per complex product in the exact-accumulation tensor-core form: 10 slice
-# pairs x 4 real products
-OZ_MMA_PER_COMPLEX_PRODUCT = 40
+# real BF16 GEMMs of d^3 per complex product in the exact-accumulation tensor-core form: 10 (adjoint)
+# or 21 (forward) slice pairs x 4 real products
+OZ_MMA_PER_COMPLEX_PRODUCT = {"adj": 40, "fwd": 84}
 
 
 def time_device_evals(ctx, u, grad, out, K, warmup, flush, stream):
