@@ -180,21 +180,29 @@ __device__ __forceinline__ int scale_exp(float m) {
 // on a grid much coarser than the row's largest value has a low part far above the high part's
 // last bit, which would push the slices past the eight bits BF16 holds exactly); the residual is
 // then carried as an error-free pair: a_s = rint(H), (H, L) <- TwoSum(H - a_s, L) 2^7, exact at
-// every step (lo = 0 for FP32 values).
-template <int NS>
+// every step.  FP32 values (PAIR false) need no second part: H - a_s is exact.
+__device__ __forceinline__ float rint_small(float h) {   // |h| < 2^22, by two additions: FRND has a quarter of their rate
+    const float m = 12582912.0f;                         // 1.5 * 2^23
+    return __fadd_rn(__fadd_rn(h, m), -m);
+}
+template <int NS, bool PAIR>
 __device__ __forceinline__ void slices(float hi, float lo, int e, bool role_a, float (&q)[NS]) {
-    float h0, l0;
-    two_sum(hi, lo, h0, l0);
-    float h = ldexpf(h0, SBITS - e), l = ldexpf(l0, SBITS - e);
+    float h0 = hi, l0 = 0.f;
+    if constexpr (PAIR) two_sum(hi, lo, h0, l0);
+    float h = ldexpf(h0, SBITS - e), l = PAIR ? ldexpf(l0, SBITS - e) : 0.f;
     float w = role_a ? (float)(1 << SBITS) : 1.0f;
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-        const float a = rintf(h);
+        const float a = rint_small(h);
         q[s] = a * w;
-        float t, u;
-        two_sum(h - a, l, t, u);
-        h = t * (float)(1 << SBITS);
-        l = u * (float)(1 << SBITS);
+        if constexpr (PAIR) {
+            float t, u;
+            two_sum(h - a, l, t, u);
+            h = t * (float)(1 << SBITS);
+            l = u * (float)(1 << SBITS);
+        } else {
+            h = (h - a) * (float)(1 << SBITS);
+        }
         w *= 1.0f / (float)(1 << SBITS);
     }
 }
@@ -240,14 +248,14 @@ __device__ __forceinline__ void store8(__nv_bfloat16* dst, const float (&v)[8]) 
 
 // the slices of eight consecutive elements k0 .. k0 + 7 of plane row `row` (zero past d), written as
 // 16-byte stores into the row's 2 NS planes; gsz: elements of a group (d rows)
-template <int NS>
+template <int NS, bool PAIR>
 __device__ __forceinline__ void put8(__nv_bfloat16* __restrict__ planes, size_t pbase, size_t gsz, int row, int rowlen,
                                      int k0, const float4 (&q)[8], int e, bool role_a) {
     float sr[8][NS], si[8][NS];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        slices<NS>(q[i].x, q[i].y, e, role_a, sr[i]);
-        slices<NS>(q[i].z, q[i].w, e, role_a, si[i]);
+        slices<NS, PAIR>(q[i].x, q[i].y, e, role_a, sr[i]);
+        slices<NS, PAIR>(q[i].z, q[i].w, e, role_a, si[i]);
     }
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
@@ -267,8 +275,9 @@ template <int NS, typename In>
 __global__ void __launch_bounds__(256)
 k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict__ exps, int d) {
     constexpr int NPART = 2 * NS;
+    constexpr bool PAIR = std::is_same_v<In, float4>;
     constexpr int KT = 64;                       // rows of M per staged tile (column layout)
-    __shared__ float4 tile[KT][33];
+    __shared__ In tile[KT][33];
     __shared__ float cmax[8][32];
     __shared__ int cexp[32];
     const OzSliceJob jb = jobs.job[blockIdx.z];
@@ -308,7 +317,7 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
 #pragma unroll
                 for (int i = 0; i < 8; ++i) v[ch][i].z = -v[ch][i].z, v[ch][i].w = -v[ch][i].w;
             }
-            put8<NS>(planes, pbase, gsz, r, rowlen, b0, v[ch], e, jb.col != 3);
+            put8<NS, PAIR>(planes, pbase, gsz, r, rowlen, b0, v[ch], e, jb.col != 3);
         }
         return;
     }
@@ -329,13 +338,15 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
         if (c < d) exps[((size_t)item * jobs.mats + jb.mat) * d + c] = e;
     }
     __syncthreads();
-    // tiles of KT rows: staged with the lanes along the columns (coalesced reads), then thread t
-    // slices column t % 32 over the eight rows 8 (t / 32) .. + 7 of the tile
-    const int tc = tid & 31, tk = (tid >> 5) * 8;
+    // tiles of KT rows: staged with the lanes along the columns (coalesced reads), then thread t slices
+    // column (t / 2) % 32 over eight rows of the tile: two neighbours write one 32-byte sector of a plane
+    // (with the lanes along the columns each wrote half a sector: d = 256, 450 items, four matrices 577 us
+    // instead of 453)
+    const int tc = (tid >> 1) & 31, tk = (tid >> 6) * 16 + (tid & 1) * 8;
     for (int k0 = 0; k0 < d; k0 += KT) {
         for (int q = warp; q < KT; q += 8) {
             const int k = k0 + q;
-            tile[q][lane] = (k < d && c < d) ? as_pairs(M[(size_t)k * d + c]) : zero4;
+            tile[q][lane] = (k < d && c < d) ? M[(size_t)k * d + c] : In{};
         }
         __syncthreads();
         const int cc = c0 + tc, kk = k0 + tk;
@@ -343,10 +354,10 @@ k_oz_slice(OzSliceJobs jobs, __nv_bfloat16* __restrict__ planes, int* __restrict
             float4 q8[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                q8[i] = tile[tk + i][tc];
+                q8[i] = as_pairs(tile[tk + i][tc]);
                 if (jb.col == 2) q8[i].z = -q8[i].z, q8[i].w = -q8[i].w;
             }
-            put8<NS>(planes, pbase, gsz, cc, rowlen, kk, q8, cexp[tc], jb.col == 2);
+            put8<NS, PAIR>(planes, pbase, gsz, cc, rowlen, kk, q8, cexp[tc], jb.col == 2);
         }
         __syncthreads();
     }
@@ -379,7 +390,7 @@ struct OzTreeEpi {
 // in FP32; forward products (OzFwdEpi) and the tree's (OzTreeEpi) as value pairs.  A persistent CTA per SM takes tiles
 // blockIdx.x, + gridDim.x, ..: while the epilogue warps add and write one tile, the products of the next
 // run, and only the read-out of tensor memory stands between the products of two tiles.
-// A forward product at d = 256 (450 items, us): 1375 with a CTA per tile; 1204 persistent; 929 with the
+// A forward product at d = 256 (450 items, us): 1375 with a CTA per tile (from 150 items); 1204 persistent; 929 with the
 // MMAs' operands in uniform registers (elect); 742 with A read once per run by the collector, 60 % of the
 // tensor rate at 1.9 GHz.  What is left: the copies alone (4.2 GB of plane tiles through L2 a launch, 2.8 GB of HBM traffic) take 599,
 // the MMAs 530.  An adjoint product (mean of single and double launches): 750, 622, 608, 583, the copies
