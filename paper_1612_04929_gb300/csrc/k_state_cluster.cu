@@ -48,7 +48,9 @@ __device__ __forceinline__ uint32_t sc_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
+// (the .aligned forms ask every thread of a warp to be there together: lanes may have parted before)
 __device__ __forceinline__ void sc_cluster_sync() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void sc_expect(uint32_t bar, uint32_t bytes) {
@@ -367,7 +369,6 @@ __global__ void __launch_bounds__(sc_max_warps(RW) * 32) k_state_cluster(StateCh
         }
     }
     if (!ok && lane == 0) atomicOr(&const_cast<DevParams*>(A.prm)->err, kErrTimeout);
-    __syncwarp();
     sc_cluster_sync();
 }
 
