@@ -982,7 +982,7 @@ static cudaError_t rev_launch(int d, int items, const RevOps<C>& ops, C* O1, C* 
 }
 
 // Ubar = G Psi^dag into out.  A tiled product of the staged factors Zf, Xf; with oz a product on the tensor
-// cores (FP32-grade as the others of the reverse mode), and full unitaries in one panel are read where
+// cores (FP32-grade as the others of the reverse mode; oz_ubar_applies), and full unitaries in one panel are read where
 // they are: 1390 -> 700 us for 450 items at d = 256, S = 256 (staging or slicing included).
 template <typename R>
 static cudaError_t ubar_launch(const BigArgs<R>& a, const StateView<R>& sv, const C_t<R>* states, const C_t<R>* Gbuf,
@@ -990,14 +990,15 @@ static cudaError_t ubar_launch(const BigArgs<R>& a, const StateView<R>& sv, cons
     using C = C_t<R>;
     const int d = a.d, items = a.wlen * a.E;
     const size_t ms = a.mstride, slice = sv.slice();
-    if (sizeof(C) == 8 && oz && sv.S == d && sv.cb == d)
+    const bool tc = sizeof(C) == 8 && oz && oz->ubar;
+    if (tc && sv.S == d && sv.cb == d)
         return oz_ubar(*oz, {Gbuf, slice, 0, 0, a.wmax * slice}, {states, slice, 1, 3, (a.wmax + 1) * slice}, a.wlen,
                        reinterpret_cast<float2*>(out), ms, st, launches);
     k_big_ubar_factors<C><<<dim3(ew_blocks((size_t)d * d), items), 256, 0, st>>>(d, sv, a.wlen, states, Gbuf, a.wmax, Zf, Xf, ms);
     if (launches) ++*launches;
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    if (sizeof(C) == 8 && oz)
+    if (tc)
         return oz_ubar(*oz, {Zf, ms, 0, 0}, {Xf, ms, 1, 1}, 0, reinterpret_cast<float2*>(out), ms, st, launches);
     err = mm_launch<C, 0>(d, items, Zf, Xf, out, ms, 1, 0, st);
     if (launches) ++*launches;

@@ -146,6 +146,7 @@ struct qoc_ctx {
     double theta_max = 0.0;              // in effect (the option, or the path's default)
     bool ps = false;                     // Paterson-Stockmeyer form of the per-slice FP32 exponential
     int nzmax = 0;                       // checkpoint segments per wave
+    bool oz_ubar = false;                // BF16_SPLIT: Ubar on the tensor cores (oz_ubar_applies)
     int state_cs = 0;                    // state mode: CTAs per cluster of the recursions (0: one CTA)
     std::vector<int> cols;               // propagated columns (positive weight)
     size_t mstride = 0;                  // elements per matrix slot of the batched path
@@ -334,29 +335,35 @@ void plan_impl(qoc_ctx* c) {
         }
         seg = best_seg;
     }
+    // norms of the propagated columns of the d x S block at `at` (scaled: their squares may leave the range)
+    auto col_norms = [&](const std::vector<double>& psi, size_t at = 0) {
+        std::vector<double> out;
+        for (int s : c->cols) {
+            double mx = 0.0, n2 = 0.0;
+            auto el = [&](int a, int q) { return psi[at + ((size_t)a * c->S + s) * 2 + q]; };
+            for (int a = 0; a < d; ++a) mx = std::max({mx, std::fabs(el(a, 0)), std::fabs(el(a, 1))});
+            for (int a = 0; a < d && mx > 0.0; ++a)
+                for (int q = 0; q < 2; ++q) n2 += (el(a, q) / mx) * (el(a, q) / mx);
+            out.push_back(mx * std::sqrt(n2));
+        }
+        return out;
+    };
+    const std::vector<double> norm0 = col_norms(c->psi0);
+    const auto range0 = std::minmax_element(norm0.begin(), norm0.end());
+    c->oz_ubar = oz_ubar_applies(*range0.first, *range0.second);
     // Full unitaries with a cost on the final state alone: both recursions as batched products over the
     // wave's tree, from d = 48 on (below, a chain step costs a few us and the tree's launches more).
     // The blocks are then one panel of all columns (row-major).
     c->tree = sizeof(R) == 4 && c->scan && S == d && d >= kTreeMinD && (c->nF == 0 || c->alpha[3] == 0.0) &&
               c->alpha[4] == 0.0;
     if (c->tree) {
-        auto grid_of = [&](const std::vector<double>& psi) {   // 2^e bounds the propagated columns' norms
-            double mx = 0.0;
-            for (int s : c->cols) {
-                double n2 = 0.0;
-                for (int a = 0; a < d; ++a)
-                    for (int q = 0; q < 2; ++q) {
-                        const double v = psi[((size_t)a * c->S + s) * 2 + q];
-                        n2 += v * v;
-                    }
-                mx = std::max(mx, n2);
-            }
-            const double b = 1.0625 * std::sqrt(mx);
+        auto grid_of = [&](const std::vector<double>& norms) {   // 2^e bounds the propagated columns' norms
+            const double b = 1.0625 * *std::max_element(norms.begin(), norms.end());
             const int e = b > 0.0 ? std::max(-100, std::min(100, (int)std::ceil(std::log2(b)))) : -100;
             return std::ldexp(1.5f, e + 11);
         };
-        c->tree_mo[0] = grid_of(c->psi0);
-        c->tree_mo[1] = grid_of(c->psiT);
+        c->tree_mo[0] = grid_of(norm0);
+        c->tree_mo[1] = grid_of(col_norms(c->psiT));
         cbw = S;
     }
     c->cb = std::min(cbw, S);
@@ -780,7 +787,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             if (big && big_rev && c->ps) {       // Paterson-Stockmeyer reverse mode (tensor cores: BF16_SPLIT)
                 int n_l = 0;
                 OzRev oz{c->opt.fault_inject, prm, d, E * wlen, E * W, c->tc_planes.as<unsigned char>(), c->tc_maps,
-                         nullptr, nullptr};
+                         nullptr, nullptr, c->oz_ubar};
                 cudaError_t e = launch_big_adj_rev_ps<R>(big_args(w), sys, sv, Sb(w), Gb(w), c->gpart.as<double>(), hp,
                                                          zbig(w), st, &n_l, use_oz(c) ? &oz : nullptr);
                 extra += n_l - 1;
@@ -789,7 +796,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             if (big && use_oz(c) && big_rev) {   // reverse mode, products on the tensor cores
                 int n_l = 0;
                 OzRev oz{c->opt.fault_inject, prm, d, E * wlen, E * W, c->tc_planes.as<unsigned char>(), c->tc_maps,
-                         nullptr, nullptr};
+                         nullptr, nullptr, c->oz_ubar};
                 cudaError_t e = launch_big_adj_rev<R>(big_args(w), sys, sv, Sb(w), Gb(w), c->gpart.as<double>(), hp.p,
                                                       hp.n, zbig(w), st, &n_l, &oz);
                 extra += n_l - 1;

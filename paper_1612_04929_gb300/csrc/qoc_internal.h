@@ -304,6 +304,7 @@ struct OzRev {
     TcMaps maps;            // oz_make_maps over the planes
     const float2* xh;       // X^dag of the wave (sliced once, into matrix 4)
     int* xh_sliced;         // host flag: X^dag already sliced for this wave
+    bool ubar = true;       // Ubar = G Psi^dag too (oz_ubar_applies)
 };
 size_t oz_plane_bytes(int d, int items);
 size_t oz_scratch_bytes(int d, int items);
@@ -317,6 +318,13 @@ cudaError_t launch_oz_mm(const OzJobs& jobs, int njobs, int d, int items, int ca
 cudaError_t oz_rev_step(const OzRev& z, const float2* const ops[4], const size_t strides[4], float2* O1, float2* O2,
                         size_t ms, int mode, int i, cudaStream_t st, int* launches);
 
+// Whether Ubar = G Psi^dag may be a product of slices: its operands are cut on one exponent per row, across
+// the propagated columns, so a column far below the row's largest loses its last bits in that operand.
+// With initial columns (whose norms the propagation keeps) within a factor of 8 of one another at least 25
+// of the 28 bits of each Psi_s are left, and a G_s that is cut short belongs to a small term of the sum.
+// Otherwise (Psi_s small where G_s is large) small factors of large terms are lost: at a ratio of 2^14 the
+// gradient's error was 2e-4, at 2^30 it was all wrong; those problems take the FP32 product.
+inline bool oz_ubar_applies(double min_norm, double max_norm) { return min_norm > 0.0 && max_norm <= 8.0 * min_norm; }
 // Ubar = A B of the operands that G and P describe (count items a member), into out
 cudaError_t oz_ubar(const OzRev& z, const OzSliceJob& G, const OzSliceJob& P, int count, float2* out, size_t ms,
                     cudaStream_t st, int* launches);
