@@ -301,56 +301,47 @@ cudaError_t launch_to_panels(const double2* src, C_t<R>* dst, int d, int S, Stat
 // them.  The FP64 pipe of this part runs at 1/64 of the FP32 rate: summing the FP32 form's
 // products in FP64 (about 16 FP64 instructions per element, conversions included) made them bound
 // by it.  Here a thread keeps one column of a panel (thread t: column t % cb, rows t / cb, t / cb +
-// ts / cb, ...; the addresses of a pass stay contiguous), sums the exact FP32 products as pairs
-// (pair_acc, about 2^-48), and takes the column's weight in FP64 once per run of equal weights.
-// With the terminal costs' rule (cost_is_terminal) an evaluation went, measured together on GB300:
-// d = 16, N = 2000 868 -> 681 us, d = 64, N = 2000 8.87 -> 7.13 ms, d = 128, N = 500 14.6 -> 11.7 ms,
-// d = 256, N = 2000 (BF16_SPLIT) 184 -> 157 ms; with C5 on (d = 27, E = 5) 1.58 -> 1.53 ms.
+// ts / cb, ...; the addresses of a pass stay contiguous), takes the column's weight in FP64 once per
+// run of equal weights, and the FP32 form sums its products without FP64 (RunSum<true>); the sources'
+// coefficients are set once per column and only the terms that act on an element are computed.
 // ------------------------------------------------------------------------------------------
-// running sum of real products: an FP32 pair in the FP32 form, FP64 in the FP64 form
-template <typename R> struct RunSum;
-template <> struct RunSum<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float a, float b) { pair_acc(hi, lo, a, b); }
-    __device__ __forceinline__ double take() {
-        const double v = (double)hi + (double)lo;
-        hi = lo = 0.f;
-        return v;
-    }
-};
-template <> struct RunSum<double> {
+// Running sum of real products, v += a b.  In FP64; or (FP32 values, TRI) over three floats: the product
+// and its rounding error are added error-free to the first two, what these round off to the third, so
+// a sum of n terms is off by about n^2 2^-72 of them, below FP64's n 2^-53 for the few hundred terms of a
+// thread (two floats: about 2^-48, 150 times FP64's error over 256 terms).  22 FP32 operations a product:
+// d = 128, S = 128, N = 500 took 142 us (two floats 113).  The exactness needs the product's error term to
+// be representable: cost_sums_fit; other norms are summed in FP64.
+template <bool TRI> struct RunSum {
     double v = 0.0;
-    __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
+    template <typename T> __device__ __forceinline__ void add(T a, T b) { v = fma((double)a, (double)b, v); }
     __device__ __forceinline__ double take() {
         const double r = v;
         v = 0.0;
         return r;
     }
 };
-
-// A real coefficient as the FP32 form multiplies it (an FP32 pair: the product with an FP32 value,
-// rounded once to FP32) or plain FP64
-template <typename R> struct Coef;
-template <> struct Coef<float> {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void set(double v) {
-        h = (float)v;
-        l = (float)(v - (double)h);
+template <> struct RunSum<true> {
+    float h = 0.f, m = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float a, float b) {
+        const float p = a * b, e = fmaf(a, b, -p);
+        float s, r, q;
+        two_sum(h, p, s, r);
+        h = s;
+        two_sum(m, r, s, q);
+        l += q;
+        two_sum(s, e, m, q);
+        l += q;
     }
-    // (hi, lo) += coefficient * x
-    __device__ __forceinline__ void mac(float& hi, float& lo, float x) const { pair_fma(hi, lo, make_float2(h, l), x, 0.f); }
-    __device__ __forceinline__ static float round(float hi, float lo) { return hi + lo; }
-};
-template <> struct Coef<double> {
-    double h = 0.0;
-    __device__ __forceinline__ void set(double v) { h = v; }
-    __device__ __forceinline__ void mac(double& hi, double&, double x) const { hi = fma(h, x, hi); }
-    __device__ __forceinline__ static double round(double hi, double) { return hi; }
+    __device__ __forceinline__ double take() {
+        const double v = (double)h + ((double)m + (double)l);
+        h = m = l = 0.f;
+        return v;
+    }
 };
 
 // WARP: one warp per slice (8 slices per block) for panels of at most 256 elements, with warp
 // shuffles for the sums; else one block per slice
-template <typename R, bool WARP>
+template <typename R, bool WARP, bool TRI>
 __global__ void __launch_bounds__(256)
 k_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, const C_t<R>* __restrict__ states, int wmax,
               CostView<R> cv, double2* __restrict__ Oj, double* __restrict__ C5j, double2* __restrict__ Ofin) {
@@ -366,7 +357,7 @@ k_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, const C_t<R>* __r
     const bool last = (j == N - 1), forb = cv.nF > 0;
     // panels wider than the threads (one panel of all columns) are walked in chunks of ts columns
     const int cw = cb < ts ? cb : ts, rows = ts / cw, a0 = t0 / cw, sc = t0 - a0 * cw;
-    RunSum<R> so[2], sf[2], s5;
+    RunSum<TRI> so[2], sf[2], s5;
     double ore = 0, oim = 0, c5 = 0, fre = 0, fim = 0, w = 0.0;
     auto flush = [&]() {
         ore = fma(w, so[0].take(), ore);
@@ -431,21 +422,29 @@ k_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, const C_t<R>* __r
     }
 }
 
+template <typename R, bool TRI>
+static void slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* states, int wmax,
+                        const CostView<R>& cv, double2* Oj, double* C5j, double2* Ofin, cudaStream_t st) {
+    if (sv.slice() <= 256)
+        k_slice_costs<R, true, TRI><<<dim3((wlen + 7) / 8, E), 256, 0, st>>>(d, sv, j0, wlen, N, states, wmax, cv, Oj,
+                                                                             C5j, Ofin);
+    else
+        k_slice_costs<R, false, TRI><<<dim3(wlen, E), 256, 0, st>>>(d, sv, j0, wlen, N, states, wmax, cv, Oj, C5j, Ofin);
+}
+
 template <typename R>
 cudaError_t launch_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* states, int wmax,
                                const CostView<R>& cv, double2* Oj, double* C5j, double2* Ofin, cudaStream_t st) {
-    if (sv.slice() <= 256)
-        k_slice_costs<R, true><<<dim3((wlen + 7) / 8, E), 256, 0, st>>>(d, sv, j0, wlen, N, states, wmax, cv, Oj,
-                                                                         C5j, Ofin);
-    else
-        k_slice_costs<R, false><<<dim3(wlen, E), 256, 0, st>>>(d, sv, j0, wlen, N, states, wmax, cv, Oj, C5j, Ofin);
+    if (sizeof(R) == 4 && cv.fit) slice_costs<R, sizeof(R) == 4>(d, sv, j0, wlen, N, E, states, wmax, cv, Oj, C5j, Ofin, st);
+    else slice_costs<R, false>(d, sv, j0, wlen, N, E, states, wmax, cv, Oj, C5j, Ofin, st);
     return cudaGetLastError();
 }
 
 template <typename R, bool WARP>
 __global__ void __launch_bounds__(256)
 k_sources(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* __restrict__ states, int wmax,
-          CostView<R> cv, const double2* __restrict__ Oj, const double2* __restrict__ Ofin, C_t<R>* __restrict__ src) {
+          CostView<R> cv, double ct, double cf, double c5, const double2* __restrict__ Oj,
+          const double2* __restrict__ Ofin, C_t<R>* __restrict__ src) {
     using C = C_t<R>;
     const int jl = WARP ? blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5) : blockIdx.x;
     if (WARP && jl >= wlen) return;
@@ -455,58 +454,64 @@ k_sources(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* 
     const C* psi = states + ((size_t)e * (wmax + 1) + jl + 1) * slice;
     const C* T = cv.path ? cv.path + (size_t)j * slice : cv.psiT;
     C* out = src + ((size_t)e * wmax + jl) * slice;
-    const double invE = 1.0 / E;
     const double2 o = Oj[(size_t)e * N + j];
     const bool last = (j == N - 1);
     const double2 of = last ? Ofin[e] : make_double2(0.0, 0.0);
-    // coefficient of T:  -(2 a67 / N) O_j w / W ;  of psiT at j = N: -2 a_fid O_N w / W
-    const double ct = -2.0 * cv.alpha[4] / N * invE / cv.Wsum;
-    const double cf = -2.0 * cv.alpha[0] * invE / cv.Wsum;
-    const double c5 = 2.0 * cv.alpha[3] * invE;
     const bool use_t = ct != 0.0, use_5 = cv.nF > 0 && c5 != 0.0;
     const int rows = ts / cb, a0 = t0 / cb, s0 = t0 - a0 * cb;
-    Coef<R> tx, ty, fx, fy, c5w;
-    double w = 0.0;
+    // Elements on which C5 alone acts, c5 w z: without FP64 in the FP32 form, the coefficient as a pair (the
+    // product is off by 2^-47 before it is rounded to FP32).  d = 27, N = 777, E = 5 took 37 us and d = 81,
+    // N = 1000 86 us; with every element and the coefficients' divisions here in FP64 82 and 133.
+    const bool c5_only = sizeof(R) == 4 && cv.fit && !use_t && !last;
     if (a0 < rows)
         for (int kb = 0; kb < sv.ncb; ++kb) {
-            const double wk = cv.w[kb * cb + s0];
-            if (wk != w) {
-                w = wk;
-                tx.set(ct * w * o.x);
-                ty.set(ct * w * o.y);
-                fx.set(cf * w * of.x);
-                fy.set(cf * w * of.y);
-                c5w.set(c5 * w);
+            const double w = cv.w[kb * cb + s0];
+            if constexpr (sizeof(R) == 4) {
+                const double cw = use_5 ? c5 * w : 0.0;
+                if (c5_only && (cw == 0.0 || (fabs(cw) >= 0x1p-40 && fabs(cw) <= 0x1p40))) {
+                    const float ch = (float)cw, cl = (float)(cw - (double)ch);
+#pragma unroll 4
+                    for (int a = a0; a < d; a += rows) {
+                        const size_t i = (size_t)kb * ps + s0 + (size_t)a * cb;
+                        C r = make_float2(0.f, 0.f);
+                        if (cw != 0.0 && cv.fmask[a]) {
+                            const C z = psi[i];
+                            r.x = ch * z.x;
+                            r.y = ch * z.y;
+                            r.x += fmaf(cl, z.x, fmaf(ch, z.x, -r.x));
+                            r.y += fmaf(cl, z.y, fmaf(ch, z.y, -r.y));
+                        }
+                        out[i] = r;
+                    }
+                    continue;
+                }
             }
+            const double tx = ct * w * o.x, ty = ct * w * o.y, fx = cf * w * of.x, fy = cf * w * of.y, c5w = c5 * w;
             const size_t base = (size_t)kb * ps + s0;
 #pragma unroll 4
             for (int a = a0; a < d; a += rows) {
                 const size_t i = base + (size_t)a * cb;
-                R xh = 0, xl = 0, yh = 0, yl = 0;
-                if (wk != 0.0) {
+                double vx = 0.0, vy = 0.0;
+                if (w != 0.0) {
                     if (use_t) {
                         const C t = T[i];
-                        tx.mac(xh, xl, t.x);
-                        ty.mac(xh, xl, -t.y);
-                        tx.mac(yh, yl, t.y);
-                        ty.mac(yh, yl, t.x);
+                        vx = tx * t.x - ty * t.y;
+                        vy = tx * t.y + ty * t.x;
                     }
                     if (use_5 && cv.fmask[a]) {
                         const C z = psi[i];
-                        c5w.mac(xh, xl, z.x);
-                        c5w.mac(yh, yl, z.y);
+                        vx += c5w * z.x;
+                        vy += c5w * z.y;
                     }
                     if (last) {
                         const C f = cv.psiT[i];
-                        fx.mac(xh, xl, f.x);
-                        fy.mac(xh, xl, -f.y);
-                        fx.mac(yh, yl, f.y);
-                        fy.mac(yh, yl, f.x);
+                        vx += fx * f.x - fy * f.y;
+                        vy += fx * f.y + fy * f.x;
                     }
                 }
                 C r;
-                r.x = Coef<R>::round(xh, xl);
-                r.y = Coef<R>::round(yh, yl);
+                r.x = (R)vx;
+                r.y = (R)vy;
                 out[i] = r;
             }
         }
@@ -523,11 +528,18 @@ template <typename R>
 cudaError_t launch_sources(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* states, int wmax,
                            const CostView<R>& cv, const double2* Oj, const double2* Ofin, C_t<R>* src,
                            cudaStream_t st) {
+    // coefficient of T:  -(2 a67 / N) O_j w / W ;  of psiT at j = N: -2 a_fid O_N w / W  (divided here: FP64
+    // divisions in every thread cost as much as the elements)
+    const double invE = 1.0 / E;
+    const double ct = -2.0 * cv.alpha[4] / N * invE / cv.Wsum;
+    const double cf = -2.0 * cv.alpha[0] * invE / cv.Wsum;
+    const double c5 = 2.0 * cv.alpha[3] * invE;
     if (sv.slice() <= 256)
-        k_sources<R, true><<<dim3((wlen + 7) / 8, E), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, Oj, Ofin,
-                                                                     src);
+        k_sources<R, true><<<dim3((wlen + 7) / 8, E), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, ct, cf, c5,
+                                                                    Oj, Ofin, src);
     else
-        k_sources<R, false><<<dim3(wlen, E), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, Oj, Ofin, src);
+        k_sources<R, false><<<dim3(wlen, E), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, ct, cf, c5, Oj, Ofin,
+                                                           src);
     return cudaGetLastError();
 }
 

@@ -146,6 +146,7 @@ struct qoc_ctx {
     double theta_max = 0.0;              // in effect (the option, or the path's default)
     bool ps = false;                     // Paterson-Stockmeyer form of the per-slice FP32 exponential
     int nzmax = 0;                       // checkpoint segments per wave
+    bool cost_fit = false;               // cost_sums_fit of every propagated column
     bool oz_ubar = false;                // BF16_SPLIT: Ubar on the tensor cores (oz_ubar_applies)
     int state_cs = 0;                    // state mode: CTAs per cluster of the recursions (0: one CTA)
     std::vector<int> cols;               // propagated columns (positive weight)
@@ -348,7 +349,13 @@ void plan_impl(qoc_ctx* c) {
         }
         return out;
     };
-    const std::vector<double> norm0 = col_norms(c->psi0);
+    const std::vector<double> norm0 = col_norms(c->psi0), normT = col_norms(c->psiT);
+    c->cost_fit = std::all_of(norm0.begin(), norm0.end(), cost_sums_fit) && std::all_of(normT.begin(), normT.end(), cost_sums_fit);
+    if (!c->path.empty())
+        for (int j = 0; j < N && c->cost_fit; ++j) {
+            const std::vector<double> n = col_norms(c->path, (size_t)j * d * c->S * 2);
+            c->cost_fit = std::all_of(n.begin(), n.end(), cost_sums_fit);
+        }
     const auto range0 = std::minmax_element(norm0.begin(), norm0.end());
     c->oz_ubar = oz_ubar_applies(*range0.first, *range0.second);
     // Full unitaries with a cost on the final state alone: both recursions as batched products over the
@@ -363,7 +370,7 @@ void plan_impl(qoc_ctx* c) {
             return std::ldexp(1.5f, e + 11);
         };
         c->tree_mo[0] = grid_of(norm0);
-        c->tree_mo[1] = grid_of(col_norms(c->psiT));
+        c->tree_mo[1] = grid_of(normT);
         cbw = S;
     }
     c->cb = std::min(cbw, S);
@@ -642,7 +649,8 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
                    c->delta.empty() ? nullptr : c->dDelta.as<double>(), u,
                    c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>()};
     CostView<R> cv{c->nF, c->fmask.as<int>(), c->colw.as<double>(), c->Wsum, c->psiTR.as<C>(),
-                   c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]}};
+                   c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]},
+                   c->cost_fit};
     DevParams* prm = c->prm.as<DevParams>();
     const int seg = c->seg;
     // A cost on the final state alone (gates, state transfer without C5 / C67) has one source, the
@@ -1170,7 +1178,8 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
                    c->delta.empty() ? nullptr : c->dDelta.as<double>(), u,
                    c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>()};
     CostView<R> cv{c->nF, c->fmask.as<int>(), c->colw.as<double>(), c->Wsum, c->psiTR.as<C>(),
-                   c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]}};
+                   c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]},
+                   c->cost_fit};
     DevParams* prm = c->prm.as<DevParams>();
     int launches = 0;
     const bool prof = c->opt.profile != 0;

@@ -59,7 +59,12 @@ struct CostView {
     const C_t<R>* psiT;     // final target, panel layout d x Spad
     const C_t<R>* path;     // N targets (panel layout) or nullptr
     double alpha[5];        // [fid, C3, C4, C5, C67]
+    bool fit = false;       // the norms are such that FP32 products may be summed without FP64 (cost_sums_fit)
 };
+// Products of two values of columns with these norms have FP32 rounding errors (relative to the norms'
+// product, above 2^-53 of it) that FP32 holds: 2^-80 2^-69 = 2^-149.  Zero columns add nothing.
+inline bool cost_sums_fit(double norm) { return norm == 0.0 || (norm >= 0x1p-40 && norm <= 0x1p40); }
+
 
 // ---- norms / (p, n) ----
 cudaError_t launch_norms(const double2* mats, int count, int d, double* norms, cudaStream_t st);
