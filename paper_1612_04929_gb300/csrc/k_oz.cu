@@ -378,7 +378,7 @@ struct OzFwdEpi {
 };
 
 struct OzAdjEpi {};
-// The tree's epilogue: out = A B grid-split with the magic mo (0: of the propagators' exponent), the
+// The tree's epilogue: out = A B grid-split with its columns' magics mo (none: of the propagators' exponent), the
 // optional second output and the optional rounded (scaled) value of TreeMm
 struct OzTreeEpi {
     TreeMm t;
@@ -627,14 +627,15 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
             } else if constexpr (std::is_same_v<Epi, OzTreeEpi>) {
                 const TreeMm& tm = fe.t;
                 const int it = fe.item0 + item, te = it / tm.count, ti = it - te * tm.count;
-                const float mo = tm.mo == 0.f ? grid_magic(prm->eu) : tm.mo;
+                const float mu = grid_magic(prm->eu);
                 const size_t o0 = (size_t)row * d + ch0;
 #pragma unroll
                 for (int q = 0; q < HC; ++q) {
                     const int e = __shfl_sync(0xffffffffu, eB[0], q);
                     if (row >= d || q >= ncols) continue;
                     const float sc = ldexpf(1.0f, eA + e - 3 * SBITS);
-                    tree_store(tm, te, ti, o0 + q, ch0 + q, make_float4(res[q].x * sc, res[q].y * sc, res[q].z * sc, res[q].w * sc), mo);
+                    tree_store(tm, te, ti, o0 + q, ch0 + q, make_float4(res[q].x * sc, res[q].y * sc, res[q].z * sc, res[q].w * sc),
+                               tm.mo ? tm.mo[ch0 + q] : mu);
                 }
             } else {
                 const size_t o0 = (size_t)item * fe.ostride + (size_t)row * d + ch0;

@@ -12,7 +12,7 @@
 // and the root takes the state (costate) across the whole wave: log2(W) launches a pass instead of a
 // scan and chains, each over all nodes of a level.  Nodes, states and costates are carried grid-split
 // (qoc_device.cuh; the U_j are unitary to the truncation, so products of them share the exponent eu,
-// and a block's columns keep the norms of Psi_0 or Psi_T), every product a split product (k_big_mm's
+// and a block's columns keep the norms of Psi_0 or Psi_T, each with a grid of its own), every product a split product (k_big_mm's
 // tiles, qoc_gemm.cuh).  The costate is propagated from Psi_T itself and scaled by the terminal
 // coefficient -2 a_fid O_N w_s / (E W) where G_j is written.
 // Measured on GB300 (evaluation): d = 128, N = 500 11.7 -> 8.3 ms; d = 64,
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(GemmSplit::NT, GemmSplit::MB) k_tree_mm(TreeMm
     const int e = item / t.count, i = item - e * t.count;
     const GemmPos<Sh> p(tile, t.tiles_c, t.d);
     const int d = t.d, cols = t.cols;
-    const float mu = grid_magic(t.prm->eu), mo = t.mo == 0.f ? mu : t.mo;
+    const float mu = grid_magic(t.prm->eu);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     const float4* A4 = static_cast<const float4*>(t.a) + e * t.ae + i * t.ai;
     const float2* A2 = static_cast<const float2*>(t.a) + e * t.ae + i * t.ai;
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(GemmSplit::NT, GemmSplit::MB) k_tree_mm(TreeMm
             two_sum(mac.acc[x][y][0], mac.acc[x][y][2], v.x, v.z);
             two_sum(mac.acc[x][y][1], mac.acc[x][y][3], v.y, v.w);
             const size_t o = (size_t)r * cols + c;
-            tree_store(t, e, i, o, c, v, mo);
+            tree_store(t, e, i, o, c, v, t.mo ? t.mo[c] : mu);
         }
 }
 
@@ -129,13 +129,13 @@ __global__ void k_tree_tail(const void* src, size_t se, int leaf, float4* dst, s
     }
 }
 
-// The block a pass starts from (pairs), split on the pass's grid, and its rounded (scaled) value
+// The block a pass starts from (pairs), split on its columns' grids, and its rounded (scaled) value
 __global__ void k_tree_init(const float4* src, size_t se, float4* dst, size_t de, float2* rnd, size_t re,
-                            const float4* coef, int cols, size_t n, float m) {
+                            const float4* coef, int cols, size_t n, const float* __restrict__ mo) {
     const int e = blockIdx.y;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float4 v = src[e * se + i];
-        dst[e * de + i] = tree_split(v, m);
+        dst[e * de + i] = tree_split(v, mo[i % cols]);
         float2 r = make_float2(v.x + v.z, v.y + v.w);
         if (coef) {
             const float4 q = coef[(size_t)e * cols + i % cols];
@@ -249,7 +249,7 @@ cudaError_t launch_tree_up(const TreeArgs& a, cudaStream_t st, int* launches) {
 }
 
 cudaError_t launch_tree_forward(const TreeArgs& a, const float4* start, size_t start_e, float4* next, size_t next_e,
-                                float2* states, size_t states_e, float mo, cudaStream_t st, int* launches) {
+                                float2* states, size_t states_e, const float* mo, cudaStream_t st, int* launches) {
     const int L = tree_levels(a.wlen);
     const size_t n = (size_t)a.d * a.S, ce = (size_t)(a.W + 1) * a.slice;
     cudaError_t err;
@@ -297,7 +297,7 @@ cudaError_t launch_tree_coef(const CostView<float>& cv, int E, int S, const doub
 }
 
 cudaError_t launch_tree_costate(const TreeArgs& a, const float4* start, size_t start_e, float4* next, size_t next_e,
-                                float2* G, size_t G_e, const float4* coef, float mo, cudaStream_t st, int* launches) {
+                                float2* G, size_t G_e, const float4* coef, const float* mo, cudaStream_t st, int* launches) {
     const int L = tree_levels(a.wlen);
     const size_t n = (size_t)a.d * a.S, ce = (size_t)(a.W + 1) * a.slice;
     cudaError_t err;

@@ -142,7 +142,6 @@ struct qoc_ctx {
     int Spad = 0, cb = 0, ncb = 0, pstride = 0, S_eff = 0;
     bool scan = false;                   // segmented-scan form of the two recursions
     bool tree = false;                   // both recursions over the wave's binary tree (k_tree.cu)
-    float tree_mo[2] = {0.f, 0.f};       // its grids: of the states (norms of Psi_0), of the costates (Psi_T)
     double theta_max = 0.0;              // in effect (the option, or the path's default)
     bool ps = false;                     // Paterson-Stockmeyer form of the per-slice FP32 exponential
     int nzmax = 0;                       // checkpoint segments per wave
@@ -162,6 +161,7 @@ struct qoc_ctx {
     TcMaps tree_maps;
     int tree_cap = 0;                    // items they hold (0: the products run on the FP32 pipes)
     DevBuf tnodes, tcarry, tcoef, tgtK;  // tree form: nodes (two wave sets), carried blocks, coefficients, Psi_T
+    DevBuf tmo;                          // its columns' grids: of the states (norms of Psi_0), of the costates (Psi_T)
     DevBuf hoff, hidx, hval;             // the controls' non-zero elements (SysView), when sparse
     DevBuf sH;                           // s H_0 .. s H_det as FP32 pairs (per-slice split exponential)
     DevBuf chebd;                        // Chebyshev coefficients of the evaluation (state mode)
@@ -195,7 +195,7 @@ struct qoc_ctx {
         const DevBuf* all[] = {&H64, &HR, &dDelta, &norms, &psiTR, &pathR, &fmask, &colw, &ckpt, &Ubuf, &states,
                                &Gbuf, &src, &carry, &Oj, &C5j, &Ofin, &gpart, &prm, &u_h, &grad_h, &out_h, &scratch,
                                &tc_planes, &Pbuf, &lv0, &lv1, &scanst, &hbuf, &Ybuf, &Zbuf, &Zbig, &sH, &chebd, &stscr, &hoff, &hidx, &hval,
-                               &tplanes, &tnodes, &tcarry, &tcoef, &tgtK,
+                               &tplanes, &tnodes, &tcarry, &tcoef, &tgtK, &tmo,
                                &frozen_d};
         size_t s = 0;
         for (auto* b : all) s += b->bytes;
@@ -363,14 +363,13 @@ void plan_impl(qoc_ctx* c) {
     // The blocks are then one panel of all columns (row-major).
     c->tree = sizeof(R) == 4 && c->scan && S == d && d >= kTreeMinD && (c->nF == 0 || c->alpha[3] == 0.0) &&
               c->alpha[4] == 0.0;
+    std::vector<float> tree_mo;   // grids of the states' columns, then of the costates': 2^e bounds the norm
     if (c->tree) {
-        auto grid_of = [&](const std::vector<double>& norms) {   // 2^e bounds the propagated columns' norms
-            const double b = 1.0625 * *std::max_element(norms.begin(), norms.end());
-            const int e = b > 0.0 ? std::max(-100, std::min(100, (int)std::ceil(std::log2(b)))) : -100;
-            return std::ldexp(1.5f, e + 11);
-        };
-        c->tree_mo[0] = grid_of(norm0);
-        c->tree_mo[1] = grid_of(normT);
+        for (const auto* norms : {&norm0, &normT})
+            for (double x : *norms) {
+                const int e = x > 0.0 ? std::max(-100, std::min(100, (int)std::ceil(std::log2(1.0625 * x)))) : -100;
+                tree_mo.push_back(std::ldexp(1.5f, e + 11));
+            }
         cbw = S;
     }
     c->cb = std::min(cbw, S);
@@ -577,11 +576,13 @@ void plan_impl(qoc_ctx* c) {
         A(c->tcarry, (size_t)E * (W + 1) * slice * sizeof(float4), "alloc tree blocks");
         A(c->tcoef, (size_t)E * S * sizeof(float4), "alloc tree coefficients");
         A(c->tgtK, slice * sizeof(K_t<R>), "alloc carried target");
+        A(c->tmo, tree_mo.size() * sizeof(float), "alloc column grids");
+        check_cuda(c, cudaMemcpyAsync(c->tmo.p, tree_mo.data(), c->tmo.bytes, cudaMemcpyHostToDevice, st), "copy column grids");
         check_cuda(c, cudaStreamSynchronize(st), "sync");
         check_cuda(c, cudaMemcpyAsync(stage.p, psiTp.data(), blk, cudaMemcpyHostToDevice, st), "copy target");
         check_cuda(c, launch_to_carry<R>(stage.as<double2>(), c->tgtK.as<K_t<R>>(), d, S, sv, 1, slice, st), "carried target");
     } else {
-        for (DevBuf* b : {&c->tnodes, &c->tcarry, &c->tcoef, &c->tgtK}) b->release();
+        for (DevBuf* b : {&c->tnodes, &c->tcarry, &c->tcoef, &c->tgtK, &c->tmo}) b->release();
     }
     c->tree_cap = 0;
     if (c->tree && use_oz(c) && d >= kOzFwdMinD && d <= kOzFwdMaxD) {
@@ -885,7 +886,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             B(sx);
             const bool next = hand_on && w + 1 < nw;
             e = launch_tree_forward(targs(w), ck(w), ck_e, next ? ck(w + 1) : nullptr, ck_e, Sb(w), (size_t)(W + 1) * slice,
-                                    c->tree_mo[0], sx, &n_l);
+                                    c->tmo.as<float>(), sx, &n_l);
             L(e, "chain (replay)", sx);
             extra += n_l - 1;
         };
@@ -914,7 +915,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             B(sx);
             const cudaError_t e = launch_tree_costate(targs(w), w == nw - 1 ? c->tgtK.as<float4>() : c->carry.as<float4>(),
                                                       w == nw - 1 ? 0 : slice, w > 0 ? c->carry.as<float4>() : nullptr, slice,
-                                                      Gb(w), (size_t)W * slice, c->tcoef.as<float4>(), c->tree_mo[1], sx, &n_l);
+                                                      Gb(w), (size_t)W * slice, c->tcoef.as<float4>(), c->tmo.as<float>() + sv.S, sx, &n_l);
             L(e, "costate (final)", sx);
             extra += n_l - 1;
             rec(ev_cost[w], sx);

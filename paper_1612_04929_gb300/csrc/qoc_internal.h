@@ -516,14 +516,15 @@ constexpr int kTreeMinD = 48;
 int tree_levels(int wlen);
 size_t tree_nodes(int W);   // per member
 cudaError_t launch_tree_up(const TreeArgs& a, cudaStream_t st, int* launches);
-// states Psi_0 .. Psi_wlen of the wave (rounded) from its first block (pairs); the last one also to next
+// states Psi_0 .. Psi_wlen of the wave (rounded) from its first block (pairs); the last one also to next;
+// mo: the grid (magic) of every column
 cudaError_t launch_tree_forward(const TreeArgs& a, const float4* start, size_t start_e, float4* next, size_t next_e,
-                                float2* states, size_t states_e, float mo, cudaStream_t st, int* launches);
+                                float2* states, size_t states_e, const float* mo, cudaStream_t st, int* launches);
 cudaError_t launch_tree_coef(const CostView<float>& cv, int E, int S, const double2* Ofin, float4* coef, cudaStream_t st);
 // costates G_1 .. G_wlen (block j - 1 of G), coef times the block propagated from start; the block below
 // the wave's first slice to next (or nullptr)
 cudaError_t launch_tree_costate(const TreeArgs& a, const float4* start, size_t start_e, float4* next, size_t next_e,
-                                float2* G, size_t G_e, const float4* coef, float mo, cudaStream_t st, int* launches);
+                                float2* G, size_t G_e, const float4* coef, const float* mo, cudaStream_t st, int* launches);
 
 // ---- per-slice costs, sources, final reduction (k_chain.cu) ----
 template <typename R>

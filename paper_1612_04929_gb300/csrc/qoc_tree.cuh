@@ -20,15 +20,15 @@ struct TreeMm {
     size_t ae, ai;
     const void* b;
     size_t be, bi;
-    float4* out;              // grid-split with mo
+    float4* out;              // grid-split with its column's mo
     size_t oe, oi;
     float4* copy;             // optional second carried output (the block handed to the next wave)
     size_t ce;
     float2* round;            // optional rounded output: states, or costates scaled by coef
     size_t re, ri;
     const float4* coef;       // per member and column (re, im hi; re, im lo), or nullptr
-    float mo;
-    const DevParams* prm;     // exponent eu of the propagators (and of out when mo is 0)
+    const float* mo;          // grid (magic) of every output column; nullptr: of the propagators' exponent
+    const DevParams* prm;     // exponent eu of the propagators (and of out without mo)
 };
 
 // element o (column c) of item (e, i): the carried output, its copy and the rounded (scaled) value
