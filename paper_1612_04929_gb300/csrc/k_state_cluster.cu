@@ -2,7 +2,7 @@
 //
 // One trajectory is a chain of matrix-vector products with X_j (p 2^n of them a slice for Taylor, K
 // for Chebyshev; see k_state.cu for the map, its adjoint and its arithmetic, which are the same
-// here).  On one CTA a product of a d = 154 system took 8.5 us, bound by that SM's issue rate and by
+// here but for the grids of Chebyshev's vectors).  On one CTA a product of a d = 154 system took 8.5 us, bound by that SM's issue rate and by
 // the barriers and shared-memory passes between products, while the other SMs had no work.  Here a
 // cluster of CS CTAs owns the trajectory, each CTA d / CS rows of X_j and a warp RW rows:
 //   * a warp keeps its rows of X_j in registers for all the products of the slice (RW x QB elements
@@ -12,12 +12,17 @@
 //     bytes complete a transaction on that CTA's mbarrier: one message a product, no other barrier.
 //     Two buffers alternate: a CTA sends message m + 2 only after it has all of message m + 1, which
 //     every warp of the cluster sends after it has read message m;
-//   * the FP32 form's grid is set once per application of the series: the vector that starts it arrives
-//     as pairs, and every warp takes its largest component and splits it in registers; the later
-//     vectors of the application are bounded by it (|phi_k| <= |v| for Chebyshev, |z| <= e^ts |v| for
-//     Taylor), so their owners send them already split.
+//   * the FP32 form splits a vector before a product on the grid of its largest component: it arrives as
+//     pairs, and every warp takes that component and splits the vector in registers.  Chebyshev's later
+//     vectors keep the grid of the one that starts the application (|phi_k| <= |v|, which that grid
+//     bounds), so their owners send them already split.  Taylor's Z_i may be e^(ts) |v|, whose grid
+//     would take up to 2 bits of the exact leading part at a norm of 1 a slice and all of it at 8, so each takes
+//     a grid of its own.
+//     Cost error against 64 bits, d = 154, N = 1000, E = 2, Chebyshev: 5.96e-9 and 3.72e-9 (two problems)
+//     with the sender's split, 5.91e-9 and 3.70e-9 with a grid per product, 5.90e-9 and 3.74e-9 in
+//     k_state_chain; d = 88, N = 600, E = 4: 1.70e-7 and 1.72e-7 in all three.
 // Bound: the latency of one message and of the dependent arithmetic of one product: at d = 154 0.76 us
-// on 16 CTAs, 0.97 on 8, 1.31 on 4 (before the split moved to the sender 0.83, 1.02, 1.41; with plain
+// on 16 CTAs, 0.97 on 8, 1.31 on 4 (with a grid per product, as Taylor has it, 0.83, 1.02, 1.41; with plain
 // remote stores and a cluster barrier per product instead of st.async 1.2 on 8).  d = 154, N = 1000,
 // K = 14, 16 members: a recursion went from 119 to 14 ms; one member: from 119 to 10.5 ms.
 // Every mbarrier wait is bounded; one that runs out sets kErrTimeout and its warp leaves the loop, the
@@ -221,11 +226,10 @@ __global__ void __launch_bounds__(sc_max_warps(RW) * 32) k_state_cluster(StateCh
         load(xc, 0);
         if (nmv > 0) send(v);
     }
-    // y = X b for the message that arrives next: this lane's row.  first: the message is the vector that
-    // starts an application, in pairs; it sets the grid of the later ones, ex2 powers of two coarser
+    // y = X b for the message that arrives next: this lane's row.  pairs: the message is a vector of pairs,
+    // split here on the grid of its largest component, which becomes mgrid
     float mgrid = 0.f;
-    const int ex2 = cheb ? 0 : A.prm->ez;
-    auto product = [&](bool first) -> K {
+    auto product = [&](bool pairs) -> K {
         const uint32_t b = got & 1;
         if (ok) ok = __all_sync(0xffffffffu, sc_wait(sc_su32(&bars[b]), (got >> 1) & 1));
         if (tid == 0) sc_expect(sc_su32(&bars[b]), bytes);   // message got + 2
@@ -235,16 +239,14 @@ __global__ void __launch_bounds__(sc_max_warps(RW) * 32) k_state_cluster(StateCh
         for (int q = 0; q < QB; ++q) zq[q] = zbuf[b][q * 32 + lane];
         ScAcc<R> acc[RW];
         if constexpr (sizeof(R) == 4) {
-            if (first) {
+            if (pairs) {
                 unsigned mb = 0u;
 #pragma unroll
                 for (int q = 0; q < QB; ++q) mb = max(mb, st_maxbits(zq[q]));
                 mb = __reduce_max_sync(0xffffffffu, mb);
-                const int ev = sc_exp(mb, cmag);
-                const float mx = sc_magic(ev);
-                mgrid = sc_magic(max(-100, min(100, ev + ex2)));
+                mgrid = sc_magic(sc_exp(mb, cmag));
 #pragma unroll
-                for (int q = 0; q < QB; ++q) zq[q] = sc_split(zq[q], mx);
+                for (int q = 0; q < QB; ++q) zq[q] = sc_split(zq[q], mgrid);
             }
 #pragma unroll
             for (int q = 0; q < QB; ++q)
@@ -307,16 +309,12 @@ __global__ void __launch_bounds__(sc_max_warps(RW) * 32) k_state_cluster(StateCh
                     const bool final_app = m + 1 == (1 << n);
 #pragma unroll 1
                     for (int i = p; i >= 1; --i) {
-                        K w = product(i == p);
+                        K w = product(true);
                         if (!fwd) st_kneg(w);          // T(X^dag) = T(-X)
                         st_kdiv(w, i);
                         st_kadd(w, v);                 // z = v + y / i
-                        if (i > 1) {
-                            send(sc_split(w, mgrid));
-                        } else {
-                            v = w;
-                            if (!final_app) send(v);
-                        }
+                        if (i == 1) v = w;
+                        if (i > 1 || !final_app) send(w);
                     }
                 }
             } else {
