@@ -703,12 +703,8 @@ template <typename C, int T>
 static cudaError_t blk_launch_t(int d, int items, const C* A11, const C* A12, const C* B11, const C* B12, C* O11,
                                 C* O12, size_t ms, int kind, int i, cudaStream_t st) {
     constexpr size_t smem = blk_smem<C, T>();
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_big_mm_blk<C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    cudaError_t e = cudaFuncSetAttribute(k_big_mm_blk<C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   // of each device
+    if (e != cudaSuccess) return e;
     const int nt = ((d + T - 1) / T) * ((d + T - 1) / T);
     k_big_mm_blk<C, T><<<dim3(nt, items), 256, smem, st>>>(d, A11, A12, B11, B12, O11, O12, ms, kind, i);
     return cudaGetLastError();

@@ -746,12 +746,8 @@ static cudaError_t slice_launch(const OzSliceJobs& jobs, int njobs, int d, int i
 template <class Cfg, class Epi>
 static cudaError_t mm_launch(const OzJobs& jobs, int njobs, const Epi& fe, int d, int items, int cap,
                              unsigned char* scratch, const TcMaps& maps, DevParams* prm, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_oz_mm<Cfg, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    cudaError_t e = cudaFuncSetAttribute(k_oz_mm<Cfg, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);   // of each device
+    if (e != cudaSuccess) return e;
     if (njobs < 1 || njobs > 2 || d > kMaxD || items > cap) return cudaErrorInvalidValue;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||

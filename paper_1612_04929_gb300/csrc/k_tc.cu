@@ -405,12 +405,8 @@ cudaError_t tc_make_maps(float* planes, int d, int items, TcMaps* maps) {
 }
 
 cudaError_t launch_tc_adj(const TcAdjArgs& a, cudaStream_t st, int* launches) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_tc_step, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    cudaError_t e = cudaFuncSetAttribute(k_tc_step, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);   // of each device
+    if (e != cudaSuccess) return e;
     auto count = [&]() { if (launches) ++*launches; };
     const int d = a.d, items = a.wlen * a.E, ld = tc_ld(d);
     TcMats m{0, 1, 2, 3, 4, 5};        // XH, Ubar, Z11 (row, col), Z12 (row, col) of set 0

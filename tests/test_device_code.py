@@ -1,5 +1,5 @@
 """Rules of the CUDA sources that no run on one GPU can show broken: convergence before warp-aligned
-instructions."""
+instructions, and launch attributes on every device."""
 import glob
 import os
 import re
@@ -23,3 +23,12 @@ def test_cluster_barriers_follow_a_warp_reconvergence():
             assert before.endswith("__syncwarp();"), (name, text[m.start() - 200:m.end()])
             found += 1
     assert found >= 1
+
+
+def test_launch_attributes_are_set_on_every_device():
+    """cudaFuncSetAttribute acts on the current device only; a flag kept by the process would leave a context
+    on another device without it, and is written by several host threads at once."""
+    for name, text in sources():
+        text = re.sub(r"//[^\n]*", "", text)
+        flags = [m.group(0) for m in re.finditer(r"\bstatic\s+(?!constexpr|const\b)(?:bool|int|std::once_flag|std::atomic<\w+>)\s+\w+\s*(?:=|;|\{)", text)]
+        assert not flags, (name, flags)
