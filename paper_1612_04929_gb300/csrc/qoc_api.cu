@@ -315,8 +315,7 @@ void plan_impl(qoc_ctx* c) {
         // costate's two segment passes; two for a terminal cost, which has no zero-carry pass), each running in whole rounds of resident CTAs, and two
         // scans of `nseg` steps (one CTA per panel); a CTA step costs col_cost(panel width).
         const long wave = ((long)N + 1) / 2;
-        const bool terminal = (c->nF == 0 || c->alpha[3] == 0.0) && c->alpha[4] == 0.0;
-        const double passes = terminal ? 2.0 : 3.0;
+        const double passes = cost_is_terminal(c->nF, c->alpha) ? 2.0 : 3.0;
         double best = -1.0;
         int best_seg = seg;
         const int lo = std::max(4, (int)std::sqrt((double)N) / 2), hi = std::min(N, 2 * (int)std::ceil(std::sqrt((double)N)));
@@ -358,11 +357,12 @@ void plan_impl(qoc_ctx* c) {
         }
     const auto range0 = std::minmax_element(norm0.begin(), norm0.end());
     c->oz_ubar = oz_ubar_applies(*range0.first, *range0.second);
+    const bool terminal = cost_is_terminal(c->nF, c->alpha);
+    const bool sources = state_mode || !terminal;   // a terminal cost has no source but the carried block
     // Full unitaries with a cost on the final state alone: both recursions as batched products over the
     // wave's tree, from d = 48 on (below, a chain step costs a few us and the tree's launches more).
     // The blocks are then one panel of all columns (row-major).
-    c->tree = sizeof(R) == 4 && c->scan && S == d && d >= kTreeMinD && (c->nF == 0 || c->alpha[3] == 0.0) &&
-              c->alpha[4] == 0.0;
+    c->tree = sizeof(R) == 4 && c->scan && S == d && d >= kTreeMinD && terminal;
     std::vector<float> tree_mo;   // grids of the states' columns, then of the costates': 2^e bounds the norm
     if (c->tree) {
         for (const auto* norms : {&norm0, &normT})
@@ -387,11 +387,13 @@ void plan_impl(qoc_ctx* c) {
     // evolution when both sets fit a memory budget (1/8 of the free device memory, between 1 and
     // 32 GiB), else the largest wave that fits.
     int W = 0;
+    const bool oz_tree = c->tree && use_oz(c) && d >= kOzFwdMinD && d <= kOzFwdMaxD;
+    int tree_items = (int)std::min<long long>((long long)E * (((long long)N + 1) / 2 + seg), kOzTreeItems);
     if (c->opt.wave_slices > 0) {
         W = ((c->opt.wave_slices + seg - 1) / seg) * seg;
     } else {
         const size_t dd0 = (size_t)d * d, ks = sizeof(K_t<R>);
-        size_t per = 2 * ((size_t)c->ustride * cs + 3 * slice * cs);          // U, states, G, sources
+        size_t per = 2 * ((size_t)c->ustride * cs + (sources ? 3 : 2) * slice * cs);   // U, states, G, sources
         if (c->path_kind == 1) per += big_scratch_per_item(d, sizeof(R) == 8, c->ps);
         if (use_tc(c)) per += tc_scratch_floats(d, 1) * sizeof(float);
         if (use_oz(c)) per += std::max(oz_scratch_bytes(d, 1), oz_fwd_on(c) ? oz_fwd_scratch_bytes(d, 1) : 0);
@@ -402,7 +404,13 @@ void plan_impl(qoc_ctx* c) {
         per *= (size_t)E;
         size_t free_b = 0, total_b = 0;
         if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = (size_t)8 << 30;
-        const size_t budget = std::min<size_t>((size_t)32 << 30, std::max<size_t>((size_t)1 << 30, free_b / 8));
+        size_t budget = std::min<size_t>((size_t)32 << 30, std::max<size_t>((size_t)1 << 30, free_b / 8));
+        // the tree's tensor-core planes are as many for any wave but the shortest: at most an eighth of it
+        if (oz_tree) {
+            const size_t one = oz_tree_scratch_bytes(d, 1);
+            tree_items = (int)std::min<size_t>(tree_items, std::max<size_t>(1, budget / 8 / one));
+            budget -= std::min(budget, tree_items * one);
+        }
         const long long w_mem = std::max<long long>(seg, (long long)(budget / std::max<size_t>(per, 1)) / seg * seg);
         const long long w_half = (((long long)N + 1) / 2 + seg - 1) / seg * seg;
         W = (int)std::min<long long>(w_half, w_mem);
@@ -542,7 +550,8 @@ void plan_impl(qoc_ctx* c) {
     A(c->Ubuf, 2 * (size_t)E * W * c->ustride * cs, "alloc U");
     A(c->states, 2 * (size_t)E * (W + 1) * slice * cs, "alloc states");
     A(c->Gbuf, 2 * (size_t)E * W * slice * cs, "alloc costates");
-    A(c->src, 2 * (size_t)E * W * slice * cs, "alloc sources");
+    if (sources) A(c->src, 2 * (size_t)E * W * slice * cs, "alloc sources");
+    else c->src.release();
     if (c->path_kind == 1) {
         c->mstride = (((size_t)d * d + 15) / 16) * 16;
         const size_t per = big_scratch_per_item(d, sizeof(R) == 8, c->ps) / ((size_t)d * d) * c->mstride;
@@ -585,8 +594,8 @@ void plan_impl(qoc_ctx* c) {
         for (DevBuf* b : {&c->tnodes, &c->tcarry, &c->tcoef, &c->tgtK, &c->tmo}) b->release();
     }
     c->tree_cap = 0;
-    if (c->tree && use_oz(c) && d >= kOzFwdMinD && d <= kOzFwdMaxD) {
-        c->tree_cap = std::min(E * (W / 2 + 1), kOzTreeItems);
+    if (oz_tree) {
+        c->tree_cap = std::min(E * (W / 2 + 1), tree_items);
         A(c->tplanes, oz_tree_scratch_bytes(d, c->tree_cap), "alloc tree slices");
         check_cuda(c, oz_tree_make_maps(c->tplanes.p, d, c->tree_cap, &c->tree_maps), "tensor maps");
     } else {
@@ -657,7 +666,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
     // A cost on the final state alone (gates, state transfer without C5 / C67) has one source, the
     // terminal block: no source kernel, and in the segmented form no zero-carry pass over the
     // segments (their h_z is zero), a fourth of the backward sweeps' work at S = d.
-    const bool terminal = cost_is_terminal(cv);
+    const bool terminal = cost_is_terminal(c->nF, c->alpha);
     // two sets of wave buffers: wave w uses set w % 2, so the serial sweep of one wave overlaps
     // the parallel kernels of its neighbour
     const size_t u_set = (size_t)E * W * c->ustride, s_set = (size_t)E * (W + 1) * slice, g_set = (size_t)E * W * slice;

@@ -537,10 +537,7 @@ cudaError_t launch_sources(int d, StateView<R> sv, int j0, int wlen, int N, int 
                            C_t<R>* src, cudaStream_t st);
 // No cost term acts on the states of slices 1 .. N - 1 (no weight on C5 and C67): every source but
 // the last slice's is zero, so the costate is G_{j-1} = U_j^dag G_j from the terminal block alone
-template <typename R>
-inline bool cost_is_terminal(const CostView<R>& cv) {
-    return (cv.nF == 0 || cv.alpha[3] == 0.0) && cv.alpha[4] == 0.0;
-}
+inline bool cost_is_terminal(int nF, const double* alpha) { return (nF == 0 || alpha[3] == 0.0) && alpha[4] == 0.0; }
 template <typename R>
 cudaError_t launch_terminal(int d, StateView<R> sv, int E, const CostView<R>& cv, const double2* Ofin, K_t<R>* out,
                             cudaStream_t st);
