@@ -1413,7 +1413,8 @@ void autotune(qoc_ctx* c, const double* u, double* grad, double* out) {
     const int wave_user = o.wave_slices;
     const std::vector<long long> key = {o.precision, c->d, c->N, c->M, c->S_eff, c->E, o.gradient, o.adjoint,
                                         o.taylor_scheme, o.sweep, c->theta_user ? (long long)(o.theta_max * 1e9) : -1,
-                                        o.plain_fp32_exp, o.reversal, wave_user, o.ckpt_stride};
+                                        o.plain_fp32_exp, o.reversal, wave_user, o.ckpt_stride,
+                                        cost_is_terminal(c->nF, c->alpha)};   // decides the recursions that run
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
