@@ -501,19 +501,40 @@ k_big_grad(const DevParams* __restrict__ prm, SysView<R> sys, int j0, int wlen, 
     if (threadIdx.x == 0) gpart[((size_t)e * sys.M + k) * sys.N + j] = prm->s * v;
 }
 
-// the same over the controls' non-zero elements, one CTA per item, a warp per control
-template <typename R>
+// the same over the controls' non-zero elements: one CTA per item and a warp per control, or (GROUPS) a CTA
+// per item and control, whose warps share the control's elements.  A Pauli or ladder control of d = 128
+// takes 6 us a launch of 250 items with a warp each; at a quarter of the elements a warp has thousands
+// one after another, and the dense contraction was faster (d = 256, M = 16, N = 60 5.8 against 5.5 ms an
+// evaluation, d = 512, M = 1 15.2 against 14.8): GSP_GROUPS
+template <typename R, bool GROUPS>
 __global__ void __launch_bounds__(256)
 k_big_grad_sparse(const DevParams* __restrict__ prm, SysView<R> sys, int j0, int wlen, const C_t<R>* __restrict__ Xbar,
                   size_t mstride, double* __restrict__ gpart) {
     const int item = blockIdx.x, jl = item % wlen, e = item / wlen;
     const C_t<R>* xb = Xbar + (size_t)item * mstride;
-    contract_sparse<R>(sys, prm, gpart, e, j0 + jl, [&](int a, int b) { return xb[(size_t)a * sys.d + b]; });
+    auto at = [&](int a, int b) { return xb[(size_t)a * sys.d + b]; };
+    if constexpr (!GROUPS) {
+        contract_sparse<R>(sys, prm, gpart, e, j0 + jl, at);
+    } else {
+        __shared__ double part[8];
+        const int k = blockIdx.y;
+        const double v = sparse_sum(sys, k, (int)threadIdx.x, 256, at);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < 8; ++w) s += part[w];
+            gpart[((size_t)e * sys.M + k) * sys.N + j0 + jl] = prm->s * s;
+        }
+    }
 }
+constexpr int GSP_GROUPS = 1024;   // elements of the largest control: 32 a lane of a warp
 template <typename R>
 static cudaError_t grad_launch(const DevParams* prm, const SysView<R>& sys, int j0, int wlen, int items,
                                const C_t<R>* Xbar, size_t ms, double* gpart, cudaStream_t st) {
-    if (sys.hoff) k_big_grad_sparse<R><<<items, 256, 0, st>>>(prm, sys, j0, wlen, Xbar, ms, gpart);
+    if (sys.hoff && sys.hmax > GSP_GROUPS)
+        k_big_grad_sparse<R, true><<<dim3(items, sys.M), 256, 0, st>>>(prm, sys, j0, wlen, Xbar, ms, gpart);
+    else if (sys.hoff) k_big_grad_sparse<R, false><<<items, 256, 0, st>>>(prm, sys, j0, wlen, Xbar, ms, gpart);
     else k_big_grad<R><<<dim3(items, sys.M), 256, 0, st>>>(prm, sys, j0, wlen, Xbar, ms, gpart);
     return cudaGetLastError();
 }

@@ -163,6 +163,7 @@ struct qoc_ctx {
     DevBuf tnodes, tcarry, tcoef, tgtK;  // tree form: nodes (two wave sets), carried blocks, coefficients, Psi_T
     DevBuf tmo;                          // its columns' grids: of the states (norms of Psi_0), of the costates (Psi_T)
     DevBuf hoff, hidx, hval;             // the controls' non-zero elements (SysView), when sparse
+    int hmax = 0;
     DevBuf sH;                           // s H_0 .. s H_det as FP32 pairs (per-slice split exponential)
     DevBuf chebd;                        // Chebyshev coefficients of the evaluation (state mode)
     DevBuf stscr;                        // state mode: the gradient kernel's per-item scratch
@@ -484,6 +485,8 @@ void plan_impl(qoc_ctx* c) {
         hoff.push_back((int)hidx.size());
     }
     if (M > 0 && (int)hoff.size() == M + 1 && hidx.size() * 4 <= M * dd) {
+        c->hmax = 0;
+        for (int k = 0; k < M; ++k) c->hmax = std::max(c->hmax, hoff[k + 1] - hoff[k]);
         hidx.push_back(0);   // never empty
         hval.push_back(C{});
         A(c->hoff, hoff.size() * sizeof(int), "alloc H_k offsets");
@@ -657,7 +660,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
     C* HR = c->HR.as<C>();
     SysView<R> sys{d, M, N, HR, HR + dd, c->Hdet.empty() ? nullptr : HR + (size_t)(M + 1) * dd,
                    c->delta.empty() ? nullptr : c->dDelta.as<double>(), u,
-                   c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>()};
+                   c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>(), c->hmax};
     CostView<R> cv{c->nF, c->fmask.as<int>(), c->colw.as<double>(), c->Wsum, c->psiTR.as<C>(),
                    c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]},
                    c->cost_fit};
@@ -1186,7 +1189,7 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
     C* HR = c->HR.as<C>();
     SysView<R> sys{d, M, N, HR, HR + dd, c->Hdet.empty() ? nullptr : HR + (size_t)(M + 1) * dd,
                    c->delta.empty() ? nullptr : c->dDelta.as<double>(), u,
-                   c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>()};
+                   c->hoff.as<int>(), c->hidx.as<int>(), c->hval.as<C>(), c->hmax};
     CostView<R> cv{c->nF, c->fmask.as<int>(), c->colw.as<double>(), c->Wsum, c->psiTR.as<C>(),
                    c->path.empty() ? nullptr : c->pathR.as<C>(), {c->alpha[0], c->alpha[1], c->alpha[2], c->alpha[3], c->alpha[4]},
                    c->cost_fit};

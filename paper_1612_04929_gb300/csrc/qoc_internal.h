@@ -35,6 +35,7 @@ struct SysView {
     const int* hoff = nullptr;
     const int* hidx = nullptr;
     const C_t<R>* hval = nullptr;
+    int hmax = 0;         // most elements of a control
 };
 
 // Column-panel layout of every d x S block on the device: the S columns are padded to

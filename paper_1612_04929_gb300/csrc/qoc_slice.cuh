@@ -16,28 +16,34 @@ namespace qoc {
 // reduction in FP64 per control) reads d^2 elements for each.  Evaluations went d = 27, E = 5, M = 6
 // 1.529 -> 1.510 ms, d = 40 1.635 -> 1.609 ms, d = 256, M = 16 (BF16_SPLIT) 157.2 -> 154.1 ms, d = 154,
 // S = 1 165.7 -> 163.8 ms.  at(a, b): Xbar's element.
+// One warp's sum over elements i0, i0 + step, .. of control k
+template <typename R, typename At>
+__device__ __forceinline__ double sparse_sum(const SysView<R>& sys, int k, int i0, int step, At at) {
+    const int i1 = sys.hoff[k + 1];
+    double v = 0.0;
+    float hi = 0.f, lo = 0.f;
+    for (int i = sys.hoff[k] + i0; i < i1; i += step) {
+        const int ab = sys.hidx[i];
+        const C_t<R> h = sys.hval[i];
+        const C_t<R> x = at(ab >> 16, ab & 0xffff);
+        if constexpr (sizeof(R) == 4) {
+            pair_acc(hi, lo, x.x, h.y);
+            pair_acc(hi, lo, -x.y, h.x);
+        } else {
+            v = fma(x.x, h.y, v);
+            v = fma(-x.y, h.x, v);
+        }
+    }
+    if constexpr (sizeof(R) == 4) v = (double)hi + (double)lo;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
 template <typename R, typename At>
 __device__ __forceinline__ void contract_sparse(const SysView<R>& sys, const DevParams* __restrict__ prm,
                                                 double* __restrict__ gpart, int e, int j, At at) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int k = warp; k < sys.M; k += nw) {
-        const int i1 = sys.hoff[k + 1];
-        double v = 0.0;
-        float hi = 0.f, lo = 0.f;
-        for (int i = sys.hoff[k] + lane; i < i1; i += 32) {
-            const int ab = sys.hidx[i];
-            const C_t<R> h = sys.hval[i];
-            const C_t<R> x = at(ab >> 16, ab & 0xffff);
-            if constexpr (sizeof(R) == 4) {
-                pair_acc(hi, lo, x.x, h.y);
-                pair_acc(hi, lo, -x.y, h.x);
-            } else {
-                v = fma(x.x, h.y, v);
-                v = fma(-x.y, h.x, v);
-            }
-        }
-        if constexpr (sizeof(R) == 4) v = (double)hi + (double)lo;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const double v = sparse_sum(sys, k, lane, 32, at);
         if (lane == 0) gpart[((size_t)e * sys.M + k) * sys.N + j] = prm->s * v;
     }
 }
