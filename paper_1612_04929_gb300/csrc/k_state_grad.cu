@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(SGT, 1) k_state_grad_lr(StateGradArgs<float> A
     // Xbar at the controls' elements; Chebyshev: Xbar = (-i / theta) sum_t w_t left right^dag
     const int nt = terms * S;
     for (int k = warp; k < A.M; k += SGW) {           // a warp per control (and its elements over the lanes)
-        float hi = 0.f, lo = 0.f;
+        double v = 0.0;   // in FP64 as in k_state_grad: two products an element, beside its sum over the terms
         for (int i = sys.hoff[k] + lane; i < sys.hoff[k + 1]; i += 32) {
             const int ab = sys.hidx[i];
             const float2 h = sys.hval[i];
@@ -210,10 +210,9 @@ __global__ void __launch_bounds__(SGT, 1) k_state_grad_lr(StateGradArgs<float> A
                 cfma_bcj(xb, make_float2(ww * q.x, ww * q.y), r[t]);
             }
             if (cheb) xb = make_float2(th * xb.y, -th * xb.x);
-            pair_acc(hi, lo, xb.x, h.y);
-            pair_acc(hi, lo, -xb.y, h.x);
+            v = fma((double)xb.x, (double)h.y, v);
+            v = fma(-(double)xb.y, (double)h.x, v);
         }
-        double v = (double)hi + (double)lo;
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) A.gpart[((size_t)e * A.M + k) * A.N + j] = A.prm->s * v;
     }
