@@ -54,9 +54,11 @@ inline int lr_ldw(int w) {
     if (((l >> 1) & 1) == 0) l += 2;
     return l;
 }
-// (the last chunk of a product may read up to LNC - 1 columns past a row: slack after the last block;
-// then the warps' partial sums of the sparse contraction)
-__host__ __device__ inline size_t lr_part_offset(int d, int ldw) { return ((size_t)6 * d * ldw + LNC) * sizeof(float2); }
+// (the last chunk of a product may read up to LNC - 1 columns past a row: slack after each block, so that the
+// last row's reads do not touch a block that the same product writes.  After the blocks the warps' partial
+// sums of the sparse contraction)
+__host__ __device__ inline size_t lr_block(int d, int ldw) { return (size_t)d * ldw + LNC; }
+__host__ __device__ inline size_t lr_part_offset(int d, int ldw) { return 6 * lr_block(d, ldw) * sizeof(float2); }
 inline size_t lr_smem(int d, int ldw) { return lr_part_offset(d, ldw) + kMaxControls * (LT / 32) * sizeof(double); }
 
 }  // namespace
@@ -94,7 +96,7 @@ __device__ __forceinline__ void lr_rows(float2 (&acc)[NJ][VW][LNC], const float2
 // y_j[:, c] = sgn_j M^dag-stored product of NJ blocks of w columns: the matrix M given as its
 // conjugate transpose Md, y = M x = (Md)^dag x.  NJ = 2 with M2 given: two matrices, one block each.
 // Row groups add their partial sums in turn (a fixed order).  Reads past w within the last chunk
-// touch the padding or the next block's columns and are not stored.  Ends with a barrier.
+// touch the padding, the next row or the slack after the block and are not stored.  Ends with a barrier.
 template <int VW, int NJ, bool TWO>
 __device__ __forceinline__ void lr_mul(const float2* __restrict__ M1, const float2* __restrict__ M2,
                                        const float2* x1, float2* y1, float sg1, const float2* x2, float2* y2, float sg2,
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(LT, 2) k_big_adj_lr(LrArgs A) {
     const int item = blockIdx.x, jl = item % A.wlen, e = item / A.wlen, j = A.j0 + jl;
     const int tid = threadIdx.x, d = A.sys.d, M = A.sys.M, r = A.r, qt = A.qt, ldw = A.ldw, p = A.p;
     const int S = A.sv.S, w1 = (qt + 1) * r;
-    const size_t blk = (size_t)d * ldw;
+    const size_t blk = lr_block(d, ldw);
     float2* Lw = reinterpret_cast<float2*>(smraw);   // L_0 .. L_qt, A2
     float2* Vw = Lw + blk;                           // V_0 .. V_qt, R
     float2* XL = Vw + blk;                           // X^dag L_0 .. X^dag L_qt, X^dag A2
@@ -202,7 +204,7 @@ __global__ void __launch_bounds__(LT, 2) k_big_adj_lr(LrArgs A) {
     auto slot = [&](int s) { return zi + (size_t)s * A.ms; };
     const float2* Xd = slot(A.cap - 1);
     const DevParams* prm = A.prm;
-    for (size_t i = tid; i < 6 * blk + LNC; i += LT) Lw[i] = make_float2(0.f, 0.f);
+    for (size_t i = tid; i < 6 * blk; i += LT) Lw[i] = make_float2(0.f, 0.f);
     __syncthreads();
     {   // L = G_j, R = Psi_{j-1}
         const size_t slice = A.sv.slice();

@@ -32,3 +32,21 @@ def test_launch_attributes_are_set_on_every_device():
         text = re.sub(r"//[^\n]*", "", text)
         flags = [m.group(0) for m in re.finditer(r"\bstatic\s+(?!constexpr|const\b)(?:bool|int|std::once_flag|std::atomic<\w+>)\s+\w+\s*(?:=|;|\{)", text)]
         assert not flags, (name, flags)
+
+
+def test_low_rank_factor_blocks_end_after_their_last_read():
+    """k_big_lr reads a block's rows in chunks of LNC columns, past the row's end in the last chunk; the block's
+    size (as the source computes it) covers the last row's reads, so that none falls into a block that the
+    same product writes."""
+    text = dict(sources())["k_big_lr.cu"]
+    lnc = int(re.search(r"constexpr int LNC = (\d+);", text).group(1))
+    block = re.search(r"const size_t blk = ([^;]+);", text).group(1)
+    body = re.search(r"size_t lr_block\(int d, int ldw\) \{ return ([^;]+); \}", text)
+    expr = (body.group(1) if body else block).replace("(size_t)", "")
+    for d in (1, 69, 154, 512):
+        for w in range(1, 65):
+            ldw = (w + 1) & ~1
+            ldw += 2 if (ldw >> 1) & 1 == 0 else 0
+            last = (d - 1) * ldw + (w - 1) // lnc * lnc + lnc - 1
+            assert last < eval(expr, {"d": d, "ldw": ldw, "LNC": lnc}), (d, w)
+            assert eval(expr, {"d": d, "ldw": ldw, "LNC": lnc}) % 2 == 0      # the next block's 16-byte loads
