@@ -206,7 +206,9 @@ typedef struct qoc_info {
 } qoc_info;
 
 /* Per-kernel timings gathered while qoc_options.profile is set: for each kernel class the number
- * of launches and the summed CUDA-event duration (ms) on the context stream. */
+ * of launches and the summed CUDA-event duration (ms) on the context stream.  The classes name the form
+ * that ran where a step has several: "tree ..." (with "(tensor cores)") in place of the segmented sweeps,
+ * "expm_adj (low rank)", "expm_adj (rank-one terms)", "state_chain (..., cluster)". */
 #define QOC_PROFILE_SLOTS 16
 typedef struct qoc_profile {
     int count;                           /* classes filled */

@@ -417,9 +417,10 @@ static cudaError_t cluster_rows(const StateChainArgs<R>& a, int cs, cudaStream_t
 // a product, about 0.55 + 0.004 rows x QB us a product (measured at d = 154: 0.77 us on 16 CTAs, 0.97 on
 // 8, 1.31 on 4).  What the device holds at once is asked, not counted: a second round doubles a
 // recursion (16 members on clusters of 8 took 2.07 us a product, on the size chosen here 1.03), and how
-// many clusters of a size fit depends on each GPC's free SMs.  0: k_state_chain's one CTA per panel
-// (wide panels, d > 192, where a warp's rows no longer fit its registers); at d = 154 that one takes
-// 8.5 us a product on up to 152 chains, slower than rounds of small clusters at any count.
+// many clusters of a size fit depends on each GPC's free SMs.  0: k_state_chain's one CTA per panel,
+// for panels of several columns, which the plan makes above two chains an SM (S E > 304 here); at d = 154
+// that one takes 8.5 us a product, so rounds of small clusters would be faster there too: not built.
+// (State mode ends near d = 167, where its gradient's block fills a CTA's shared memory.)
 template <typename R>
 int state_cluster_size(int d, const StateView<R>& sv, int E) {
     if (sv.cb != 1 || d > 192) return 0;

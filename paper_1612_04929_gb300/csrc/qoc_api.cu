@@ -796,14 +796,16 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
         }
         return launch_expm_fwd_fused<R>(prm, sys, j0, wlen, E, Ub(w), c->ustride, W, zstore(w), st);
     };
+    // few columns: the same derivative with low-rank cotangents (BF16_SPLIT keeps its dense products on the
+    // tensor cores)
+    const bool big_lr = big && big_rev && c->ps && c->opt.precision == QOC_PREC_FP32 && big_lr_applies(d, sv.S, hp.p, hp.n);
+    const char* adj_class = big_lr ? "expm_adj (low rank)" : "expm_adj";
     auto expm_adj = [&](int w) -> cudaError_t {
         const int j0 = w * W, wlen = std::min(W, N - j0);
         if (c->opt.gradient == QOC_GRAD_FIRST_ORDER)
             return launch_grad_first_order<R>(sys, sv, j0, wlen, E, Sb(w), Gb(w), W, c->dt, c->gpart.as<double>(), st);
         if constexpr (sizeof(R) == 4) {
-            // few columns: the same derivative with low-rank cotangents (BF16_SPLIT keeps its dense
-            // products on the tensor cores)
-            if (big && big_rev && c->ps && c->opt.precision == QOC_PREC_FP32 && big_lr_applies(d, sv.S, hp.p, hp.n))
+            if (big_lr)
                 return launch_big_adj_lr(big_args(w), sys, sv, Sb(w), Gb(w), c->gpart.as<double>(), hp, zbig(w), st);
             if (big && big_rev && c->ps) {       // Paterson-Stockmeyer reverse mode (tensor cores: BF16_SPLIT)
                 int n_l = 0;
@@ -888,18 +890,19 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
         };
         const size_t ck_e = (size_t)c->nseg_total * slice;
         auto ck = [&](int w) { return c->ckpt.as<K>() + (size_t)(w * W / seg) * slice; };   // first block of wave w
+        const bool tc = c->tree_cap > 0;
         auto forward = [&](int w, bool hand_on) {
             int n_l = 0;
             B(sx);
             cudaError_t e = launch_tree_up(targs(w), sx, &n_l);
-            L(e, "seg_products", sx);
+            L(e, tc ? "tree nodes (tensor cores)" : "tree nodes", sx);
             extra += n_l - 1;
             n_l = 0;
             B(sx);
             const bool next = hand_on && w + 1 < nw;
             e = launch_tree_forward(targs(w), ck(w), ck_e, next ? ck(w + 1) : nullptr, ck_e, Sb(w), (size_t)(W + 1) * slice,
                                     c->tmo.as<float>(), sx, &n_l);
-            L(e, "chain (replay)", sx);
+            L(e, tc ? "tree states (tensor cores)" : "tree states", sx);
             extra += n_l - 1;
         };
         for (int w = 0; w < nw; ++w) {
@@ -928,7 +931,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             const cudaError_t e = launch_tree_costate(targs(w), w == nw - 1 ? c->tgtK.as<float4>() : c->carry.as<float4>(),
                                                       w == nw - 1 ? 0 : slice, w > 0 ? c->carry.as<float4>() : nullptr, slice,
                                                       Gb(w), (size_t)W * slice, c->tcoef.as<float4>(), c->tmo.as<float>() + sv.S, sx, &n_l);
-            L(e, "costate (final)", sx);
+            L(e, tc ? "tree costates (tensor cores)" : "tree costates", sx);
             extra += n_l - 1;
             rec(ev_cost[w], sx);
             if (w >= 1 && w - 1 < nw - 2) {                // set (w - 1) % 2: wave w + 1's, whose adjoint is on st
@@ -938,7 +941,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             }
             wait(st, ev_cost[w]);
             B(st);
-            L(expm_adj(w), "expm_adj", st);
+            L(expm_adj(w), adj_class, st);
         }
         rec(ev_join, sx);
         wait(st, ev_join);
@@ -1013,7 +1016,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             }
             wait(st, ev_cost[w]);
             B(st);
-            L(expm_adj(w), "expm_adj", st);
+            L(expm_adj(w), adj_class, st);
         }
     } else {
         // ---- forward: exponentials on st; the segment products and the scan over segments
@@ -1115,7 +1118,7 @@ void evaluate_impl(qoc_ctx* c, const double* u, double* grad, double* out, const
             }
             wait(st, ev_cost[w]);
             B(st);
-            L(expm_adj(w), "expm_adj", st);
+            L(expm_adj(w), adj_class, st);
         }
     }
     rec(ev_join, sx);
@@ -1273,7 +1276,7 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
                             (store_next && w + 1 < nw) ? ck + (size_t)(w + 1) * slice : nullptr, ck_es,
                             states, (size_t)(W + 1) * slice, nullptr, 0, prm, chebd, c->state_cs};
         B();
-        L(launch_state_chain<R>(a, st), "state_chain (forward)");
+        L(launch_state_chain<R>(a, st), c->state_cs ? "state_chain (forward, cluster)" : "state_chain (forward)");
     };
     for (int w = 0; w < nw; ++w) {
         const int j0 = w * W, wlen = std::min(W, N - j0);
@@ -1297,7 +1300,7 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
         StateChainArgs<R> b{d, E, wlen, 1, sv, X, xs, c->carry.as<K>(), slice, c->carry.as<K>(), slice,
                             G, (size_t)W * slice, src, (size_t)W * slice, prm, chebd, c->state_cs};
         B();
-        L(launch_state_chain<R>(b, st), "state_chain (costate)");
+        L(launch_state_chain<R>(b, st), c->state_cs ? "state_chain (costate, cluster)" : "state_chain (costate)");
         if (c->opt.gradient == QOC_GRAD_FIRST_ORDER) {
             B();
             L(launch_grad_first_order<R>(sys, sv, j0, wlen, E, states, G, W, c->dt, c->gpart.as<double>(), st),
@@ -1308,7 +1311,7 @@ void evaluate_state_impl(qoc_ctx* c, const double* u, double* grad, double* out)
             B();
             if constexpr (sizeof(R) == 4) {
                 if (grad_lr) {
-                    L(launch_state_grad_lr(g, sys, p, n, st), "expm_adj");
+                    L(launch_state_grad_lr(g, sys, p, n, st), "expm_adj (rank-one terms)");
                     continue;
                 }
             }
