@@ -297,30 +297,25 @@ cudaError_t launch_to_panels(const double2* src, C_t<R>* dst, int d, int S, Stat
 // ------------------------------------------------------------------------------------------
 // per-slice costs and sources
 //
-// Both kernels read every state once and do a few multiply-adds per element, so HBM should bound
-// them.  The FP64 pipe of this part runs at 1/64 of the FP32 rate: summing the FP32 form's
-// products in FP64 (about 16 FP64 instructions per element, conversions included) made them bound
-// by it.  Here a thread keeps one column of a panel (thread t: column t % cb, rows t / cb, t / cb +
-// ts / cb, ...; the addresses of a pass stay contiguous), takes the column's weight in FP64 once per
-// run of equal weights, and the FP32 form sums its products without FP64 (RunSum<true>); the sources'
-// coefficients are set once per column and only the terms that act on an element are computed.
+// Both kernels read every state once and do a few multiply-adds per element, so HBM should bound them.  What
+// did: the FP64 pipe (1/64 of the FP32 rate) where the FP32 form's products were summed in FP64; and, for
+// launches of few slices, the instruction cache: with the loops unrolled and the last slice's terms in code
+// of their own a launch of 50 slices of d = 30 took 37 us, most of it fetching code, as one loop 12 us.  So
+// the FP32 form's cost sums run without FP64 (RunSum), in one loop that loads an element ahead; sources set
+// their coefficients once per run of equal weights, compute the terms that act on an element, and take C5
+// alone without FP64.
+// Two launches of an evaluation, costs / sources (before, with FP64 throughout | with pairs of floats in unrolled
+// loops | now): d = 30, S = 30, N = 400 43 / 54 | 68 / 78 | 31 / 24 us; d = 64, S = 64, N = 2000 (terminal) 401 | 90
+// | 88; d = 81, S = 16, N = 1000 135 / 122 | 85 / 99 | 58 / 35; d = 81, S = 81, N = 100 111 / 125 | 148 / 140 | 48 / 69;
+// d = 256, S = 256, N = 60 938 / 1047 | 332 / 417 | 234 / 501 (the last slice's target terms are FP64);
+// FP64 form, d = 60, S = 60, N = 30 57 / 63 | 123 / 149 | 42 / 47.
 // ------------------------------------------------------------------------------------------
-// Running sum of real products, v += a b.  In FP64; or (FP32 values, TRI) over three floats: the product
-// and its rounding error are added error-free to the first two, what these round off to the third, so
-// a sum of n terms is off by about n^2 2^-72 of them, below FP64's n 2^-53 for the few hundred terms of a
-// thread (two floats: about 2^-48, 150 times FP64's error over 256 terms).  22 FP32 operations a product:
-// d = 128, S = 128, N = 500 took 142 us (two floats 113).  The exactness needs the product's error term to
-// be representable: cost_sums_fit; other norms are summed in FP64.
-template <bool TRI> struct RunSum {
-    double v = 0.0;
-    template <typename T> __device__ __forceinline__ void add(T a, T b) { v = fma((double)a, (double)b, v); }
-    __device__ __forceinline__ double take() {
-        const double r = v;
-        v = 0.0;
-        return r;
-    }
-};
-template <> struct RunSum<true> {
+// Running sum of products of FP32 values over three floats: the product and its rounding error are added
+// error-free to the first two, what these round off to the third, so a sum of n terms is off by about n^2
+// 2^-72 of them, below FP64's n 2^-53 for the few hundred terms of a thread (two floats: about 2^-48, 150
+// times FP64's error over 256 terms).  22 FP32 operations a product.  The exactness needs the product's
+// error term to be representable: cost_sums_fit.
+struct RunSum {
     float h = 0.f, m = 0.f, l = 0.f;
     __device__ __forceinline__ void add(float a, float b) {
         const float p = a * b, e = fmaf(a, b, -p);
@@ -336,6 +331,42 @@ template <> struct RunSum<true> {
         const double v = (double)h + ((double)m + (double)l);
         h = m = l = 0.f;
         return v;
+    }
+};
+
+// A thread's elements of a panel-layout block: every ts-th one from t0 on (consecutive threads, consecutive
+// addresses), without the panels' padding and without a division per element
+struct CostWalk {
+    int d, cb, ps, ncb, da, dc;
+    int kb, a, c;     // panel, row and column of the panel
+    int s;            // column of the block
+    size_t i;         // offset in the block
+    __device__ __forceinline__ CostWalk(int d_, int cb_, int ps_, int ncb_, int t0, int ts)
+        : d(d_), cb(cb_), ps(ps_), ncb(ncb_) {
+        da = ts / cb;
+        dc = ts - da * cb;
+        kb = 0;
+        a = t0 / cb;
+        c = t0 - a * cb;
+        wrap();
+    }
+    __device__ __forceinline__ void wrap() {
+        while (a >= d) {
+            a -= d;
+            ++kb;
+        }
+        s = kb * cb + c;
+        i = (size_t)kb * ps + (size_t)a * cb + c;
+    }
+    __device__ __forceinline__ bool on() const { return kb < ncb; }
+    __device__ __forceinline__ void next() {
+        a += da;
+        c += dc;
+        if (c >= cb) {
+            c -= cb;
+            ++a;
+        }
+        wrap();
     }
 };
 
@@ -355,52 +386,78 @@ k_slice_costs(int d, StateView<R> sv, int j0, int wlen, int N, const C_t<R>* __r
     const C* psi = states + ((size_t)e * (wmax + 1) + jl + 1) * slice;
     const C* T = cv.path ? cv.path + (size_t)j * slice : cv.psiT;
     const bool last = (j == N - 1), forb = cv.nF > 0;
-    // panels wider than the threads (one panel of all columns) are walked in chunks of ts columns
-    const int cw = cb < ts ? cb : ts, rows = ts / cw, a0 = t0 / cw, sc = t0 - a0 * cw;
-    RunSum<TRI> so[2], sf[2], s5;
-    double ore = 0, oim = 0, c5 = 0, fre = 0, fim = 0, w = 0.0;
-    auto flush = [&]() {
-        ore = fma(w, so[0].take(), ore);
-        oim = fma(w, so[1].take(), oim);
-        if (forb) c5 = fma(w, s5.take(), c5);
-        if (last) {
-            fre = fma(w, sf[0].take(), fre);
-            fim = fma(w, sf[1].take(), fim);
-        }
-    };
-    if (a0 < rows)
-        for (int ch = 0, nch = (cb + cw - 1) / cw; ch < sv.ncb * nch; ++ch) {
-            const int kb = ch / nch, s0 = (ch - kb * nch) * cw + sc;
-            if (s0 >= cb) continue;
-            const double wk = cv.w[kb * cb + s0];
-            if (wk != w) {
-                if (w != 0.0) flush();
-                w = wk;
-            }
-            if (wk == 0.0) continue;
-            const size_t base = (size_t)kb * ps + s0;
-#pragma unroll 4
-            for (int a = a0; a < d; a += rows) {
-                const size_t i = base + (size_t)a * cb;
-                const C z = psi[i], t = T[i];
+    double ore = 0, oim = 0, c5 = 0, fre = 0, fim = 0;
+    // the overlaps with T; then, in the last slice of a path, those with psiT
+    const bool twice = last && cv.path;
+#pragma unroll 1
+    for (int pass = 0; pass < (twice ? 2 : 1); ++pass) {
+        const C* Tp = pass ? cv.psiT : T;
+        const bool five = forb && pass == 0;
+        double re = 0, im = 0;
+        CostWalk at(d, cb, ps, sv.ncb, t0, ts);
+        if constexpr (TRI) {
+            RunSum so[2], s5;
+            long long w = 0, wk = 0, wn = 0;
+            auto flush = [&]() {
+                const double x = __longlong_as_double(w);
+                re = fma(x, so[0].take(), re);
+                im = fma(x, so[1].take(), im);
+                if (five) c5 = fma(x, s5.take(), c5);
+            };
+            C z, t, zn, tn;
+            int a = 0;
+            auto load = [&]() {   // the next element, while this one is summed
+                if (!at.on()) return;
+                zn = psi[at.i];
+                tn = Tp[at.i];
+                wn = __double_as_longlong(cv.w[at.s]);
+            };
+            load();
+#pragma unroll 1
+            while (at.on()) {
+                z = zn;
+                t = tn;
+                wk = wn;
+                a = at.a;
+                at.next();
+                load();
+                if (wk == 0) continue;
+                if (wk != w) {
+                    if (w != 0) flush();
+                    w = wk;
+                }
                 so[0].add(t.x, z.x);
                 so[0].add(t.y, z.y);
                 so[1].add(t.x, z.y);
                 so[1].add(-t.y, z.x);
-                if (forb && cv.fmask[a]) {
+                if (five && cv.fmask[a]) {
                     s5.add(z.x, z.x);
                     s5.add(z.y, z.y);
                 }
-                if (last) {
-                    const C f = cv.psiT[i];
-                    sf[0].add(f.x, z.x);
-                    sf[0].add(f.y, z.y);
-                    sf[1].add(f.x, z.y);
-                    sf[1].add(-f.y, z.x);
-                }
+            }
+            if (w != 0) flush();
+        } else {
+#pragma unroll 4
+            for (; at.on(); at.next()) {
+                const double w = cv.w[at.s];
+                const C z = psi[at.i], t = Tp[at.i];
+                re += w * ((double)t.x * z.x + (double)t.y * z.y);
+                im += w * ((double)t.x * z.y - (double)t.y * z.x);
+                if (five && cv.fmask[at.a]) c5 += w * ((double)z.x * z.x + (double)z.y * z.y);
             }
         }
-    if (w != 0.0) flush();
+        if (pass == 0) {
+            ore = re;
+            oim = im;
+        } else {
+            fre = re;
+            fim = im;
+        }
+    }
+    if (last && !twice) {
+        fre = ore;
+        fim = oim;
+    }
     auto sum = [&](double v) {
         if (WARP) {
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -458,63 +515,63 @@ k_sources(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* 
     const bool last = (j == N - 1);
     const double2 of = last ? Ofin[e] : make_double2(0.0, 0.0);
     const bool use_t = ct != 0.0, use_5 = cv.nF > 0 && c5 != 0.0;
-    const int rows = ts / cb, a0 = t0 / cb, s0 = t0 - a0 * cb;
-    // Elements on which C5 alone acts, c5 w z: without FP64 in the FP32 form, the coefficient as a pair (the
-    // product is off by 2^-47 before it is rounded to FP32).  d = 27, N = 777, E = 5 took 37 us and d = 81,
-    // N = 1000 86 us; with every element and the coefficients' divisions here in FP64 82 and 133.
+    // Where C5 alone acts, c5 w z: without FP64 in the FP32 form, the coefficient as a pair (the product is off
+    // by 2^-47 before it is rounded to FP32), set when the weight changes (its bits: FP64 comparisons would cost
+    // as much as the products)
     const bool c5_only = sizeof(R) == 4 && cv.fit && !use_t && !last;
-    if (a0 < rows)
-        for (int kb = 0; kb < sv.ncb; ++kb) {
-            const double w = cv.w[kb * cb + s0];
-            if constexpr (sizeof(R) == 4) {
-                const double cw = use_5 ? c5 * w : 0.0;
-                if (c5_only && (cw == 0.0 || (fabs(cw) >= 0x1p-40 && fabs(cw) <= 0x1p40))) {
-                    const float ch = (float)cw, cl = (float)(cw - (double)ch);
-#pragma unroll 4
-                    for (int a = a0; a < d; a += rows) {
-                        const size_t i = (size_t)kb * ps + s0 + (size_t)a * cb;
-                        C r = make_float2(0.f, 0.f);
-                        if (cw != 0.0 && cv.fmask[a]) {
-                            const C z = psi[i];
-                            r.x = ch * z.x;
-                            r.y = ch * z.y;
-                            r.x += fmaf(cl, z.x, fmaf(ch, z.x, -r.x));
-                            r.y += fmaf(cl, z.y, fmaf(ch, z.y, -r.y));
-                        }
-                        out[i] = r;
-                    }
-                    continue;
-                }
-            }
-            const double tx = ct * w * o.x, ty = ct * w * o.y, fx = cf * w * of.x, fy = cf * w * of.y, c5w = c5 * w;
-            const size_t base = (size_t)kb * ps + s0;
-#pragma unroll 4
-            for (int a = a0; a < d; a += rows) {
-                const size_t i = base + (size_t)a * cb;
-                double vx = 0.0, vy = 0.0;
-                if (w != 0.0) {
-                    if (use_t) {
-                        const C t = T[i];
-                        vx = tx * t.x - ty * t.y;
-                        vy = tx * t.y + ty * t.x;
-                    }
-                    if (use_5 && cv.fmask[a]) {
-                        const C z = psi[i];
-                        vx += c5w * z.x;
-                        vy += c5w * z.y;
-                    }
-                    if (last) {
-                        const C f = cv.psiT[i];
-                        vx += fx * f.x - fy * f.y;
-                        vy += fx * f.y + fy * f.x;
-                    }
-                }
-                C r;
-                r.x = (R)vx;
-                r.y = (R)vy;
-                out[i] = r;
+    long long w = 0;
+    double tx = 0.0, ty = 0.0, fx = 0.0, fy = 0.0, c5w = 0.0;   // coefficients of columns of weight w
+    float qh = 0.f, ql = 0.f;
+    bool quick = false;
+    for (CostWalk at(d, cb, ps, sv.ncb, t0, ts); at.on(); at.next()) {
+        C r;
+        r.x = r.y = 0;
+        const long long wk = __double_as_longlong(cv.w[at.s]);
+        const bool f = wk != 0 && use_5 && cv.fmask[at.a];
+        if (wk != 0 && wk != w) {
+            w = wk;
+            const double x = __longlong_as_double(w);
+            c5w = c5 * x;
+            quick = c5_only && fabs(c5w) >= 0x1p-40 && fabs(c5w) <= 0x1p40;
+            if (c5_only) {
+                qh = (float)c5w;
+                ql = (float)(c5w - (double)qh);
+            } else {
+                tx = ct * x * o.x;
+                ty = ct * x * o.y;
+                fx = cf * x * of.x;
+                fy = cf * x * of.y;
             }
         }
+        if (c5_only && (quick || !f)) {
+            if (f) {
+                const C z = psi[at.i];
+                const float zx = (float)z.x, zy = (float)z.y, px = qh * zx, py = qh * zy;
+                r.x = px + fmaf(ql, zx, fmaf(qh, zx, -px));
+                r.y = py + fmaf(ql, zy, fmaf(qh, zy, -py));
+            }
+        } else if (wk != 0) {
+            double vx = 0.0, vy = 0.0;
+            if (use_t) {
+                const C t = T[at.i];
+                vx = tx * t.x - ty * t.y;
+                vy = tx * t.y + ty * t.x;
+            }
+            if (f) {
+                const C z = psi[at.i];
+                vx += c5w * z.x;
+                vy += c5w * z.y;
+            }
+            if (last) {
+                const C g = cv.psiT[at.i];
+                vx += fx * g.x - fy * g.y;
+                vy += fx * g.y + fy * g.x;
+            }
+            r.x = (R)vx;
+            r.y = (R)vy;
+        }
+        out[at.i] = r;
+    }
     // the panels' 16-byte padding (past d * cb) is copied with them: keep it zero
     for (int kb = 0; kb < sv.ncb; ++kb)
         for (int i = d * cb + t0; i < ps; i += ts) {
