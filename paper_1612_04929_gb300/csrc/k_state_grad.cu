@@ -221,6 +221,10 @@ __global__ void __launch_bounds__(SGT, 1) k_state_grad_lr(StateGradArgs<float> A
 // applies: FP32 form, sparse controls, few enough columns chunks for the registers, and a term to have
 bool state_grad_lr_applies(const SysView<float>& sys, int d, int S, int p, int n, int K, bool cheb) {
     const int terms = sg_terms(p, n, cheb ? K : 0);
+    // small d with several columns: the columns go one after another here, and a CTA of k_state_grad takes little
+    // more than one (d = 16, 900 slices, Chebyshev: S = 2 133 us against 193 there, S = 4 246 against 213, S = 8
+    // 324 against 217; d = 24, S = 8 334 against 387)
+    if (d < 24 && S > 2) return false;
     if (!sys.hoff || d > 32 * kSgMaxChunks || (cheb && K < 1) || (!cheb && n > 16)) return false;
     if (!cheb && p > kChebMax) return false;
     return (long long)terms * S < 4096 && sg_smem(d, S, p, n, cheb ? K : 0) <= kMaxDynSmem;
