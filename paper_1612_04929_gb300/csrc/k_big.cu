@@ -707,9 +707,14 @@ static cudaError_t mm_launch(int d, int items, const E* A, const E* B, E* Cm, si
     if constexpr (sizeof(E) == 16 && MODE == 0) {          // FP64
         QOC_MM(GemmWide);
     } else if constexpr (sizeof(E) == 16) {
+        if constexpr (MODE == 1)
+            if (gemm_split_small(d, items, sm_count())) QOC_MM(GemmSplitS);
         QOC_MM(GemmSplit);
     } else {
-        switch (gemm_plain_mt(d)) {
+        switch (gemm_plain_mt(d, items, sm_count())) {
+            case 1: QOC_MM(GemmPlain1);
+            case 2: QOC_MM(GemmPlain2);
+            case 3: QOC_MM(GemmPlain3);
             case 4:
                 if (d % GemmPlain4::T == 0) QOC_MM(GemmPlain4F);
                 QOC_MM(GemmPlain4);
@@ -988,7 +993,10 @@ static cudaError_t rev_launch(int d, int items, const RevOps<C>& ops, C* O1, C* 
     if constexpr (sizeof(C) == 16) {
         return rev_launch_t<C, GemmWide>(d, items, ops, O1, O2, ms, mode, i, st);
     } else {
-        switch (gemm_plain_mt(d)) {
+        switch (gemm_plain_mt(d, items, sm_count())) {
+            case 1: return rev_launch_t<C, GemmPlain1>(d, items, ops, O1, O2, ms, mode, i, st);
+            case 2: return rev_launch_t<C, GemmPlain2>(d, items, ops, O1, O2, ms, mode, i, st);
+            case 3: return rev_launch_t<C, GemmPlain3>(d, items, ops, O1, O2, ms, mode, i, st);
             case 4:
                 if (d % GemmPlain4::T == 0) return rev_launch_t<C, GemmPlain4F>(d, items, ops, O1, O2, ms, mode, i, st);
                 return rev_launch_t<C, GemmPlain4>(d, items, ops, O1, O2, ms, mode, i, st);

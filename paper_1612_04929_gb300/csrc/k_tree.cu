@@ -63,9 +63,8 @@ struct MacSplitConj {
 };
 
 // AK: 0 A carried, 1 A rounded propagators, 2 A carried and taken as A^dag; BL: B rounded propagators
-template <int AK, bool BL>
-__global__ void __launch_bounds__(GemmSplit::NT, GemmSplit::MB) k_tree_mm(TreeMm t) {
-    using Sh = GemmSplit;
+template <int AK, bool BL, class Sh>
+__global__ void __launch_bounds__(Sh::NT, Sh::MB) k_tree_mm(TreeMm t) {
     constexpr int MT = Sh::MT, G = Sh::G;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int tiles = t.tiles_r * t.tiles_c;
@@ -168,15 +167,23 @@ __global__ void k_tree_coef(CostView<float> cv, int E, int cols, const double2* 
 
 int tree_ew_blocks(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 64); }
 
+template <int AK, bool BL, class Sh>
+cudaError_t mm_tiles(TreeMm t, cudaStream_t st) {
+    constexpr size_t smem = Sh::template smem<float4>();
+    cudaError_t e = cudaFuncSetAttribute(k_tree_mm<AK, BL, Sh>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    t.tiles_r = Sh::tiles(t.d);
+    t.tiles_c = Sh::tiles(t.cols);
+    k_tree_mm<AK, BL, Sh><<<t.tiles_r * t.tiles_c * t.E * t.count, Sh::NT, smem, st>>>(t);
+    return cudaGetLastError();
+}
+
 template <int AK, bool BL>
 cudaError_t mm(const TreeArgs& a, const TreeMm& t, cudaStream_t st, int* launches) {
     if (a.oz) return oz_tree_product(*a.oz, t, AK, BL, a.prm, st, launches);
-    constexpr size_t smem = GemmSplit::smem<float4>();
-    cudaError_t e = cudaFuncSetAttribute(k_tree_mm<AK, BL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_tree_mm<AK, BL><<<t.tiles_r * t.tiles_c * t.E * t.count, GemmSplit::NT, smem, st>>>(t);
     ++*launches;
-    return cudaGetLastError();
+    if (gemm_split_small(t.d, (long)t.E * t.count, sm_count())) return mm_tiles<AK, BL, GemmSplitS>(t, st);
+    return mm_tiles<AK, BL, GemmSplit>(t, st);
 }
 
 TreeMm base(const TreeArgs& a, int cols) {
@@ -184,8 +191,6 @@ TreeMm base(const TreeArgs& a, int cols) {
     t.d = a.d;
     t.cols = cols;
     t.E = a.E;
-    t.tiles_r = GemmSplit::tiles(a.d);
-    t.tiles_c = GemmSplit::tiles(cols);
     t.prm = a.prm;
     return t;
 }

@@ -361,9 +361,9 @@ void plan_impl(qoc_ctx* c) {
     const bool terminal = cost_is_terminal(c->nF, c->alpha);
     const bool sources = state_mode || !terminal;   // a terminal cost has no source but the carried block
     // Full unitaries with a cost on the final state alone: both recursions as batched products over the
-    // wave's tree, from d = 48 on (below, a chain step costs a few us and the tree's launches more).
+    // wave's tree (tree_applies).
     // The blocks are then one panel of all columns (row-major).
-    c->tree = sizeof(R) == 4 && c->scan && S == d && d >= kTreeMinD && terminal;
+    c->tree = sizeof(R) == 4 && c->scan && S == d && tree_applies(d, (long)N * E) && terminal;
     std::vector<float> tree_mo;   // grids of the states' columns, then of the costates': 2^e bounds the norm
     if (c->tree) {
         for (const auto* norms : {&norm0, &normT})

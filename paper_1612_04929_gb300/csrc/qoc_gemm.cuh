@@ -11,14 +11,16 @@
 //          16 x 16, MT = 4: 53; MT = 2 (the former tile up to d = 96): 41; grids that are no multiple of
 //          four warps, 20 x 20 or 21 x 21: 38 (the schedulers' loads differ)
 //   plain  16 x 16 threads, MT = 4: 44, MT = 5: 47, MT = 6: 46; 8 x 8, MT = 4: 39
-// so split products take 32 x 32 tiles of 64 threads (d = 154 as 160 rows, not 192), and plain products
-// the 16 x 16 grid with the MT that pads least for its rate.  Rows of an edge tile past d are left out
+// so split products take 32 x 32 tiles of 64 threads (d = 154 as 160 rows, not 192), or 16 x 16 tiles where
+// there are few products or 32 pads much, and plain products the 16 x 16 grid with an MT that depends on d and
+// on their number (gemm_time).  Rows of an edge tile past d are left out
 // in the plain products, whose tiles are large; in the split ones the branches (591 against 548 us) or
 // loops of their own for the edges (instruction cache) cost more than the padding.  Against the former
 // tiles a split product went, per 300 items of d = 154, 700 -> 548 us (the plain-operand chain products
 // 366 -> 277); per 500 of d = 81 161 -> 113 (chain), 195 -> 194
 // (others); d = 128 is as before (264 us per 250).
 #pragma once
+#include <algorithm>
 #include <type_traits>
 
 #include "qoc_device.cuh"
@@ -38,18 +40,44 @@ struct GemmShape {
     template <typename E> static constexpr size_t smem() { return ST * sizeof(E) * ((size_t)T * (kGemmK + 1) + (size_t)kGemmK * (T + 1)); }
 };
 using GemmSplit = GemmShape<4, 8, 2, 6, false>;
+using GemmSplitS = GemmShape<2, 8, 2, 12, false>;    // small tiles: few items, or d that 32 pads
+using GemmPlain1 = GemmShape<1, 16, 3, 6, true>;     // 1 to 3: few items
+using GemmPlain2 = GemmShape<2, 16, 3, 4, true>;
+using GemmPlain3 = GemmShape<3, 16, 3, 3, true>;
 using GemmPlain4 = GemmShape<4, 16, 3, 2, true>;
 using GemmPlain4F = GemmShape<4, 16, 3, 2, false>;   // d a multiple of 64: nothing to leave out (203 -> 194 us)
 using GemmPlain5 = GemmShape<5, 16, 3, 2, true>;
 using GemmPlain6 = GemmShape<6, 16, 3, 2, true>;
 using GemmWide = GemmShape<2, 16, 2, 2, true>;       // FP64 operands (bound by the FP64 pipe)
-// outputs a side of a plain FP32 product of size d: least padded work over the measured rate
-inline int gemm_plain_mt(int d) {
-    const double rate[3] = {44, 47, 46};
+inline int sm_count() {   // of the current device
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    return std::max(n, 1);
+}
+// Time of a launch of `items` products in tiles of one shape, in units that scale with d: a CTA alone on an SM
+// takes `alone`, a full SM gives one every `each`, and the SMs' CTAs come in whole numbers.
+inline double gemm_time(int d, long items, int T, double alone, double each, int sms) {
+    const long n = (d + T - 1) / T, ctas = n * n * items;
+    return std::max(alone, (double)((ctas + sms - 1) / sms) * each);
+}
+// Shapes by that model; alone and each as measured at d = 128 (us; launches of 1 and of 400 products):
+// split   32 x 32 tiles 24.8 and 9.2, 16 x 16 10.6 and 2.8
+// plain   T = 16 .. 96 11, 23, 33, 45, 63, 88 and 4.2, 9.9, 17.6, 33, 46.5, 75
+// It picks the fastest shape, or one within 15 % of it, of 1 to 400 products of d = 48 .. 256.  From a product
+// an SM on, plain tiles of at least 64: the smaller ones are no faster then (400 of d = 81 133 us as 48 x 48,
+// 135 as 96 x 96) and take more of the chip from kernels beside them (a batch of sixteen problems 172.7 against
+// 175.2 ms).  By padding alone, few products ran on few SMs: 50 of d = 81 as one 96 x 96 tile each took 62 us a reverse step, now 27;
+// an evaluation of d = 81, N = 100 with the Horner series went from 2.02 (32 x 32 tiles) to 2.63 ms.
+inline bool gemm_split_small(int d, long items, int sms) {
+    return gemm_time(d, items, 16, 10.6, 2.8, sms) < gemm_time(d, items, 32, 24.8, 9.2, sms);
+}
+inline int gemm_plain_mt(int d, long items, int sms) {
+    const double alone[6] = {11, 23, 33, 45, 63, 88}, each[6] = {4.2, 9.9, 17.6, 33, 46.5, 75};
     int best = 4;
     double cost = 1e300;
-    for (int mt = 4; mt <= 6; ++mt) {
-        const double w = (double)((d + 16 * mt - 1) / (16 * mt)) * 16 * mt, c = w * w / rate[mt - 4];
+    for (int mt = items < sms ? 1 : 4; mt <= 6; ++mt) {
+        const double c = gemm_time(d, items, 16 * mt, alone[mt - 1], each[mt - 1], sms);
         if (c < cost) {
             cost = c;
             best = mt;

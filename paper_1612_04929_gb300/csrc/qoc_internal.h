@@ -513,7 +513,11 @@ struct TreeArgs {
     DevParams* prm;
     const OzTree* oz;       // or nullptr
 };
-constexpr int kTreeMinD = 48;
+// from which size and length on.  Evaluations with the sweeps over the same with the tree (N = 16, 60, 100, 200, 400,
+// 2000): d = 40 0.89, 0.80, 0.78, 0.77, 0.89, 1.04; d = 48 0.94, 0.88, 0.90, 0.98, 1.21, 1.29; d = 56 0.98, 0.96, 1.01,
+// 1.15, 1.41, 1.15; d = 64 1.00, 1.03, 1.10, 1.23, 1.32, 1.20; d = 72 1.00, 1.00, 1.07, 1.13, 1.17, 1.21; d = 128
+// 1.37 to 1.59 (a level's launch takes longer than a chain's step where it has few products of little work)
+inline bool tree_applies(int d, long slices) { return d >= 64 || (d >= 48 && slices >= 200); }
 int tree_levels(int wlen);
 size_t tree_nodes(int W);   // per member
 cudaError_t launch_tree_up(const TreeArgs& a, cudaStream_t st, int* launches);

@@ -15,7 +15,7 @@ __device__ __forceinline__ float4 tree_split(const float4 v, float m) {
 // One batched product of a level.  Item (e, i): A = a + e ae + i ai (matrices d x d), B = b + e be + i bi
 // (d x cols), out likewise.  A or B may be the slice propagators (float2, rounded; split here).
 struct TreeMm {
-    int d, cols, E, count, tiles_r, tiles_c;
+    int d, cols, E, count, tiles_r, tiles_c;   // tiles: set with the launch's shape
     const void* a;
     size_t ae, ai;
     const void* b;

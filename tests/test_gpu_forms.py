@@ -27,13 +27,16 @@ TREE_TC = {t + " (tensor cores)" for t in TREE}
 
 
 @pytest.mark.parametrize("precision,d,S,nF,opt,want", [
-    ("fp32", 48, 48, 0, {}, TREE), ("fp32", 47, 47, 0, {}, set()), ("fp32", 64, 63, 0, {}, set()),
+    ("fp32", 48, 48, 0, dict(N=200), TREE), ("fp32", 48, 48, 0, dict(N=199), set()), ("fp32", 63, 63, 0, dict(N=50, E=4), TREE),
+    ("fp32", 63, 63, 0, {}, set()), ("fp32", 64, 64, 0, {}, TREE), ("fp32", 47, 47, 0, dict(N=200), set()),
+    ("fp32", 64, 63, 0, {}, set()),
     ("fp32", 64, 64, 0, dict(sweep="serial"), set()), ("fp64", 64, 64, 0, {}, set()), ("fp32", 64, 64, 2, {}, set()),
     ("fp32", 130, 130, 0, {}, TREE), ("tf32", 70, 70, 0, {}, TREE), ("bf16", 127, 127, 0, {}, TREE),
     ("bf16", 128, 128, 0, {}, TREE_TC), ("bf16", 384, 384, 0, {}, TREE_TC), ("bf16", 385, 385, 0, {}, TREE)])
 def test_tree(precision, d, S, nF, opt, want):
     alpha = GATE if nF == 0 else np.array([1.0, 0.01, 0.02, 0.5, 0.0])
-    prob = sy.random_problem(d=d, M=1, N=17, S=S, seed=11, nF=nF, dt=1.0 / d, alpha=alpha)
+    opt = dict(opt)
+    prob = sy.random_problem(d=d, M=1, N=opt.pop("N", 17), E=opt.pop("E", 1), S=S, seed=11, nF=nF, dt=1.0 / d, alpha=alpha)
     got = classes(prob, precision, **opt)
     assert got & (TREE | TREE_TC) == want
     assert ("chain (replay)" in got or "chain" in got or "costate (final)" in got or "costate" in got) or want
@@ -70,7 +73,7 @@ def test_state_recursion(precision, d, S, E, cluster, exponential):
 
 
 @pytest.mark.parametrize("exponential", ["taylor", "chebyshev"])
-@pytest.mark.parametrize("precision,d,dense,terms", [("fp32", 9, False, True), ("fp32", 160, False, True), ("fp32", 161, False, False),
+@pytest.mark.parametrize("precision,d,dense,terms", [("fp32", 9, False, True), ("fp32", 24, False, True), ("fp32", 160, False, True), ("fp32", 161, False, False),
                                                      ("fp32", 40, True, False), ("fp64", 40, False, False)])
 def test_state_gradient(precision, d, dense, terms, exponential):
     kw = dict(d=d, M=2, N=3, S=1, seed=14, nF=1, dt=0.5 / d)
