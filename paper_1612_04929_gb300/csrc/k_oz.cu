@@ -547,6 +547,11 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
             int eB[HC / 32];   // this lane's columns' exponents, broadcast by shuffle
 #pragma unroll
             for (int j = 0; j < HC / 32; ++j) eB[j] = ch0 + 32 * j + lane < d ? eBp[ch0 + 32 * j + lane] : 0;
+            float mB = 0.f;   // the tree's: its column's grid, likewise
+            if constexpr (std::is_same_v<Epi, OzTreeEpi>) {
+                static_assert(HC == 32, "a column a lane");
+                mB = !fe.t.mo ? grid_magic(prm->eu) : (ch0 + lane < d ? fe.t.mo[ch0 + lane] : 0.f);
+            }
             if (!__all_sync(0xffffffffu, mbar_wait(&acc_full, (uint32_t)(n & 1), limit))) {
                 if (lane == 0) atomicOr(&prm->err, kErrTimeout);
                 break;
@@ -627,15 +632,14 @@ k_oz_mm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
             } else if constexpr (std::is_same_v<Epi, OzTreeEpi>) {
                 const TreeMm& tm = fe.t;
                 const int it = fe.item0 + item, te = it / tm.count, ti = it - te * tm.count;
-                const float mu = grid_magic(prm->eu);
                 const size_t o0 = (size_t)row * d + ch0;
 #pragma unroll
                 for (int q = 0; q < HC; ++q) {
                     const int e = __shfl_sync(0xffffffffu, eB[0], q);
+                    const float mo = __shfl_sync(0xffffffffu, mB, q);
                     if (row >= d || q >= ncols) continue;
                     const float sc = ldexpf(1.0f, eA + e - 3 * SBITS);
-                    tree_store(tm, te, ti, o0 + q, ch0 + q, make_float4(res[q].x * sc, res[q].y * sc, res[q].z * sc, res[q].w * sc),
-                               tm.mo ? tm.mo[ch0 + q] : mu);
+                    tree_store(tm, te, ti, o0 + q, ch0 + q, make_float4(res[q].x * sc, res[q].y * sc, res[q].z * sc, res[q].w * sc), mo);
                 }
             } else {
                 const size_t o0 = (size_t)item * fe.ostride + (size_t)row * d + ch0;
