@@ -391,8 +391,8 @@ struct OzTreeEpi {
 // blockIdx.x, + gridDim.x, ..: while the epilogue warps add and write one tile, the products of the next
 // run, and only the read-out of tensor memory stands between the products of two tiles.
 // A forward product at d = 256 (450 items, us): 1375 with a CTA per tile (from 150 items); 1204 persistent; 929 with the
-// MMAs' operands in uniform registers (elect); 742 with A read once per run by the collector, 60 % of the
-// tensor rate at 1.9 GHz.  What is left: the copies alone (4.2 GB of plane tiles through L2 a launch, 2.8 GB of HBM traffic) take 599,
+// MMAs' operands in uniform registers (elect); 742 with A read once per run by the collector, 1.71 PFLOP/s
+// of executed MMAs, 0.90 of the measured cuBLAS burst rate.  What is left: the copies alone (4.2 GB of plane tiles through L2 a launch, 2.8 GB of HBM traffic) take 599,
 // the MMAs 530.  An adjoint product (mean of single and double launches): 750, 622, 608, 583, the copies
 // alone 490.
 // ------------------------------------------------------------------------------------------

@@ -15,8 +15,8 @@
 // and a block's columns keep the norms of Psi_0 or Psi_T, each with a grid of its own), every product a split product (k_big_mm's
 // tiles, qoc_gemm.cuh).  The costate is propagated from Psi_T itself and scaled by the terminal
 // coefficient -2 a_fid O_N w_s / (E W) where G_j is written.
-// Measured on GB300 (evaluation): d = 128, N = 500 11.7 -> 8.3 ms; d = 64,
-// N = 2000 7.05 -> 6.13 ms; d = 256, N = 2000 (BF16_SPLIT) 153 -> 142 ms.
+// Measured on GB300 (evaluation): d = 128, N = 500 11.7 -> 8.1 ms; d = 64,
+// N = 2000 7.05 -> 5.85 ms; d = 256, N = 2000 (BF16_SPLIT) 153 -> 142 ms; where it pays: tree_applies.
 //
 // BF16_SPLIT with 128 <= d <= 384 runs the same products on the tensor cores (k_oz.cu: both operands cut
 // into six seven-bit slices, accurate as the split product; the epilogue writes what k_tree_mm writes):
