@@ -336,24 +336,33 @@ void plan_impl(qoc_ctx* c) {
         }
         seg = best_seg;
     }
-    // norms of the propagated columns of the d x S block at `at` (scaled: their squares may leave the range)
-    auto col_norms = [&](const std::vector<double>& psi, size_t at = 0) {
-        std::vector<double> out;
-        for (int s : c->cols) {
-            double mx = 0.0, n2 = 0.0;
-            auto el = [&](int a, int q) { return psi[at + ((size_t)a * c->S + s) * 2 + q]; };
-            for (int a = 0; a < d; ++a) mx = std::max({mx, std::fabs(el(a, 0)), std::fabs(el(a, 1))});
-            for (int a = 0; a < d && mx > 0.0; ++a)
-                for (int q = 0; q < 2; ++q) n2 += (el(a, q) / mx) * (el(a, q) / mx);
-            out.push_back(mx * std::sqrt(n2));
-        }
-        return out;
+    // largest components and norms of the propagated columns of a d x S block (norms of the scaled columns:
+    // squares may leave the range)
+    auto col_max = [&](const double* psi) {
+        std::vector<double> mx(S, 0.0);
+        for (int a = 0; a < d; ++a)
+            for (int s = 0; s < S; ++s) {
+                const double* z = psi + ((size_t)a * c->S + c->cols[s]) * 2;
+                mx[s] = std::max({mx[s], std::fabs(z[0]), std::fabs(z[1])});
+            }
+        return mx;
+    };
+    auto col_norms = [&](const std::vector<double>& psi) {
+        std::vector<double> mx = col_max(psi.data()), n2(S, 0.0);
+        for (int a = 0; a < d; ++a)
+            for (int s = 0; s < S; ++s)
+                for (int q = 0; q < 2 && mx[s] > 0.0; ++q) {
+                    const double z = psi[((size_t)a * c->S + c->cols[s]) * 2 + q] / mx[s];
+                    n2[s] += z * z;
+                }
+        for (int s = 0; s < S; ++s) mx[s] *= std::sqrt(n2[s]);
+        return mx;
     };
     const std::vector<double> norm0 = col_norms(c->psi0), normT = col_norms(c->psiT);
     c->cost_fit = std::all_of(norm0.begin(), norm0.end(), cost_sums_fit) && std::all_of(normT.begin(), normT.end(), cost_sums_fit);
     if (!c->path.empty())
         for (int j = 0; j < N && c->cost_fit; ++j) {
-            const std::vector<double> n = col_norms(c->path, (size_t)j * d * c->S * 2);
+            const std::vector<double> n = col_max(c->path.data() + (size_t)j * d * c->S * 2);   // within 2^5 of the norms
             c->cost_fit = std::all_of(n.begin(), n.end(), cost_sums_fit);
         }
     const auto range0 = std::minmax_element(norm0.begin(), norm0.end());
