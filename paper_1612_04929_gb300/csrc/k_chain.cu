@@ -505,7 +505,9 @@ k_sources(int d, StateView<R> sv, int j0, int wlen, int N, int E, const C_t<R>* 
     using C = C_t<R>;
     const int jl = WARP ? blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5) : blockIdx.x;
     if (WARP && jl >= wlen) return;
-    const int t0 = WARP ? (threadIdx.x & 31) : threadIdx.x, ts = WARP ? 32 : blockDim.x;
+    // a slice's elements over the CTAs of its column of the grid
+    const int t0 = WARP ? (threadIdx.x & 31) : blockIdx.z * blockDim.x + threadIdx.x;
+    const int ts = WARP ? 32 : blockDim.x * gridDim.z;
     const int e = blockIdx.y, j = j0 + jl, cb = sv.cb, ps = sv.pstride;
     const size_t slice = sv.slice();
     const C* psi = states + ((size_t)e * (wmax + 1) + jl + 1) * slice;
@@ -595,8 +597,14 @@ cudaError_t launch_sources(int d, StateView<R> sv, int j0, int wlen, int N, int 
         k_sources<R, true><<<dim3((wlen + 7) / 8, E), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, ct, cf, c5,
                                                                     Oj, Ofin, src);
     else
-        k_sources<R, false><<<dim3(wlen, E), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, ct, cf, c5, Oj, Ofin,
-                                                           src);
+    {
+        // at least two CTAs an SM for few slices, and no CTA with more than 8192 elements: the last slice's FP64
+        // terms took 250 us on one CTA at d = 256, S = 256
+        const long fill = 304 / ((long)wlen * E), most = (long)(sv.slice() / 2048), cut = (long)((sv.slice() + 8191) / 8192);
+        const int nz = (int)std::max<long>(1, std::max(cut, std::min(fill, most)));
+        k_sources<R, false><<<dim3(wlen, E, nz), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, ct, cf, c5, Oj,
+                                                               Ofin, src);
+    }
     return cudaGetLastError();
 }
 

@@ -77,7 +77,8 @@ inline int gemm_plain_mt(int d, long items, int sms) {
     int best = 4;
     double cost = 1e300;
     for (int mt = items < sms ? 1 : 4; mt <= 6; ++mt) {
-        const double c = gemm_time(d, items, 16 * mt, alone[mt - 1], each[mt - 1], sms);
+        // the smaller tiles only where they are clearly ahead (their CTAs' last rounds cost more than the model says)
+        const double c = gemm_time(d, items, 16 * mt, alone[mt - 1], each[mt - 1], sms) * (mt < 4 ? 1.35 : 1.0);
         if (c < cost) {
             cost = c;
             best = mt;
