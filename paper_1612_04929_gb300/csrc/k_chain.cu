@@ -307,7 +307,8 @@ cudaError_t launch_to_panels(const double2* src, C_t<R>* dst, int d, int S, Stat
 // Two launches of an evaluation, costs / sources (before, with FP64 throughout | with pairs of floats in unrolled
 // loops | now): d = 30, S = 30, N = 400 43 / 54 | 68 / 78 | 31 / 24 us; d = 64, S = 64, N = 2000 (terminal) 401 | 90
 // | 88; d = 81, S = 16, N = 1000 135 / 122 | 85 / 99 | 58 / 35; d = 81, S = 81, N = 100 111 / 125 | 148 / 140 | 48 / 69;
-// d = 256, S = 256, N = 60 938 / 1047 | 332 / 417 | 234 / 501 (the last slice's target terms are FP64);
+// d = 256, S = 256, N = 60 938 / 1047 | 332 / 417 | 239 / 114 (the last slice's target terms are FP64, over several
+// CTAs: 501 on one);
 // FP64 form, d = 60, S = 60, N = 30 57 / 63 | 123 / 149 | 42 / 47.
 // ------------------------------------------------------------------------------------------
 // Running sum of products of FP32 values over three floats: the product and its rounding error are added
@@ -599,7 +600,7 @@ cudaError_t launch_sources(int d, StateView<R> sv, int j0, int wlen, int N, int 
     else
     {
         // at least two CTAs an SM for few slices, and no CTA with more than 8192 elements: the last slice's FP64
-        // terms took 250 us on one CTA at d = 256, S = 256
+        // terms alone took one CTA some 400 us at d = 256, S = 256
         const long fill = 304 / ((long)wlen * E), most = (long)(sv.slice() / 2048), cut = (long)((sv.slice() + 8191) / 8192);
         const int nz = (int)std::max<long>(1, std::max(cut, std::min(fill, most)));
         k_sources<R, false><<<dim3(wlen, E, nz), 256, 0, st>>>(d, sv, j0, wlen, N, E, states, wmax, cv, ct, cf, c5, Oj,
